@@ -95,6 +95,19 @@ template <typename T>
 kf_status trsm_right(cudaStream_t s, bool trans, int M, int n, const T* L, int64_t ldl,
                      const T* dinv, int nb, T* B, int64_t ldb, int* status);
 
+// S = L L^T for the m x m innovation covariance (lower triangle, in place), the inverses of its 32 x 32
+// diagonal blocks (dinv: ceil(m / 32) blocks of 1024), L^{-1} (m x m with zeros above the diagonal, when
+// not null) and nu <- L^{-1} nu (when not null), float64, one launch; bit for bit what potrf and
+// trsm_right give with 32-wide blocks.  m <= kInnovFactorMaxM.  work: innovation_factor_work(m)
+// doubles (16-byte aligned); flags: innovation_factor_flags(m) ints, zero before the first launch (every
+// launch leaves them zero), both used by one stream at a time.  A bad pivot sets KF_ERR_NOT_PD
+// (step, pivot), a non-finite nu KF_ERR_NUMERIC (after the factor).
+constexpr int kInnovFactorMaxM = 960;
+size_t innovation_factor_work(int64_t m);
+size_t innovation_factor_flags(int64_t m);
+kf_status innovation_factor(cudaStream_t s, int m, double* S, int64_t lds, double* dinv, double* Linv, double* nu,
+                            double* work, int* flags, int* status, int step);
+
 // ---------------------------------------------------------------- small ops
 
 // dst[i, j] = (Tdst) src[i, j] for i < rows, j < cols; pad columns cols..ld_dst-1 zeroed

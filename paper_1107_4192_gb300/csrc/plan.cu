@@ -65,6 +65,7 @@ struct kf_plan_s {
   char *P = nullptr, *Ut = nullptr, *Zb = nullptr, *KV = nullptr, *VK = nullptr, *Hb = nullptr, *tmpN = nullptr;
   char *Fb = nullptr, *S0b = nullptr;
   double *S = nullptr, *S0 = nullptr, *Sdinv = nullptr, *partials = nullptr;
+  int* Sflags = nullptr;  // task flags of innovation_factor
   char *Sl = nullptr, *Sldinv = nullptr;
   char *Lb = nullptr, *Ldinv = nullptr, *Jb = nullptr;
   float* Wi = nullptr;    // L^{-1} for the tensor-core solve (mixed mode, float32 solve)
@@ -114,6 +115,13 @@ namespace {
 
 size_t cov_count(int kind, int64_t n) { return kind == 0 ? 1 : kind == 1 ? (size_t)n : (size_t)n * n; }
 
+// Doubles at kf_plan_s::partials: the split-K partials of S (CUDA-core paths), then, once S is summed,
+// the work space of its factorisation.
+size_t partials_count(int64_t m) {
+  const size_t split = (size_t)kSplitsS * m * m;
+  return m <= kInnovFactorMaxM ? std::max(split, innovation_factor_work(m)) : split;
+}
+
 struct Sizes {
   uint64_t workspace = 0, slot = 0;
   int64_t ldN = 0, ldm = 0;
@@ -133,7 +141,7 @@ Sizes sizes_for(const kf_desc* d) {
   w += 2 * N * ldm * z.b;                   // Ut, Z
   w += 2 * N * 2 * ldm * z.b;               // KV, VK
   w += m * ldN * z.b;                       // Hb
-  w += 2 * m * m * 8 + round_up(m, 64) * 64 * 8 + kSplitsS * m * m * 8;  // S, S0, Sdinv, partials
+  w += 2 * m * m * 8 + round_up(m, 64) * 64 * 8 + partials_count(m) * 8;  // S, S0, Sdinv, partials
   w += (m * m + round_up(m, 64) * 64) * z.b + m * m * z.b;               // Sl, Sldinv, S0b
   const int64_t nbs = z.sb == 8 ? 64 : 128;
   w += 2 * N * ldN * z.sb + round_up(N, nbs) * nbs * z.sb;                 // Lb, Jb, Ldinv
@@ -157,7 +165,7 @@ Sizes sizes_for(const kf_desc* d) {
   w += cov_count(d->q_kind, N) * 8 + m * N * 8 + cov_count(d->r_kind, m) * 8;
   // split planes: rows up to max(N, m), k up to max(ldN, 2 ldm) (the Joseph product's rank 2m)
   if (d->prec == KF_PREC_MIXED_BF16X3) w += tc_scratch_bytes(std::max(N, m), std::max(ldN, 2 * ldm));
-  w += 4096;
+  w += 4096;  // status word, flags of innovation_factor (at most 3.8 KB)
   z.workspace = w;
   return z;
 }
@@ -348,15 +356,39 @@ kf_status predict_cov(kf_plan_s* p, const B* src, B* dst) {
 
 // ------------------------------------------------------------ filter step
 
-// Covariance part of one filter step t (and the mean update when y != NULL):
-// uses the working P = P_{t|t-1}, writes P_{t|t} to its store slot and
-// leaves P_{t+1|t} in the working P.
 // Block size of the m x m innovation Cholesky (float64): 32-wide leaves and
 // panels.  Its float64 work is bound by the float64 pipe of the SMs it reaches,
 // so smaller blocks (more parallel panel / trailing products, cheaper leaves)
 // finish sooner than the 64-wide blocks used for large float64 matrices.
 constexpr int kSBlock = 32;
 
+// S = L L^T in place with the inverses of its diagonal blocks (Sdinv), L^{-1} into Linv (when not null)
+// and, when y != NULL, nu <- L^{-1} (y - H x_{t|t-1}), all float64.  One launch up to kInnovFactorMaxM
+// sensors; above that block kernels, whose launches then carry enough work each.
+kf_status factor_innovation(kf_plan_s* p, int64_t t, const double* y, double* Linv) {
+  cudaStream_t s = p->s;
+  const int m = (int)p->m;
+  if (m <= kInnovFactorMaxM) {
+    // a non-finite nu is reported by the factorisation, after a bad pivot of S
+    if (y) KF_TRY(innovation(s, m, p->N, p->H, p->xpred + t * p->N, y, p->nu, nullptr, (int)t));
+    return innovation_factor(s, m, p->S, m, p->Sdinv, Linv, y ? p->nu : nullptr, p->partials, p->Sflags, p->status,
+                             (int)t);
+  }
+  KF_TRY(potrf<double>(s, p->S, m, m, p->Sdinv, kSBlock, p->status, (int)t));
+  if (Linv) {  // I L^{-1}
+    KF_TRY(eye(s, m, Linv, m));
+    KF_TRY(trsm_right<double>(s, false, m, m, p->S, m, p->Sdinv, kSBlock, Linv, m, p->status));
+  }
+  if (y) {  // the 1 x m row solve nu^T L^{-T}
+    KF_TRY(innovation(s, m, p->N, p->H, p->xpred + t * p->N, y, p->nu, p->status, (int)t));
+    KF_TRY(trsm_right<double>(s, true, 1, m, p->S, m, p->Sdinv, kSBlock, p->nu, m, p->status));
+  }
+  return KF_OK;
+}
+
+// Covariance part of one filter step t (and the mean update when y != NULL):
+// uses the working P = P_{t|t-1}, writes P_{t|t} to its store slot and
+// leaves P_{t+1|t} in the working P.
 template <typename B>
 kf_status filter_step(kf_plan_s* p, int64_t t, const double* y, double* diag_out) {
   cudaStream_t s = p->s;
@@ -381,7 +413,7 @@ kf_status filter_step(kf_plan_s* p, int64_t t, const double* y, double* diag_out
   const bool joseph = p->d.joseph_every > 0 && (t % p->d.joseph_every) == 0;
   if (joseph) KF_CUDA_TRY(cudaMemcpyAsync(p->S0, p->S, (size_t)m * m * 8, cudaMemcpyDeviceToDevice, s));
   const int nbS = kSBlock;
-  KF_TRY(potrf<double>(s, p->S, m, m, p->Sdinv, nbS, p->status, (int)t));
+  KF_TRY(factor_innovation(p, t, y, nullptr));
   const B* L = (const B*)p->S;
   const B* Ld = (const B*)p->Sdinv;
   if (sizeof(B) != sizeof(double)) {
@@ -397,12 +429,7 @@ kf_status filter_step(kf_plan_s* p, int64_t t, const double* y, double* diag_out
   B* Z = (B*)p->Zb;
   KF_TRY((copy2d<B, B>(s, Z, ldm, Ut, ldm, N, m)));
   KF_TRY(trsm_right<B>(s, true, N, m, L, m, Ld, nbS, Z, ldm, p->status));
-  if (y) {
-    KF_TRY(innovation(s, m, N, p->H, p->xpred + t * N, y, p->nu, p->status, (int)t));
-    // nu <- L^{-1} nu  (as the 1 x m row solve nu^T L^{-T}), float64
-    KF_TRY(trsm_right<double>(s, true, 1, m, p->S, m, p->Sdinv, nbS, p->nu, m, p->status));
-    KF_TRY(gemv<B>(s, N, m, Z, ldm, p->nu, p->xpred + t * N, 1.0, p->xfilt + t * N));
-  }
+  if (y) KF_TRY(gemv<B>(s, N, m, Z, ldm, p->nu, p->xpred + t * N, 1.0, p->xfilt + t * N));
   const bool ident = p->d.f_kind == KF_F_IDENTITY;
   B* dst = (B*)p->slot_ptr(t);
   GemmParams<B> u;  // P_{t|t} = P - Z Z^T  (symmetric by construction), P <- P_{t|t} + Q when F = I
@@ -515,11 +542,7 @@ kf_status filter_step_mixed(kf_plan_s* p, int64_t t, const double* y, double* di
   }
   const bool joseph = p->d.joseph_every > 0 && (t % p->d.joseph_every) == 0;
   if (joseph) KF_CUDA_TRY(cudaMemcpyAsync(p->S0, p->S, (size_t)m * m * 8, cudaMemcpyDeviceToDevice, s));
-  const int nbS = kSBlock;
-  KF_TRY(potrf<double>(s, p->S, m, m, p->Sdinv, nbS, p->status, (int)t));
-  // L^{-1} = I L^{-1} (m x m, float64)
-  KF_TRY(eye(s, m, p->Linv, m));
-  KF_TRY(trsm_right<double>(s, false, m, m, p->S, m, p->Sdinv, nbS, p->Linv, m, p->status));
+  KF_TRY(factor_innovation(p, t, y, p->Linv));
   double* Z = p->Z64;
   {
     KF_TRY(oz_slice(s, Ut, ldm, 1, N, m, LV, p->sUt));
@@ -529,11 +552,7 @@ kf_status filter_step_mixed(kf_plan_s* p, int64_t t, const double* y, double* di
     e.status = p->status; e.step = (int)t;
     KF_TRY(oz_gemm(s, p->sUt, p->sL, N, m, m, LV, e));
   }
-  if (y) {
-    KF_TRY(innovation(s, m, N, p->H, p->xpred + t * N, y, p->nu, p->status, (int)t));
-    KF_TRY(trsm_right<double>(s, true, 1, m, p->S, m, p->Sdinv, nbS, p->nu, m, p->status));
-    KF_TRY(gemv<double>(s, N, m, Z, ldm, p->nu, p->xpred + t * N, 1.0, p->xfilt + t * N));
-  }
+  if (y) KF_TRY(gemv<double>(s, N, m, Z, ldm, p->nu, p->xpred + t * N, 1.0, p->xfilt + t * N));
   const bool ident = p->d.f_kind == KF_F_IDENTITY;
   OzEpilogue u;  // P_{t|t} = P - Z Z^T: float64 result, float32 copy to the store
   u.alpha = -1.0;
@@ -648,11 +667,9 @@ kf_status filter_first_fp64(kf_plan_s* p, const double* P0, const double* y, dou
   KF_TRY((innovation_cov<double, double>(s, m, N, p->H, N, p->U64, ldm, p->d.r_kind, p->R, p->S, m, p->partials,
                                         kSplitsS)));
   const int nbS = kSBlock;
-  KF_TRY(potrf<double>(s, p->S, m, m, p->Sdinv, nbS, p->status, 1));
+  KF_TRY(factor_innovation(p, 1, y, nullptr));
   KF_TRY((copy2d<double, double>(s, p->Z64, ldm, p->U64, ldm, N, m)));
   KF_TRY(trsm_right<double>(s, true, N, m, p->S, m, p->Sdinv, nbS, p->Z64, ldm, p->status));
-  KF_TRY(innovation(s, m, N, p->H, p->xpred + N, y, p->nu, p->status, 1));
-  KF_TRY(trsm_right<double>(s, true, 1, m, p->S, m, p->Sdinv, nbS, p->nu, m, p->status));
   KF_TRY(gemv<double>(s, N, m, p->Z64, ldm, p->nu, p->xpred + N, 1.0, p->xfilt + N));
   GemmParams<double> u;  // P_{1|1} = P_{1|0} - Z Z^T
   u.M = N; u.N = N; u.K = m;
@@ -1094,7 +1111,8 @@ kf_status kf_plan(kf_plan_t* out, const kf_desc* d) {
   A(&p->S, m * m * 8);
   A(&p->S0, m * m * 8);
   A(&p->Sdinv, round_up(m, 64) * 64 * 8);
-  A(&p->partials, kSplitsS * m * m * 8);
+  A(&p->partials, partials_count(m) * 8);
+  if (m <= kInnovFactorMaxM) A(&p->Sflags, innovation_factor_flags(m) * sizeof(int));
   A(&p->Sl, m * m * b);
   A(&p->Sldinv, round_up(m, 64) * 64 * b);
   A(&p->S0b, m * m * b);

@@ -1,0 +1,61 @@
+"""The one-launch factorisation of the innovation covariance (eqn 8) at the edges of its tiles, through
+the C ABI against the float64 oracle, and its failure reports.
+
+Sizes: one row, a tile less / more one, several tiles with ragged ends, and both sides of the largest m it
+takes (above it block kernels do the same).  Tolerance: the float64 path's 1e-10 on means and diag P.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_1107_4192_gb300 import binding as B  # noqa: E402
+from paper_1107_4192_gb300 import solver, synth  # noqa: E402
+from tests.helpers import diag_of, rel_err_elementwise, rel_err_per_step, run_oracle  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1107_4192_gb300 import build
+    build.build()
+    B.lib()
+
+
+@pytest.mark.parametrize("N,m", [(40, 1), (40, 31), (40, 32), (40, 33), (60, 64), (60, 65), (130, 97), (90, 306),
+                                 (64, 960), (64, 961)])
+def test_filter_at_tile_edges(N, m):
+    prob = synth.random_walk_problem(N, m, 3, seed=N + m)
+    out, ref = solver.run(prob, prec=B.KF_PREC_FP64), run_oracle(prob)
+    assert rel_err_per_step(out["x_filt"], ref["x_filt"]) <= 1e-10
+    assert rel_err_elementwise(out["diagP_filt"], diag_of(ref["P_filt"])) <= 1e-10
+
+
+def _filter(plan, d, T, N):
+    x = torch.empty(T, N, dtype=torch.float64, device="cuda")
+    return B.kf_filter(plan.handle, d.F, d.F_rowptr, d.F_col, d.Q, d.H, d.R, d.Y, d.x0, d.P0, x, raise_on_error=False) + (x,)
+
+
+@pytest.mark.parametrize("prec,solve", [(B.KF_PREC_FP64, B.KF_SOLVE_FP64), (B.KF_PREC_MIXED_BF16X3, B.KF_SOLVE_FP32)])
+def test_failure_in_a_later_tile_then_recovery(prec, solve):
+    """A singular S whose bad pivot lies in the third tile, then a non-finite sample, then good data on
+    the same plan: the reports are those of the block algorithm, and nothing is left behind."""
+    N, m, T = 150, 100, 3
+    prob = synth.random_walk_problem(N, m, T, seed=9)
+    good = solver.upload(prob)
+    with solver.Plan.for_inputs(good, N, m, T, prec=prec, solve_prec=solve) as plan:
+        st, step, x0 = _filter(plan, good, T, N)
+        assert st == B.KF_OK
+        bad = solver.upload(prob)
+        bad.H[80:] = 0.0
+        bad.R = torch.zeros_like(bad.R)
+        st, step, _ = _filter(plan, bad, T, N)
+        assert st == B.KF_ERR_NOT_PD and step == 1
+        nan = solver.upload(prob)
+        nan.Y[1, 70] = float("nan")
+        st, step, _ = _filter(plan, nan, T, N)
+        assert st == B.KF_ERR_NUMERIC and step == 2
+        st, step, x1 = _filter(plan, good, T, N)
+        assert st == B.KF_OK and torch.equal(x0, x1)
