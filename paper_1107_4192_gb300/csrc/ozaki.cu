@@ -6,7 +6,7 @@
 // digits (|q_p| <= 128) as bf16 planes, in integer arithmetic on the bits of
 // x (the float64 units of this GPU would make float64 slicing the slow part).
 //
-// Product (oz_gemm_kernel): one 128 x 64 output tile per CTA, 18 warps.
+// Product (oz_gemm_kernel): one 128 x 64 output tile per CTA, 19 warps.
 //   warp 0  one lane issues the TMA loads (64-byte swizzle) of all slices of a
 //           32-wide k-slice (two MMA k-steps) of A and B into a shared-memory
 //           stage;
@@ -19,12 +19,15 @@
 //           128-wide chunk it commits the level's buffer to its "ready"
 //           barrier, and a level's next chunk starts (overwriting) in a buffer
 //           the epilogue has drained;
-//   warps 2-17 per chunk and level, read the accumulator (an exact integer
+//   warp 2  the gate: waits for each k-step's operands and drained buffer and releases it to warp 1;
+//   warps 3-18 per chunk and level, read the accumulator (an exact integer
 //           below 2^24), convert it to an integer and add it into 64-bit
 //           fixed-point accumulators in registers (levels 0-2 and levels 3..
 //           in two of them); at the end scale by the row and column exponents
 //           and apply the float64 epilogue.
 // Every pipeline wait is bounded (kernel argument, as in the split-bf16 kernel).
+#include <type_traits>
+
 #include "ozaki.cuh"
 #include "tc_ptx.cuh"
 
@@ -36,17 +39,20 @@ constexpr int OZ_BM = 128;      // output rows per CTA (TMEM lanes)
 constexpr int OZ_BN = 64;       // output columns per CTA (TMEM columns per level)
 constexpr int OZ_KC = 128;      // values of k per exact chunk
 constexpr int OZ_EPI_WARPS = 16;  // 4 TMEM lane quadrants x 4 column quarters of 16
-constexpr int OZ_GATE_WARP = 2 + OZ_EPI_WARPS;  // waits for each k-step's operands and buffer
-constexpr int OZ_THREADS = 32 * (3 + OZ_EPI_WARPS);
+constexpr int OZ_GATE_WARP = 2;   // waits for each k-step's operands and buffer
+constexpr int OZ_EPI0 = 3;        // first epilogue warp
+constexpr int OZ_THREADS = 32 * (OZ_EPI0 + OZ_EPI_WARPS);
 constexpr int OZ_GROUP = 8;     // row tiles per rasterisation group (operand reuse in L2)
 constexpr int OZ_ROW_PAD = 128;
 constexpr int kOzBK = 32;       // k per pipeline stage of the launched kernels (two MMA k-steps)
 constexpr int kOzBadRow = 0x7fffffff;  // exponent marking a row that holds an infinity or NaN
 
-// LV slice levels; BK values of k per pipeline stage, one swizzled row of bf16 (16: 32-byte
-// swizzle, one MMA k-step; 32: 64-byte swizzle, two k-steps, half the stages and wider TMA rows).
-template <int LV, int BK>
+// LV slice levels, LA <= LV slices of A and LV of B; BK values of k per pipeline stage, one swizzled row
+// of bf16 (16: 32-byte swizzle, one MMA k-step; 32: 64-byte swizzle, two k-steps, half the stages and wider
+// TMA rows).
+template <int LV, int LA, int BK>
 struct OzCfg {
+  static_assert(LA >= 1 && LA <= LV, "slices of A");
   static_assert(BK == 16 || BK == 32, "one 32- or 64-byte swizzled row of bf16 per stage");
   static constexpr int SWZ = BK * 2;                         // swizzle width in bytes
   static constexpr uint32_t LAYOUT = BK == 16 ? kLayoutSw32 : kLayoutSw64;  // descriptor swizzle mode
@@ -56,7 +62,7 @@ struct OzCfg {
   static constexpr int CKS = OZ_KC / 16;                     // k-steps per exact chunk
   static constexpr int A_BYTES = OZ_BM * BK * 2;
   static constexpr int B_BYTES = OZ_BN * BK * 2;
-  static constexpr int STAGE_BYTES = LV * (A_BYTES + B_BYTES);
+  static constexpr int STAGE_BYTES = LA * A_BYTES + LV * B_BYTES;
   static constexpr int FIT = (210 * 1024) / STAGE_BYTES;
   static constexpr int STAGES = FIT > 8 ? 8 : FIT;
   static_assert(STAGES >= 2, "double-buffered pipeline");
@@ -84,6 +90,108 @@ __device__ __forceinline__ double oz_qv(int kind, const double* q, int64_t ldq, 
   if (kind == 1) return i == j ? q[i] : 0.0;
   if (kind == 2) return q[(int64_t)i * ldq + j];
   return 0.0;
+}
+
+// The epilogue keeps off the float64 unit, which runs one warp instruction per 19 cycles and SM: a tile of
+// 128 x 64 elements with the six or so float64 operations per element of the plain formulas (two
+// scalings, their sum, alpha, beta, a zero from Q, the float32 conversion) cost 16 us, as much as the
+// products of a short K.  Scaling and conversions are integer operations on the bits with the same
+// rounding (to nearest, ties to even); what is left is at most one float64 addition per element, and
+// a tile's sweep takes 3 us (M x N x K = 1664 x 128 x 128: the launch 28 us before, 15 us now).
+
+__device__ __noinline__ double scaled_general(unsigned long long m, int e) { return scalbn((double)m, e); }
+
+// (H 2^32 + L) 2^e rounded to float64, for a magnitude whose leading bit is bit 62 (so that rounding up
+// cannot overflow; any bits lost before are or-ed into bit 0); sign is the result's sign bit.
+__device__ __forceinline__ double round53(uint32_t H, uint32_t L, int e, uint32_t sign) {
+  const uint32_t add = 0x1ffu + ((L >> 10) & 1u);  // ties to even
+  const uint32_t l = L + add;
+  const uint32_t h = H + (l < add ? 1u : 0u);
+  const uint32_t mh = h >> 10, ml = __funnelshift_r(l, h, 10);
+  const int E = 1023 + 62 + e;  // biased exponent of the leading bit
+  if ((unsigned)(E - 1) > 2043u) {
+    const double v = scaled_general(((unsigned long long)mh << 32) | ml, e + 10);
+    return __hiloint2double(__double2hiint(v) | (int)sign, __double2loint(v));
+  }
+  return __hiloint2double((int)((mh + ((uint32_t)(E - 1) << 20)) | sign), (int)ml);  // mh holds the leading bit
+}
+
+// t 2^e rounded to float64, |t| < 2^63.
+__device__ __forceinline__ double fixed_to_double(long long t, int e) {
+  const uint32_t sgn = (uint32_t)(t >> 63);
+  const unsigned long long u = ((unsigned long long)t ^ (((unsigned long long)sgn << 32) | sgn)) + (sgn & 1u);
+  uint32_t hi = (uint32_t)(u >> 32), lo = (uint32_t)u;
+  if (hi == 0) {
+    if (lo == 0) return 0.0;
+    hi = lo >> 1;  // keeps the leading bit below bit 63
+    lo = lo << 31;
+    e -= 31;
+    if (hi == 0) {  // u == 1
+      hi = 1u << 30;
+      lo = 0;
+      e -= 31;
+    }
+  }
+  const int sh = __clz((int)hi) - 1;
+  return round53(__funnelshift_l(lo, hi, sh), lo << sh, e - sh, sgn & 0x80000000u);
+}
+
+// (hi 2^s + lo) 2^e rounded to float64, for s <= 32, |hi| < 2^61, |lo| < 2^(30 + s) (K <= 2^20 keeps within).
+__device__ __forceinline__ double fixed_to_double(long long hi, long long lo, int s, int e) {
+  // in units 2^(s - 32): hi 2^32 + lo 2^(32 - s), as a 96-bit integer (w2, w1, w0)
+  const long long l = (long long)((unsigned long long)lo << (32 - s));
+  const long long top = hi + (l >> 32);
+  const uint32_t sgn = (uint32_t)(top >> 63);
+  uint32_t w0 = (uint32_t)l ^ sgn;
+  unsigned long long w = (unsigned long long)top ^ (((unsigned long long)sgn << 32) | sgn);
+  if (sgn && ++w0 == 0) ++w;
+  e -= 32 - s;
+  const uint32_t w2 = (uint32_t)(w >> 32), w1 = (uint32_t)w;
+  if (w2 == 0) {  // below 2^64
+    if (w1 == 0) {
+      const double v = fixed_to_double((long long)w0, e);
+      return __hiloint2double(__double2hiint(v) | (int)(w0 ? sgn & 0x80000000u : 0u), __double2loint(v));
+    }
+    const int n = __clz((int)w1);
+    if (n == 0) return round53(w1 >> 1, (w1 << 31) | (w0 >> 1) | (w0 & 1u), e + 1, sgn & 0x80000000u);
+    return round53(__funnelshift_l(w0, w1, n - 1), w0 << (n - 1), e - (n - 1), sgn & 0x80000000u);
+  }
+  const int sh = __clz((int)w2) - 1;  // |top| < 2^62
+  const uint32_t lost = w0 << sh;
+  return round53(__funnelshift_l(w1, w2, sh), __funnelshift_l(w0, w1, sh) | (lost ? 1u : 0u), e + 32 - sh,
+                 sgn & 0x80000000u);
+}
+
+// float64 to float32, to nearest, ties to even.
+__device__ __noinline__ float narrow_general(double v) { return (float)v; }
+__device__ __forceinline__ float narrow(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const unsigned E = (unsigned)(b >> 52) & 0x7ffu;
+  if (E - 897u > 1149u - 897u) return narrow_general(v);  // outside float32's normal range (zero, infinity, NaN too)
+  const unsigned long long mag = (b & 0x7fffffffffffffffull) - (896ull << 52);
+  unsigned f = (unsigned)(mag >> 29);
+  const unsigned rem = (unsigned)mag & 0x1fffffffu;
+  f += (rem > 0x10000000u || (rem == 0x10000000u && (f & 1))) ? 1u : 0u;
+  return __uint_as_float(f | ((unsigned)(b >> 32) & 0x80000000u));
+}
+
+// alpha c + beta cin.  alpha_unit and beta_unit are set on the host (a float64 comparison costs as much as
+// an addition), and the general form is a call: inlined, its float64 instructions would be predicated, and
+// predicated-off ones still take their turn.
+__device__ __noinline__ double oz_axpby_general(double alpha, double c, double beta, double cin) {
+  return fma(beta, cin, alpha * c);
+}
+template <bool CIN>
+__device__ __forceinline__ double oz_axpby(const OzEpilogue& e, double c, double cin) {
+  if (e.alpha_unit == 0 || (CIN && !e.beta_unit)) return oz_axpby_general(e.alpha, c, CIN ? e.beta : 0.0, CIN ? cin : 0.0);
+  const double ac = __longlong_as_double(__double_as_longlong(c) ^ (e.alpha_unit < 0 ? 1ll << 63 : 0ll));
+  if constexpr (CIN) return cin + ac;
+  return ac;
+}
+
+// v + Q[i][j]
+__device__ __forceinline__ double oz_addq(double v, int kind, const double* q, int64_t ldq, int i, int j) {
+  return (kind == 2 || (kind >= 0 && i == j)) ? v + oz_qv(kind, q, ldq, i, j) : v;
 }
 
 __device__ __forceinline__ void oz_apply(const OzEpilogue& e, int gi, int gj, double c) {
@@ -115,6 +223,8 @@ struct OzArgs {
   int M, N, nk;                  // nk = k-slices of BK (all of K)
   int kt_per_split;              // k-slices per split (blockIdx.y)
   double* partials;              // splits > 1: raw sums, split s at partials + s M N (ld N)
+  long long* sums;               // exact splits: integer sums, split s at sums + s M ld_sums
+  int64_t ld_sums;
   int a_rows_pad, b_rows_pad;    // plane p starts at row p * rows_pad of its map
   const int* ea;
   const int* eb;
@@ -242,9 +352,10 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(const T* X, int64_t ld, i
 
 // One level's drain by an epilogue warp: read its 16 accumulator columns (exact integers below
 // 2^24), hand the buffer back to the MMA issuer, and add the values into the 64-bit fixed-point
-// sums (levels 0-2 in units of level 2, levels 3.. in units of level LV-1).
-template <int L, int LV>
-__device__ __forceinline__ void oz_drain(uint32_t taddr, uint32_t dbar, int lane, long long (&hi)[16],
+// sums: all levels in units of level LV-1 (lo), or where that needs more than 64 bits (WIDE) levels 0-2
+// in units of level 2 (hi) and the others in lo.
+template <int L, int LV, bool WIDE>
+__device__ __forceinline__ void oz_drain(uint32_t taddr, uint32_t dbar, int lane, long long (&hi)[WIDE ? 16 : 1],
                                          long long (&lo)[16]) {
   if constexpr (L < LV) {
     uint32_t r[16];
@@ -255,7 +366,7 @@ __device__ __forceinline__ void oz_drain(uint32_t taddr, uint32_t dbar, int lane
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
       const long long v = (long long)__float2int_rn(__uint_as_float(r[j]));
-      if constexpr (L < 3)
+      if constexpr (WIDE && L < 3)
         hi[j] += v << (8 * (2 - L));
       else
         lo[j] += v << (8 * (LV - 1 - L));
@@ -274,14 +385,14 @@ __device__ __forceinline__ void oz_drain(uint32_t taddr, uint32_t dbar, int lane
 // overwrites the accumulator instead of adding to it (at the first k-step every level starts, and
 // all of pa = 0's MMAs overwrite).  `pre` runs after the MMAs of the first A slices, about half
 // of the k-step's work.
-template <int LV, int BK, int R, typename Pre>
+template <int LV, int LA, int BK, int R, typename Pre>
 __device__ __forceinline__ void oz_issue_kstep(bool leader, uint32_t tmem, uint64_t adesc0, uint64_t bdesc0, int cm,
                                                bool first_step, Pre&& pre) {
-  using C = OzCfg<LV, BK>;
+  using C = OzCfg<LV, LA, BK>;
   constexpr int LS = R == 0 ? 0 : C::CKS - R;
-  constexpr int PRE_AFTER = LV >= 5 ? 2 : 1;
+  constexpr int PRE_AFTER = LA >= 5 ? 2 : 1;
 #pragma unroll
-  for (int pa = 0; pa < LV; ++pa) {
+  for (int pa = 0; pa < LA; ++pa) {
     if (pa == PRE_AFTER) pre();
     int l0 = pa;
 #pragma unroll
@@ -330,9 +441,9 @@ __device__ __forceinline__ bool oz_gate_wait(uint32_t addr, uint32_t t, volatile
   }
 }
 
-template <int LV, int BK>
+template <int LV, int LA, bool WIDE, int BK>
 __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(const __grid_constant__ OzMaps maps, const OzArgs a) {
-  using C = OzCfg<LV, BK>;
+  using C = OzCfg<LV, LA, BK>;
   extern __shared__ uint8_t smem_raw[];
   // grouped rasterisation: OZ_GROUP row tiles sweep the column tiles together
   const int tiles_m = (a.M + OZ_BM - 1) / OZ_BM, tiles_n = (a.N + OZ_BN - 1) / OZ_BN;
@@ -407,10 +518,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(const __grid_con
       mbar_expect_tx(full_bar(s), C::STAGE_BYTES);
       const int x = (kt0 + it) * BK;
 #pragma unroll
-      for (int p = 0; p < LV; ++p) tma_load_2d(st + p * C::A_BYTES, &maps.a, x, p * a.a_rows_pad + m0, full_bar(s));
+      for (int p = 0; p < LA; ++p) tma_load_2d(st + p * C::A_BYTES, &maps.a, x, p * a.a_rows_pad + m0, full_bar(s));
 #pragma unroll
       for (int p = 0; p < LV; ++p)
-        tma_load_2d(st + LV * C::A_BYTES + p * C::B_BYTES, &maps.b, x, p * a.b_rows_pad + n0, full_bar(s));
+        tma_load_2d(st + LA * C::A_BYTES + p * C::B_BYTES, &maps.b, x, p * a.b_rows_pad + n0, full_bar(s));
       last_round[s] = it / C::STAGES;
     }
     if (*abort_flag) {  // let issued copies land before the CTA's shared memory goes away
@@ -431,7 +542,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(const __grid_con
       const int s = it % C::STAGES;
       const uint32_t st = base + s * C::STAGE_BYTES;
       const uint64_t adesc_s = smem_desc_sw(st, C::SBO, C::LAYOUT);
-      const uint64_t bdesc_s = smem_desc_sw(st + LV * C::A_BYTES, C::SBO, C::LAYOUT);
+      const uint64_t bdesc_s = smem_desc_sw(st + LA * C::A_BYTES, C::SBO, C::LAYOUT);
 #pragma unroll
       for (int j = 0; j < C::KS; ++j) {
         const int t = it * C::KS + j;  // k-step
@@ -457,14 +568,14 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(const __grid_con
         // k-step j reads the next 32 bytes of every swizzled row (start address in 16-byte units)
         const uint64_t adesc0 = adesc_s + (uint64_t)(2 * j), bdesc0 = bdesc_s + (uint64_t)(2 * j);
         switch (r) {
-          case 0: oz_issue_kstep<LV, BK, 0>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
-          case 1: oz_issue_kstep<LV, BK, 1>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
-          case 2: oz_issue_kstep<LV, BK, 2>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
-          case 3: oz_issue_kstep<LV, BK, 3>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
-          case 4: oz_issue_kstep<LV, BK, 4>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
-          case 5: oz_issue_kstep<LV, BK, 5>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
-          case 6: oz_issue_kstep<LV, BK, 6>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
-          default: oz_issue_kstep<LV, BK, 7>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
+          case 0: oz_issue_kstep<LV, LA, BK, 0>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
+          case 1: oz_issue_kstep<LV, LA, BK, 1>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
+          case 2: oz_issue_kstep<LV, LA, BK, 2>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
+          case 3: oz_issue_kstep<LV, LA, BK, 3>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
+          case 4: oz_issue_kstep<LV, LA, BK, 4>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
+          case 5: oz_issue_kstep<LV, LA, BK, 5>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
+          case 6: oz_issue_kstep<LV, LA, BK, 6>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
+          default: oz_issue_kstep<LV, LA, BK, 7>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
         }
         __syncwarp();
         mma_issued = true;
@@ -527,13 +638,15 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(const __grid_con
       __syncwarp();
       if (lane == 0) oz_gate_store(gate_addr, (uint32_t)(t + 1));
     }
-  } else if (warp >= 2) {
+  } else if (warp >= OZ_EPI0) {
     // ---------------- epilogue: exact level sums into 64-bit fixed point, then scale and store
-    const int q = warp % 4, h = (warp - 2) / 4;  // TMEM lane quadrant (fixed by the warp index), column quarter
+    const int q = warp % 4, h = (warp - OZ_EPI0) / 4;  // TMEM lane quadrant (fixed by the warp index), column quarter
     const int gi = m0 + 32 * q + lane;
-    long long hi[16], lo[16];  // levels 0-2 in units of level 2; levels 3.. in units of level LV-1
+    long long hi[WIDE ? 16 : 1], lo[16];  // the element's fixed-point sums (oz_drain)
 #pragma unroll
-    for (int j = 0; j < 16; ++j) hi[j] = lo[j] = 0;
+    for (int j = 0; j < 16; ++j) lo[j] = 0;
+#pragma unroll
+    for (int j = 0; j < (WIDE ? 16 : 1); ++j) hi[j] = 0;
     bool ok = true;
     // drain events in the MMA issuer's order: at k-step t, the level whose staggered chunk ends
     // there; at the last k-step, every level
@@ -559,85 +672,219 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(const __grid_con
         const uint32_t dbar = drained_bar(b);
         // compile-time level, so the shifts are constants and the conversions 32-bit
         switch (l) {
-          case 0: oz_drain<0, LV>(taddr, dbar, lane, hi, lo); break;
-          case 1: oz_drain<1, LV>(taddr, dbar, lane, hi, lo); break;
-          case 2: oz_drain<2, LV>(taddr, dbar, lane, hi, lo); break;
-          case 3: oz_drain<3, LV>(taddr, dbar, lane, hi, lo); break;
-          case 4: oz_drain<4, LV>(taddr, dbar, lane, hi, lo); break;
-          case 5: oz_drain<5, LV>(taddr, dbar, lane, hi, lo); break;
-          case 6: oz_drain<6, LV>(taddr, dbar, lane, hi, lo); break;
+          case 0: oz_drain<0, LV, WIDE>(taddr, dbar, lane, hi, lo); break;
+          case 1: oz_drain<1, LV, WIDE>(taddr, dbar, lane, hi, lo); break;
+          case 2: oz_drain<2, LV, WIDE>(taddr, dbar, lane, hi, lo); break;
+          case 3: oz_drain<3, LV, WIDE>(taddr, dbar, lane, hi, lo); break;
+          case 4: oz_drain<4, LV, WIDE>(taddr, dbar, lane, hi, lo); break;
+          case 5: oz_drain<5, LV, WIDE>(taddr, dbar, lane, hi, lo); break;
+          case 6: oz_drain<6, LV, WIDE>(taddr, dbar, lane, hi, lo); break;
           default: break;
         }
       }
     }
-    // Stage the tile's product values in shared memory (the operand stages are idle once the last
-    // chunk has been drained), then sweep it by rows for the direct outputs (lane -> column, so every
-    // warp access is contiguous) and by columns for the mirrored and transposed outputs.
+    // Stage the tile's integer sums in shared memory (the operand stages are idle once the last chunk has
+    // been drained), then sweep it by rows for the direct outputs (lane -> column, so every warp access is
+    // contiguous) and by columns for the mirrored and transposed outputs.  The scaling to float64 is done in
+    // the row sweep's loop: a CTA runs this once, so unrolled code would mostly wait for its instructions
+    // (per-thread unrolled scaling and batched rows took 30 k cycles per tile, this loop about a third).
+    // A slot of the first plane holds the sum, and after the row sweep the value.
     constexpr int PITCH = OZ_BN + 1;  // odd pitch: row and column sweeps are both conflict-free
-    static_assert((size_t)OZ_BM * PITCH * sizeof(double) <= (size_t)C::STAGES * C::STAGE_BYTES, "tile fits");
-    double* tile = reinterpret_cast<double*>(gbase);
-    if (ok) {
-      const int ei = gi < a.M ? a.ea[gi] : 0;
+    constexpr int SH = 8 * (LV - 3);  // unit of hi over the unit of lo
+    static_assert((size_t)OZ_BM * PITCH * (WIDE ? 2 : 1) * sizeof(double) <= (size_t)C::STAGES * C::STAGE_BYTES, "tile fits");
+    long long* tile1 = reinterpret_cast<long long*>(gbase);
+    constexpr int PLANE = OZ_BM * PITCH;  // wide sums: lo in the first plane, hi in the second
+    if (a.sums) {
+      if (ok && gi < a.M) {  // columns padded to 64
+        longlong2* dst = reinterpret_cast<longlong2*>(a.sums + ((int64_t)blockIdx.y * a.M + gi) * a.ld_sums + n0 + h * 16);
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const int gj = n0 + h * 16 + j;
-        const int ej = gj < a.N ? a.eb[gj] : 0;
-        const int sc = ei + ej - 14;
-        tile[(32 * q + lane) * PITCH + h * 16 + j] =
-            (ei == kOzBadRow || ej == kOzBadRow)
-                ? __longlong_as_double(0x7ff8000000000000ll)  // a non-finite operand row
-                : scalbn((double)hi[j], sc - 16) + scalbn((double)lo[j], sc - 8 * (LV - 1));
+        for (int j = 0; j < 16; j += 2)
+          dst[j / 2] = make_longlong2(lo[j], lo[j + 1]);
+      }
+    } else if (ok) {
+      const int slot = (32 * q + lane) * PITCH + h * 16;
+#pragma unroll
+      for (int j = 0; j < 16; ++j) tile1[slot + j] = lo[j];
+      if constexpr (WIDE) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) tile1[PLANE + slot + j] = hi[j];
       }
     }
     asm volatile("bar.sync 1, %0;" ::"n"(32 * OZ_EPI_WARPS) : "memory");
-    const bool go = !*abort_flag;
-    const int ew = warp - 2;  // epilogue warp 0..15
+    const bool go = !*abort_flag && !a.sums;
+    const int ew = warp - OZ_EPI0;  // epilogue warp 0..15
     const OzEpilogue& e = a.e;
     double* part = a.partials ? a.partials + (int64_t)blockIdx.y * a.M * a.N : nullptr;
-    if (go) {
-      for (int r = ew; r < OZ_BM; r += OZ_EPI_WARPS) {
-        const int gi2 = m0 + r;
-        if (gi2 >= a.M) break;
+    auto value_slot = [&](int r, int c) { return reinterpret_cast<double*>(tile1) + r * PITCH + c; };
+    // One row per warp and turn, two columns per lane.  A sweep is bound by its instructions, and one loop
+    // for every kind of output takes twice the time of a loop for the kind at hand, so the usual kinds have
+    // their own loop for the tiles that hold no diagonal element; the others take the general one.
+    const bool crosses = n0 < m0 + OZ_BM && n0 + OZ_BN > m0;
+    const bool fast = e.simple == 2 || (e.simple == 1 && !crosses);
+    constexpr int NR = OZ_BM / OZ_EPI_WARPS;  // rows per warp
+    constexpr int SC = -14 - 8 * (LV - 1);
+    const int gj0 = n0 + lane, gj1 = gj0 + 32;
+    const bool in0 = gj0 < a.N, in1 = gj1 < a.N;
+    const int ej0 = go && in0 ? a.eb[gj0] : 0, ej1 = go && in1 ? a.eb[gj1] : 0;
+    const int my_row = m0 + ew + OZ_EPI_WARPS * lane;
+    const int ei_all = go && lane < NR && my_row < a.M ? a.ea[my_row] : 0;
+    const bool any_bad = __any_sync(0xffffffffu, ej0 == kOzBadRow || ej1 == kOzBadRow || ei_all == kOzBadRow);
+    const bool columns = !part && (e.sym || e.outT);  // the column sweep wants the values
+    auto product = [&](int r, int ei, double& v0, double& v1) {
+      if constexpr (WIDE) {
+        const long long* t = tile1 + r * PITCH + lane;
+        v0 = fixed_to_double(t[PLANE], t[0], SH, ei + SC + ej0);
+        v1 = fixed_to_double(t[PLANE + 32], t[32], SH, ei + SC + ej1);
+      } else {
+        v0 = fixed_to_double(tile1[r * PITCH + lane], ei + SC + ej0);
+        v1 = fixed_to_double(tile1[r * PITCH + lane + 32], ei + SC + ej1);
+      }
+      if (any_bad) {  // a non-finite operand row
+        const double nan = __longlong_as_double(0x7ff8000000000000ll);
+        if (ei == kOzBadRow || ej0 == kOzBadRow) v0 = nan;
+        if (ei == kOzBadRow || ej1 == kOzBadRow) v1 = nan;
+      }
+    };
+    auto fast_sweep = [&](auto with_cin, auto with_f32) {
+      constexpr bool CIN = decltype(with_cin)::value, F32 = decltype(with_f32)::value;
+      const int64_t first = m0 + ew;
+      // every row's cin before the first store (cin may be the output array)
+      double cb[CIN ? NR : 1][2];
+      if constexpr (CIN) {
+        const double* pc = e.cin + first * e.ldcin + gj0;
+        const int64_t step = OZ_EPI_WARPS * e.ldcin;
 #pragma unroll
-        for (int cc = 0; cc < OZ_BN; cc += 32) {
-          const int c = cc + lane, gj = n0 + c;
+        for (int k = 0; k < NR; ++k) {
+          const bool row = m0 + ew + OZ_EPI_WARPS * k < a.M;
+          cb[k][0] = row && in0 ? pc[0] : 0.0;
+          cb[k][1] = row && in1 ? pc[32] : 0.0;
+          pc += step;
+        }
+      }
+      const int64_t ld = part ? (int64_t)a.N : e.out ? e.ldo : e.ldo2;
+      double* po = (part ? part : e.out ? e.out : e.out2) + first * ld + gj0;
+      const int64_t so = OZ_EPI_WARPS * ld, sf = OZ_EPI_WARPS * e.ldof;
+      float* pf = F32 ? e.outf + first * e.ldof + gj0 : nullptr;
+      const unsigned long long flip = !part && e.alpha_unit < 0 ? 1ull << 63 : 0ull;
+#pragma unroll 1
+      for (int k = 0; k < NR; ++k) {
+        const int r = ew + OZ_EPI_WARPS * k;
+        if (m0 + r >= a.M) break;
+        double v0, v1;
+        product(r, __shfl_sync(0xffffffffu, ei_all, k), v0, v1);
+        v0 = __longlong_as_double(__double_as_longlong(v0) ^ flip);
+        v1 = __longlong_as_double(__double_as_longlong(v1) ^ flip);
+        if constexpr (CIN) {
+          v0 = cb[0][0] + v0;
+          v1 = cb[0][1] + v1;
+#pragma unroll
+          for (int j = 0; j + 1 < NR; ++j) {
+            cb[j][0] = cb[j + 1][0];
+            cb[j][1] = cb[j + 1][1];
+          }
+        }
+        if (in0) po[0] = v0;
+        if (in1) po[32] = v1;
+        po += so;
+        if constexpr (F32) {
+          if (in0) pf[0] = narrow(v0);
+          if (in1) pf[32] = narrow(v1);
+          pf += sf;
+        }
+        if (columns) {
+          *value_slot(r, lane) = v0;
+          *value_slot(r, lane + 32) = v1;
+        }
+      }
+    };
+    auto general_sweep = [&]() {
+#pragma unroll 1
+      for (int k = 0; k < NR; ++k) {
+        const int r = ew + OZ_EPI_WARPS * k, gi2 = m0 + r;
+        if (gi2 >= a.M) break;
+        double v0, v1;
+        product(r, __shfl_sync(0xffffffffu, ei_all, k), v0, v1);
+#pragma unroll 1
+        for (int u = 0; u < 2; ++u) {
+          const int gj = u ? gj1 : gj0;
+          double v = u ? v1 : v0;
           if (gj >= a.N || (e.sym && gj > gi2)) continue;
-          const double cval = tile[r * PITCH + c];
           if (part) {
-            part[(int64_t)gi2 * a.N + gj] = cval;
+            part[(int64_t)gi2 * a.N + gj] = v;
             continue;
           }
-          double v = e.alpha * cval;
-          if (e.cin) v += e.beta * e.cin[(int64_t)gi2 * e.ldcin + gj];
+          v = e.cin ? oz_axpby<true>(e, v, e.cin[(int64_t)gi2 * e.ldcin + gj]) : oz_axpby<false>(e, v, 0.0);
           if (gi2 == gj) v += e.delta;
-          if (e.radd_kind >= 0) v += oz_qv(e.radd_kind, e.radd, e.ldradd, gi2, gj);
+          v = oz_addq(v, e.radd_kind, e.radd, e.ldradd, gi2, gj);
           if (e.out) e.out[(int64_t)gi2 * e.ldo + gj] = v;
-          if (e.outf) e.outf[(int64_t)gi2 * e.ldof + gj] = (float)v;
-          if (e.out2) e.out2[(int64_t)gi2 * e.ldo2 + gj] = v + oz_qv(e.q_kind, e.q, e.ldq, gi2, gj);
+          if (e.outf) e.outf[(int64_t)gi2 * e.ldof + gj] = narrow(v);
+          if (e.out2) e.out2[(int64_t)gi2 * e.ldo2 + gj] = oz_addq(v, e.q_kind, e.q, e.ldq, gi2, gj);
           if (gi2 == gj) {
             if (e.diag_out) e.diag_out[gi2] = v;
             if (e.check_diag && !(v > 0.0 && isfinite(v))) status_set(e.status, KF_ERR_NUMERIC, e.step, gi2);
           }
-          tile[r * PITCH + c] = v;  // for the column sweep
+          *value_slot(r, lane + 32 * u) = v;
         }
       }
+    };
+    if (go) {
+      if (part || (fast && !e.cin)) {
+        fast_sweep(std::false_type{}, std::false_type{});
+      } else if (!WIDE && fast) {  // the wide sums leave no registers for a batch of cin
+        if constexpr (!WIDE) {
+          if (e.outf)
+            fast_sweep(std::true_type{}, std::true_type{});
+          else
+            fast_sweep(std::true_type{}, std::false_type{});
+        }
+      } else {
+        general_sweep();
+      }
     }
-    if (!part && (e.sym || e.outT)) {
+    if (columns && !a.sums) {
       asm volatile("bar.sync 1, %0;" ::"n"(32 * OZ_EPI_WARPS) : "memory");
-      if (go) {
+      const int rows = min(OZ_BM, a.M - m0);
+      // columns (gj, gi) of the mirrored and transposed outputs: consecutive lanes write consecutive places
+      auto fast_columns = [&](double* dst, int64_t ld, float* dstf) {
+        dst += (int64_t)(n0 + ew) * ld + m0 + lane;
+        const int64_t sd = OZ_EPI_WARPS * ld, sf = OZ_EPI_WARPS * e.ldof;
+        if (dstf) dstf += (int64_t)(n0 + ew) * e.ldof + m0 + lane;
+#pragma unroll 1
+        for (int c = ew; c < OZ_BN && n0 + c < a.N; c += OZ_EPI_WARPS) {
+          double v[OZ_BM / 32];
+#pragma unroll
+          for (int k = 0; k < OZ_BM / 32; ++k) v[k] = *value_slot(lane + 32 * k, c);
+#pragma unroll
+          for (int k = 0; k < OZ_BM / 32; ++k)
+            if (lane + 32 * k < rows) dst[32 * k] = v[k];
+          dst += sd;
+          if (dstf) {
+#pragma unroll
+            for (int k = 0; k < OZ_BM / 32; ++k)
+              if (lane + 32 * k < rows) dstf[32 * k] = narrow(v[k]);
+            dstf += sf;
+          }
+        }
+      };
+      if (go && fast && e.outT) {
+        fast_columns(e.outT, e.ldoT, nullptr);
+      } else if (go && fast) {
+        fast_columns(e.out ? e.out : e.out2, e.out ? e.ldo : e.ldo2, e.outf);
+      } else if (go) {
+#pragma unroll 1
         for (int c = ew; c < OZ_BN; c += OZ_EPI_WARPS) {
           const int gj = n0 + c;
           if (gj >= a.N) break;
-#pragma unroll
-          for (int rr = 0; rr < OZ_BM; rr += 32) {
-            const int r = rr + lane, gi2 = m0 + r;
-            if (gi2 >= a.M || (e.sym && gj > gi2)) continue;
-            const double v = tile[r * PITCH + c];
+#pragma unroll 1
+          for (int r = lane; r < rows; r += 32) {
+            const int gi2 = m0 + r;
+            if (e.sym && gj > gi2) continue;
+            const double v = *value_slot(r, c);
             if (e.outT) e.outT[(int64_t)gj * e.ldoT + gi2] = v;
-            if (e.sym && gi2 != gj) {  // mirror (gj, gi2): consecutive lanes write consecutive columns
+            if (e.sym && gi2 != gj) {  // mirror (gj, gi2)
               if (e.out) e.out[(int64_t)gj * e.ldo + gi2] = v;
-              if (e.outf) e.outf[(int64_t)gj * e.ldof + gi2] = (float)v;
-              if (e.out2) e.out2[(int64_t)gj * e.ldo2 + gi2] = v + oz_qv(e.q_kind, e.q, e.ldq, gj, gi2);
+              if (e.outf) e.outf[(int64_t)gj * e.ldof + gi2] = narrow(v);
+              if (e.out2) e.out2[(int64_t)gj * e.ldo2 + gi2] = oz_addq(v, e.q_kind, e.q, e.ldq, gj, gi2);
             }
           }
         }
@@ -670,10 +917,49 @@ __global__ void oz_reduce_kernel(int M, int N, int splits, const double* partial
   }
 }
 
-template <int LV, int BK>
+// Exact splits: integer sums of one 32 x 32 tile over the splits, scaled once, so the result is the one an
+// unsplit product gives; out along rows, outT along columns through shared memory.
+__global__ void __launch_bounds__(256) oz_sums_reduce_kernel(int M, int N, int splits, const long long* sums, int64_t ld,
+                                                             const int* ea, const int* eb, int scale, OzEpilogue e) {
+  __shared__ double tile[32][33];
+  __shared__ int skip;
+  if (threadIdx.x == 0) skip = status_failed(e.status) ? 1 : 0;
+  __syncthreads();
+  if (skip) return;
+  const int m0 = blockIdx.y * 32, n0 = blockIdx.x * 32, lane = threadIdx.x % 32, w = threadIdx.x / 32;
+  long long t[4] = {0, 0, 0, 0};
+  for (int sp = 0; sp < splits; ++sp) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int gi = m0 + w + 8 * k;
+      if (gi < M) t[k] += sums[((int64_t)sp * M + gi) * ld + n0 + lane];
+    }
+  }
+  const int gj = n0 + lane;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int gi = m0 + w + 8 * k;
+    if (gi >= M || gj >= N) continue;
+    const int ei = ea[gi], ej = eb[gj];
+    const double c = (ei == kOzBadRow || ej == kOzBadRow) ? __longlong_as_double(0x7ff8000000000000ll)
+                                                          : fixed_to_double(t[k], ei + ej + scale);
+    const double v = e.cin ? oz_axpby<true>(e, c, e.cin[(int64_t)gi * e.ldcin + gj]) : oz_axpby<false>(e, c, 0.0);
+    if (e.out) e.out[(int64_t)gi * e.ldo + gj] = v;
+    tile[w + 8 * k][lane] = v;
+  }
+  if (!e.outT) return;
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int gjt = n0 + w + 8 * k, gi = m0 + lane;
+    if (gjt < N && gi < M) e.outT[(int64_t)gjt * e.ldoT + gi] = tile[lane][w + 8 * k];
+  }
+}
+
+template <int LV, int LA, bool WIDE, int BK>
 kf_status launch_oz(cudaStream_t s, const OzSlices& A, const OzSlices& B, int M, int N, int K, const OzEpilogue& e,
-                    int splits, double* partials) {
-  using C = OzCfg<LV, BK>;
+                    int splits, double* partials, long long* sums) {
+  using C = OzCfg<LV, LA, BK>;
   OzMaps maps;
   KF_TRY(tma_map_bf16(&maps.a, A.planes, (int64_t)A.S * A.rows_pad, A.ldk, A.ldk, BK, OZ_BM, C::SWZ));
   KF_TRY(tma_map_bf16(&maps.b, B.planes, (int64_t)B.S * B.rows_pad, B.ldk, B.ldk, BK, OZ_BN, C::SWZ));
@@ -683,20 +969,35 @@ kf_status launch_oz(cudaStream_t s, const OzSlices& A, const OzSlices& B, int M,
   a.nk = (int)ceil_div(K, BK);
   // whole exact chunks per split, so chunk boundaries do not depend on the split
   a.kt_per_split = (int)(ceil_div(ceil_div(K, OZ_KC), splits) * C::CK);
-  a.partials = splits > 1 ? partials : nullptr;
+  a.partials = splits > 1 && !sums ? partials : nullptr;
+  a.sums = sums;
+  a.ld_sums = round_up(N, OZ_BN);
   a.a_rows_pad = (int)A.rows_pad;
   a.b_rows_pad = (int)B.rows_pad;
   a.ea = A.exps;
   a.eb = B.exps;
   a.e = e;
+  a.e.alpha_unit = e.alpha == 1.0 ? 1 : e.alpha == -1.0 ? -1 : 0;
+  a.e.beta_unit = e.beta == 1.0;
+  // one float64 output (plus a float32 copy with cin, or its transpose), unit alpha and beta, diagonal R and Q
+  const bool plain = a.e.alpha_unit != 0 && (!e.cin || a.e.beta_unit) && e.radd_kind != 2 && e.q_kind != 2 &&
+                     (e.out != nullptr) != (e.out2 != nullptr) && (!e.outf || e.cin) && !(e.sym && e.outT);
+  const bool no_diagonal = !e.sym && e.delta == 0.0 && e.radd_kind < 0 && e.q_kind < 0 && !e.diag_out;
+  a.e.simple = !plain ? 0 : no_diagonal ? 2 : 1;
   a.wait_ns = g_tc_wait_ns.load();
-  KF_CUDA_TRY(smem_limit_per_device((const void*)oz_gemm_kernel<LV, BK>, (int)C::SMEM));
+  KF_CUDA_TRY(smem_limit_per_device((const void*)oz_gemm_kernel<LV, LA, WIDE, BK>, (int)C::SMEM));
   const int64_t tiles = ceil_div(M, OZ_BM) * ceil_div(N, OZ_BN);
   if (g_oz_timer) g_oz_timer->before(s);
-  oz_gemm_kernel<LV, BK><<<dim3((unsigned)tiles, (unsigned)splits), OZ_THREADS, C::SMEM, s>>>(maps, a);
+  oz_gemm_kernel<LV, LA, WIDE, BK><<<dim3((unsigned)tiles, (unsigned)splits), OZ_THREADS, C::SMEM, s>>>(maps, a);
   if (g_oz_timer) g_oz_timer->after(s);
   note_launch();
   KF_TRY(launch_check("oz_gemm"));
+  if (sums) {
+    oz_sums_reduce_kernel<<<dim3((unsigned)ceil_div(N, 32), (unsigned)ceil_div(M, 32)), 256, 0, s>>>(
+        M, N, splits, sums, a.ld_sums, A.exps, B.exps, -14 - 8 * (LV - 1), a.e);
+    note_launch();
+    return launch_check("oz_sums_reduce");
+  }
   if (splits > 1) {
     const int64_t total = (int64_t)M * N;
     oz_reduce_kernel<<<(unsigned)std::min<int64_t>(ceil_div(total, 256), 4096), 256, 0, s>>>(M, N, splits, partials, e);
@@ -709,6 +1010,17 @@ kf_status launch_oz(cudaStream_t s, const OzSlices& A, const OzSlices& B, int M,
 }  // namespace
 
 thread_local TcLaunchTimer* g_oz_timer = nullptr;
+
+// Splits of K that give every SM a CTA when the output has too few tiles (U^T = P H^T at N = 1664, m = 128:
+// 26 tiles; 74 us as one pass over K, 25 us in five splits and 7 us for their sum).  At least two chunks per
+// split: its fixed part (pipeline fill, drain, epilogue, the sum) is worth about three.
+int64_t oz_sums_splits(int64_t M, int64_t N, int64_t K) {
+  const int64_t tiles = ceil_div(M, OZ_BM) * ceil_div(N, OZ_BN), chunks = ceil_div(K, OZ_KC);
+  if (tiles >= 152 || chunks < 4) return 1;
+  const int64_t s = std::min<int64_t>(std::min<int64_t>(152 / tiles, chunks / 2), 16);
+  if (s < 2) return 1;
+  return ceil_div(chunks, ceil_div(chunks, s));
+}
 
 uint64_t oz_slice_bytes(int64_t rows, int64_t cols, int S) {
   const uint64_t rp = round_up(std::max<int64_t>(rows, 1), OZ_ROW_PAD), ldk = round_up(std::max<int64_t>(cols, 1), 64);
@@ -741,22 +1053,36 @@ kf_status oz_slice(cudaStream_t s, const void* X, int64_t ld, int f64, int64_t r
 }
 
 kf_status oz_gemm(cudaStream_t s, const OzSlices& A, const OzSlices& B, int M, int N, int K, int levels,
-                  const OzEpilogue& e, int splits, double* partials) {
+                  const OzEpilogue& e, int splits, double* partials, const OzSums& work, int a_slices) {
+  const int la = a_slices > 0 ? a_slices : levels;
   if (M <= 0 || N <= 0) return KF_OK;
   if (K < 1 || K > (1 << 20)) return KF_ERR_ARG;
   if (!e.out && !e.outf && !e.outT && !e.out2 && !e.diag_out) return KF_ERR_ARG;
   if (M > A.rows || N > B.rows || K > A.ldk || K > B.ldk) return KF_ERR_ARG;
-  if (A.filled < levels || B.filled < levels || (e.sym && M != N)) return KF_ERR_ARG;
+  if (A.filled < la || B.filled < levels || (e.sym && M != N)) return KF_ERR_ARG;
   if (splits < 1 || splits > 64 || (splits > 1 && !partials)) return KF_ERR_ARG;
+  long long* sums = nullptr;
+  if (splits == 1 && levels == 5 && work.p && K <= kOzSumsMaxK && !e.sym && !e.outf && !e.out2 && !e.diag_out &&
+      e.radd_kind < 0 && e.delta == 0.0) {
+    const int64_t want = oz_sums_splits(M, N, K);
+    if (want > 1 && want * M * round_up(N, OZ_BN) <= work.count) {
+      splits = (int)want;
+      sums = work.p;
+    }
+  }
   // whole exact chunks per split, every split non-empty
   const int64_t chunks = ceil_div(K, OZ_KC);
   splits = (int)std::min<int64_t>(splits, chunks);
   splits = (int)ceil_div(chunks, ceil_div(chunks, splits));
-  switch (levels) {
-    case 4: return launch_oz<4, kOzBK>(s, A, B, M, N, K, e, splits, partials);
-    case 5: return launch_oz<5, kOzBK>(s, A, B, M, N, K, e, splits, partials);
-    case 6: return launch_oz<6, kOzBK>(s, A, B, M, N, K, e, splits, partials);
-    case 7: return launch_oz<7, kOzBK>(s, A, B, M, N, K, e, splits, partials);
+  // the sums of all levels fit 64 bits up to K 2^(8 LV + 6.1) < 2^62
+  const bool narrow_sums = levels < 5 || (levels == 5 && K <= kOzSumsMaxK);
+  switch (levels * 16 + la) {
+    case 4 * 16 + 4: return launch_oz<4, 4, false, kOzBK>(s, A, B, M, N, K, e, splits, partials, sums);
+    case 5 * 16 + 5:
+      return narrow_sums ? launch_oz<5, 5, false, kOzBK>(s, A, B, M, N, K, e, splits, partials, sums)
+                         : launch_oz<5, 5, true, kOzBK>(s, A, B, M, N, K, e, splits, partials, sums);
+    case 6 * 16 + 6: return launch_oz<6, 6, true, kOzBK>(s, A, B, M, N, K, e, splits, partials, sums);
+    case 7 * 16 + 7: return launch_oz<7, 7, true, kOzBK>(s, A, B, M, N, K, e, splits, partials, sums);
   }
   return KF_ERR_ARG;
 }

@@ -77,6 +77,8 @@ struct OzEpilogue {
   int sym = 0;
   int* status = nullptr;  // KF_ERR_TIMEOUT on an expired wait; kernels skip when already failed
   int step = 0;
+  // set by oz_gemm: alpha is 1 or -1 (else 0), beta is 1; the epilogue's usual forms (1: away from the diagonal)
+  int alpha_unit = 0, beta_unit = 0, simple = 0;
 };
 
 // Optional event timing of the exact-slice kernel launches alone (installed by a plan while it
@@ -88,7 +90,20 @@ extern thread_local TcLaunchTimer* g_oz_timer;
 // slices).  K <= 2^20.  splits > 1 divides K among that many CTAs per output
 // tile, whose float64 partial sums (splits x M x N doubles at `partials`) are
 // added in a fixed order by a second kernel that applies the epilogue.
+//
+// work (five levels, splits == 1, plain out / outT / cin epilogues): products with too few tiles for the GPU
+// and a long K are split too, into 64-bit integer sums (M x N rounded up to 64 per split) that a second kernel
+// adds; integers, so the result is bit for bit the unsplit one.
+// a_slices > 0: A has only that many slices (its other slices are zero by construction), and only their
+// products are formed.
+struct OzSums {
+  long long* p = nullptr;
+  int64_t count = 0;
+};
+constexpr int kOzSumsMaxK = 1 << 15;
+int64_t oz_sums_splits(int64_t M, int64_t N, int64_t K);  // the splits such a product gets (1: none)
 kf_status oz_gemm(cudaStream_t s, const OzSlices& A, const OzSlices& B, int M, int N, int K, int levels,
-                  const OzEpilogue& e, int splits = 1, double* partials = nullptr);
+                  const OzEpilogue& e, int splits = 1, double* partials = nullptr, const OzSums& work = OzSums{},
+                  int a_slices = 0);
 
 }  // namespace kfm

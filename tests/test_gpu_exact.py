@@ -201,3 +201,56 @@ def test_exact_product_wait_limit_timeout_then_recovery():
     ref, ea, eb = exact_sliced_product(A, Bm, 7)
     scale = np.ldexp(1.0, (ea[:, None] + eb[None, :]).astype(np.int64))
     assert np.all(np.abs(C.cpu().numpy() - ref) <= 2.0 ** -50 * scale + 4 * np.spacing(np.abs(ref)))
+
+
+@pytest.mark.parametrize("levels,K", [(5, 32768), (5, 32769), (6, 4096), (7, 8192)])
+def test_exact_product_largest_sums(levels, K):
+    """Same-sign rows of the largest digits: the fixed-point sums reach their largest magnitude on both
+    sides of the K up to which one 64-bit sum holds all levels; random rows beside them."""
+    rng = np.random.default_rng(levels + K)
+    M, N = 5, 3
+    A = rng.standard_normal((M, K))
+    Bm = rng.standard_normal((N, K))
+    A[0] = 1.0 - 2.0 ** -50
+    A[1] = -(1.0 - 2.0 ** -50)
+    Bm[0] = 1.0 - 2.0 ** -50
+    ref, ea, eb = exact_sliced_product(A, Bm, levels)
+    C = torch.zeros(M, N, dtype=torch.float64, device="cuda")
+    B.kfx_gemm_exact(levels, M, N, K, 1.0, torch.from_numpy(A).cuda(), K, torch.from_numpy(Bm).cuda(), K, 0.0, 0.0,
+                     C, N)
+    # the sums are exact integers, scaled with one rounding
+    assert np.array_equal(C.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("alpha,beta,delta", [(1.0, 1.0, 0.0), (-1.0, 1.0, 0.0), (-1.0, 0.0, 1.0), (0.5, -2.0, 0.25)])
+@pytest.mark.parametrize("M,N", [(128, 64), (129, 65), (300, 200), (40, 400)])
+def test_exact_product_epilogue_forms(alpha, beta, delta, M, N):
+    """The epilogue's own loops for unit alpha and beta and its general one, on tiles with and without
+    diagonal elements and with ragged edges: the same product plus the same float64 operations."""
+    rng = np.random.default_rng(M + N)
+    K, levels = 90, 5
+    A, Bm, C0 = rng.standard_normal((M, K)), rng.standard_normal((N, K)), rng.standard_normal((M, N))
+    dA, dB = torch.from_numpy(A).cuda(), torch.from_numpy(Bm).cuda()
+    P = torch.zeros(M, N, dtype=torch.float64, device="cuda")
+    B.kfx_gemm_exact(levels, M, N, K, 1.0, dA, K, dB, K, 0.0, 0.0, P, N)
+    C = torch.from_numpy(C0.copy()).cuda()
+    B.kfx_gemm_exact(levels, M, N, K, alpha, dA, K, dB, K, beta, delta, C, N)
+    ref = alpha * P.cpu().numpy()
+    if beta != 0.0:
+        ref = ref + beta * C0
+    ref += delta * np.eye(M, N)
+    assert np.allclose(C.cpu().numpy(), ref, rtol=4e-16, atol=4e-16 * np.abs(ref).max())  # fused or not
+
+
+@pytest.mark.parametrize("N,m", [(512, 64), (640, 40), (1100, 130)])
+def test_filter_products_split_over_k(N, m):
+    """U^T = P H^T with few output tiles is split over K into integer sums: the mixed filter against the
+    oracle at sizes with two and more splits.  Tolerance: the product's bound 2^-35 K on diag P, and the
+    mixed path's 1e-4 on means; a lost or doubled split is an error of order one."""
+    from paper_1107_4192_gb300 import solver, synth
+    from tests.helpers import diag_of, rel_err_elementwise, rel_err_per_step, run_oracle
+    prob = synth.mesh_problem(N, m, 3, seed=N)
+    out = solver.run(prob, prec=B.KF_PREC_MIXED_BF16X3, solve_prec=B.KF_SOLVE_FP64_MEAN, joseph_every=2)
+    ref = run_oracle(prob)
+    assert rel_err_elementwise(out["diagP_filt"], diag_of(ref["P_filt"])) <= 2.0 ** -35 * N
+    assert rel_err_per_step(out["x_filt"], ref["x_filt"]) <= 1e-4
