@@ -19,7 +19,7 @@
 //           128-wide chunk it commits the level's buffer to its "ready"
 //           barrier, and a level's next chunk starts (overwriting) in a buffer
 //           the epilogue has drained;
-//   warp 2  the gate: waits for each k-step's operands and drained buffer and releases it to warp 1;
+//   warp 2  the gate: waits for each step's operands and drained buffer and releases it to warp 1;
 //   warps 3-18 per chunk and level, read the accumulator (an exact integer
 //           below 2^24), convert it to an integer and add it into 64-bit
 //           fixed-point accumulators in registers (levels 0-2 and levels 3..
@@ -37,9 +37,9 @@ namespace {
 
 constexpr int OZ_BM = 128;      // output rows per CTA (TMEM lanes)
 constexpr int OZ_BN = 64;       // output columns per CTA (TMEM columns per level)
-constexpr int OZ_KC = 128;      // values of k per exact chunk
+constexpr int OZ_SPLIT_K = 128; // K splits begin at multiples of this
 constexpr int OZ_EPI_WARPS = 16;  // 4 TMEM lane quadrants x 4 column quarters of 16
-constexpr int OZ_GATE_WARP = 2;   // waits for each k-step's operands and buffer
+constexpr int OZ_GATE_WARP = 2;   // waits for each step's operands and buffer
 constexpr int OZ_EPI0 = 3;        // first epilogue warp
 constexpr int OZ_THREADS = 32 * (OZ_EPI0 + OZ_EPI_WARPS);
 constexpr int OZ_GROUP = 8;     // row tiles per rasterisation group (operand reuse in L2)
@@ -57,9 +57,19 @@ struct OzCfg {
   static constexpr int SWZ = BK * 2;                         // swizzle width in bytes
   static constexpr uint32_t LAYOUT = BK == 16 ? kLayoutSw32 : kLayoutSw64;  // descriptor swizzle mode
   static constexpr uint32_t SBO = 8 * SWZ;                   // bytes between 8-row groups
-  static constexpr int KS = BK / 16;                         // MMA k-steps per stage
-  static constexpr int CK = OZ_KC / BK;                      // stages per exact chunk
-  static constexpr int CKS = OZ_KC / 16;                     // k-steps per exact chunk
+  // values of k per exact chunk: a level has at most LA slice pairs, whose products are at most 2^14 in
+  // magnitude, so a chunk sums to an integer of at most 2^24, exact in float32.  As long as that allows: draining
+  // a level costs the epilogue about 1100 cycles whatever the chunk's length, and with 128 for all the
+  // drains, not the MMAs, set the pace of the products with few slices of A (<7, 3> 21.1 ms and <5, 2>
+  // 14.4 ms at N = 8196; with these chunks 19.7 and 12.5 ms).
+  static constexpr int KC = LA <= 2 ? 512 : LA <= 4 ? 256 : LA == 5 ? 192 : 128;
+  // SK MMA k-steps (of 16) make one step, the unit in which levels start chunks and the roles synchronise: a
+  // whole stage where a chunk still has more stages than there are levels, since a step costs about 390
+  // cycles (gate, commits, an empty MMA queue) beside its MMAs (N = 8196: <7, 3> 19.7 -> 15.8 ms, 0.74 of the
+  // sustained bf16 rate; <5, 2> 12.5 -> 9.4 ms).
+  static constexpr int SK = KC / BK > LV ? BK / 16 : 1;
+  static constexpr int KS = BK / 16 / SK;                    // steps per stage
+  static constexpr int CKS = KC / (16 * SK);                 // steps per exact chunk
   static constexpr int A_BYTES = OZ_BM * BK * 2;
   static constexpr int B_BYTES = OZ_BN * BK * 2;
   static constexpr int STAGE_BYTES = LA * A_BYTES + LV * B_BYTES;
@@ -70,10 +80,8 @@ struct OzCfg {
   // so the buffer a level leaves is drained while the MMAs continue in the spare one
   static constexpr int NB = LV + 1;
   static_assert(NB * OZ_BN <= 512, "one TMEM accumulator per level plus a spare");
-  static_assert(LV < CKS && CKS == 8, "one level changes chunk per k-step; eight k-step patterns");
-  // a level has at most LV slice pairs whose products are below 2^14 in magnitude, so one
-  // chunk of OZ_KC values of k sums to an integer below 2^24: exact in float32
-  static_assert(LV * OZ_KC * 16384 <= (1 << 24), "exact chunk");
+  static_assert(LV < CKS, "one level changes chunk per step");
+  static_assert(LA * KC * 16384 <= (1 << 24), "exact chunk");
   static_assert(2 * STAGES + 2 * NB + 1 <= 28, "barriers fit their 256 bytes");
   static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024 + 256;
   // instruction descriptor: D = f32, A = B = bf16, both K-major, M >> 4; N >> 3 at bit 17 per MMA
@@ -259,11 +267,19 @@ __device__ __forceinline__ unsigned long long mag_bits(double x) {
 __device__ __forceinline__ unsigned long long mag_bits(float x) {
   return ((unsigned long long)(__float_as_uint(x) & 0x7FFFFFFFu)) << 29;  // same order as a double's bits
 }
-__device__ __forceinline__ int frexp_exponent(unsigned long long mag, bool f32) {
-  const double v = f32 ? (double)__uint_as_float((unsigned)(mag >> 29)) : __longlong_as_double((long long)mag);
-  int e = 0;
-  if (v > 0.0) frexp(v, &e);
-  return e;
+// Magnitude bits from which on a value is an infinity or NaN.
+template <typename T>
+__device__ __forceinline__ unsigned long long mag_inf() {
+  return sizeof(T) == 8 ? 0x7FF0000000000000ull : 0x7F800000ull << 29;
+}
+// The binary exponent e of magnitude bits: 2^(e-1) <= value < 2^e (0 for zero), as frexp gives it.
+template <typename T>
+__device__ __forceinline__ int mag_exponent(unsigned long long mag) {
+  const int E = (int)(mag >> 52);
+  if (E > 0) return E - (sizeof(T) == 8 ? 1022 : 126);
+  if (mag == 0) return 0;
+  const int top = 63 - __clzll((long long)mag);  // subnormal: leading bit of the mantissa
+  return sizeof(T) == 8 ? top - 1073 : top - 29 - 148;
 }
 
 // x 2^shift rounded to the nearest integer, ties to even (exact integer arithmetic).
@@ -275,77 +291,241 @@ __device__ __forceinline__ long long fixed_rne(long long mant, int exp2, bool ne
     r = total >= 63 ? 0 : mant << total;
   } else {
     const int sh = -total;
-    if (sh >= 63) {
-      r = 0;
-    } else {
-      long long q = mant >> sh;
-      const long long rem = mant & ((1ll << sh) - 1), half = 1ll << (sh - 1);
-      if (rem > half || (rem == half && (q & 1))) ++q;
-      r = q;
-    }
+    r = sh >= 63 ? 0 : (mant + ((1ll << (sh - 1)) - 1) + ((mant >> sh) & 1)) >> sh;
   }
   return neg ? -r : r;
 }
 
-// Slices of one row: X[r][k] = 2^(e - 7 - 8(S-1)) X_int with X_int = RNE(X[r][k] 2^(7 + 8(S-1) - e)),
-// written in signed base-256 digits q_0 .. q_{S-1} (each rounded to nearest, ties to even, so
-// |q_p| <= 128), all in integer arithmetic.
+// Eight consecutive values of a row, from k0 on (zero at and beyond cols).
 template <typename T>
-__global__ void __launch_bounds__(256) oz_slice_kernel(const T* X, int64_t ld, int64_t rows, int64_t cols, int S,
-                                                       __nv_bfloat16* planes, int64_t rows_pad, int64_t ldk,
-                                                       int* exps) {
-  __shared__ unsigned long long red[8];
-  const int64_t r = blockIdx.x;
-  const T* row = X + r * ld;
-  unsigned long long mx = 0;
-  if (r < rows)
-    for (int64_t k = threadIdx.x; k < cols; k += blockDim.x) {
-      const unsigned long long v = mag_bits(row[k]);
-      mx = v > mx ? v : mx;
+__device__ __forceinline__ void load8(const T* row, int64_t k0, int64_t cols, bool vec, T (&v)[8]) {
+  if (vec && k0 + 8 <= cols) {
+    if constexpr (sizeof(T) == 8) {
+#pragma unroll
+      for (int i = 0; i < 8; i += 2) {
+        const double2 d = *reinterpret_cast<const double2*>(row + k0 + i);
+        v[i] = d.x;
+        v[i + 1] = d.y;
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; i += 4) {
+        const float4 f = *reinterpret_cast<const float4*>(row + k0 + i);
+        v[i] = f.x;
+        v[i + 1] = f.y;
+        v[i + 2] = f.z;
+        v[i + 3] = f.w;
+      }
     }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = k0 + i < cols ? row[k0 + i] : T(0);
+  }
+}
+
+// Signed base-256 digits of eight integers |x| <= 2^(8S - 1), written as bf16 to S planes (16-byte stores).
+// Digit p is q_p = Q_p - 256 Q_{p-1} with Q_p = x / 2^(8(S-1-p)) rounded to nearest, ties to even: the
+// successive rounding of the remainders, since a remainder differs from x by multiples of 256 2^(8(S-1-p)).
+// The low 32 bits of each Q_p are enough.
+__device__ __forceinline__ void write_digits8(const long long (&x)[8], int S, __nv_bfloat16* dst, int64_t pstride) {
+  uint32_t prev[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) prev[i] = 0;
+  for (int p = 0; p < S; ++p, dst += pstride) {
+    const int sp = 8 * (S - 1 - p);
+    uint32_t w[4];
+    float f[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      uint32_t q;
+      if (sp > 0)
+        q = (uint32_t)((x[i] + ((1ll << (sp - 1)) - 1) + ((x[i] >> sp) & 1)) >> sp);
+      else
+        q = (uint32_t)x[i];
+      const uint32_t d = q - (prev[i] << 8);
+      prev[i] = q;
+      f[i] = __uint_as_float(0x4B400000u + d) - 12582912.0f;  // (float)(int)d for |d| < 2^22
+    }
+#pragma unroll
+    for (int i = 0; i < 8; i += 2)  // |d| <= 128: exact in bf16, the upper half of the float32
+      w[i / 2] = __byte_perm(__float_as_uint(f[i]), __float_as_uint(f[i + 1]), 0x7632);
+    *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+
+template <typename T>
+__device__ __forceinline__ void slice8(const T (&v)[8], int shift, bool bad, int S, __nv_bfloat16* dst, int64_t pstride) {
+  long long x[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    long long mant;
+    int exp2;
+    bool neg;
+    decompose(v[i], mant, exp2, neg);
+    x[i] = bad ? 0 : fixed_rne(mant, exp2, neg, shift);
+  }
+  write_digits8(x, S, dst, pstride);
+}
+
+// Maximum over the warp (kGroup 32) or the 256-thread block, to all its threads.
+template <int kGroup>
+__device__ __forceinline__ unsigned long long group_max(unsigned long long mx) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const unsigned long long v = __shfl_xor_sync(0xffffffffu, mx, o);
     mx = v > mx ? v : mx;
   }
-  if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = mx;
-  __syncthreads();
-  mx = red[0];
-  for (int w = 1; w < (int)blockDim.x / 32; ++w) mx = red[w] > mx ? red[w] : mx;
-  const bool row_bad = mx >= 0x7FF0000000000000ull;  // an infinity or NaN: zero slices, marked exponent
-  const int e = row_bad ? 0 : frexp_exponent(mx, sizeof(T) == 4);  // max |X[r]| < 2^e
-  if (threadIdx.x == 0) exps[r] = row_bad ? kOzBadRow : e;
+  if constexpr (kGroup == 256) {
+    __shared__ unsigned long long red[8];
+    if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = mx;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < 8; ++w) mx = red[w] > mx ? red[w] : mx;
+  }
+  return mx;
+}
+
+// Slices of the rows: X[r][k] = 2^(e - 7 - 8(S-1)) X_int with X_int = RNE(X[r][k] 2^(7 + 8(S-1) - e)), in
+// signed base-256 digits (|q_p| <= 128), all in integer arithmetic.  A group (a warp for short rows, else a
+// 256-thread block) holds its row in registers, 8 NCH values per thread, so a row is read once: HBM-bound from
+// a few thousand columns on (5124 x 5124 float64, 5 slices: 246 us with the digits in 64-bit arithmetic and two
+// reads, 85 us now; 1664 x 128: 14.5 us and 5 us).  NCH = 0: two passes, for rows too long for that.
+template <typename T, int kGroup, int NCH>
+__global__ void __launch_bounds__(256) oz_slice_kernel(const T* X, int64_t ld, int64_t rows, int64_t cols, int S,
+                                                       __nv_bfloat16* planes, int64_t rows_pad, int64_t ldk,
+                                                       int* exps) {
+  constexpr int kRows = 256 / kGroup;
+  const int64_t r = (int64_t)blockIdx.x * kRows + threadIdx.x / kGroup;  // rows_pad is a multiple of kRows
+  const int t = threadIdx.x % kGroup;
+  const T* row = X + (r < rows ? r : 0) * ld;
+  const int64_t n = r < rows ? cols : 0;  // rows beyond the matrix are zero
+  const bool vec = (reinterpret_cast<uintptr_t>(X) & 15) == 0 && (ld * sizeof(T)) % 16 == 0;
+  unsigned long long mx = 0;
+  T v[NCH > 0 ? NCH : 1][8];
+  if constexpr (NCH > 0) {
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) load8(row, (int64_t)(c * kGroup + t) * 8, n, vec, v[c]);
+#pragma unroll
+    for (int c = 0; c < NCH; ++c)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const unsigned long long m = mag_bits(v[c][i]);
+        mx = m > mx ? m : mx;
+      }
+  } else {
+    for (int64_t k = t; k < n; k += kGroup) {
+      const unsigned long long m = mag_bits(row[k]);
+      mx = m > mx ? m : mx;
+    }
+  }
+  mx = group_max<kGroup>(mx);
+  const bool bad = mx >= mag_inf<T>();  // an infinity or NaN: zero slices, marked exponent
+  const int e = bad ? 0 : mag_exponent<T>(mx);  // max |X[r]| < 2^e
+  if (t == 0) exps[r] = bad ? kOzBadRow : e;
   const int shift = 7 + 8 * (S - 1) - e;
   const int64_t pstride = rows_pad * ldk;
-  for (int64_t k0 = threadIdx.x * 8; k0 < ldk; k0 += (int64_t)blockDim.x * 8) {
-    long long xi[8];
+  __nv_bfloat16* dst = planes + r * ldk;
+  if constexpr (NCH > 0) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      xi[i] = 0;
-      if (r < rows && k0 + i < cols && !row_bad) {
-        long long mant;
-        int exp2;
-        bool neg;
-        decompose(row[k0 + i], mant, exp2, neg);
-        xi[i] = fixed_rne(mant, exp2, neg, shift);
+    for (int c = 0; c < NCH; ++c) {
+      const int64_t k0 = (int64_t)(c * kGroup + t) * 8;
+      if (k0 < ldk) slice8(v[c], shift, bad, S, dst + k0, pstride);
+    }
+  } else {
+    for (int64_t k0 = (int64_t)t * 8; k0 < ldk; k0 += kGroup * 8) {
+      load8(row, k0, n, vec, v[0]);
+      slice8(v[0], shift, bad, S, dst + k0, pstride);
+    }
+  }
+}
+
+// Row exponents alone (float32), as oz_slice_kernel finds them.
+__global__ void __launch_bounds__(256) oz_exps_kernel(const float* X, int64_t ld, int64_t n, int* exps) {
+  const int64_t r = blockIdx.x;
+  unsigned long long mx = 0;
+  const float* row = X + r * ld;
+  if (r < n)
+    for (int64_t k = threadIdx.x * 4; k < n; k += 1024) {  // ld is a multiple of 4 and rows are 16-byte aligned
+      const float4 f = *reinterpret_cast<const float4*>(row + k);
+      const float v[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const unsigned long long m = k + i < n ? mag_bits(v[i]) : 0;
+        mx = m > mx ? m : mx;
       }
     }
-    for (int p = 0; p < S; ++p) {
-      const int sp = 8 * (S - 1 - p);
-      uint32_t w[4];
+  mx = group_max<256>(mx);
+  if (threadIdx.x == 0) exps[r] = mx >= mag_inf<float>() ? kOzBadRow : mag_exponent<float>(mx);
+}
+
+// A symmetric float32 matrix rounded so that three slices hold it exactly and it stays symmetric: element
+// (i, j) to the nearest multiple of 2^(max(e_i, e_j) - 23), written back, with its three slices by rows.
+__global__ void __launch_bounds__(256) oz_slice_symmetric_kernel(float* X, int64_t ld, int64_t n, __nv_bfloat16* planes,
+                                                                 int64_t rows_pad, int64_t ldk, const int* exps) {
+  const int64_t r = blockIdx.x;
+  const int er = exps[r];
+  const bool live = r < n && er != kOzBadRow;
+  float* row = X + (r < n ? r : 0) * ld;
+  for (int64_t k0 = threadIdx.x * 8; k0 < ldk; k0 += 256 * 8) {
+    long long x[8];
+    float v[8];
+    load8(row, k0, live ? n : 0, true, v);
 #pragma unroll
-      for (int i = 0; i < 8; i += 2) {
-        __nv_bfloat16 h[2];
+    for (int i = 0; i < 8; ++i) {
+      const int ek = k0 + i < n ? exps[k0 + i] : er;
+      const int g = ek == kOzBadRow ? er : max(er, ek);
+      long long mant;
+      int exp2;
+      bool neg;
+      decompose(v[i], mant, exp2, neg);
+      const long long q = fixed_rne(mant, exp2, neg, 23 - g);
+      x[i] = q << min(g - er, 40);  // |x| <= 2^23: the grid only gets coarser as g - er grows
+      v[i] = ldexpf((float)q, g - 23);
+    }
+    write_digits8(x, 3, planes + r * ldk + k0, rows_pad * ldk);
+    if (live) {
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          long long q = xi[i + j];
-          if (sp > 0) q = (q + (1ll << (sp - 1)) - 1 + ((q >> sp) & 1)) >> sp;
-          xi[i + j] -= q << sp;
-          h[j] = __float2bfloat16_rn((float)q);
-        }
-        w[i / 2] = (uint32_t)__bfloat16_as_ushort(h[0]) | ((uint32_t)__bfloat16_as_ushort(h[1]) << 16);
-      }
-      *reinterpret_cast<uint4*>(planes + p * pstride + r * ldk + k0) = make_uint4(w[0], w[1], w[2], w[3]);
+      for (int i = 0; i < 8; ++i)
+        if (k0 + i < n) row[k0 + i] = v[i];
+    }
+  }
+}
+
+// Two slices Cs of the rows of a float32 correction C (rounded to nearest), and X = Y + Cs in float64 for a
+// float32 Y.
+__global__ void __launch_bounds__(256) oz_slice_correction_kernel(const float* C, const float* Y, int64_t ld, int64_t n,
+                                                                  __nv_bfloat16* planes, int64_t rows_pad, int64_t ldk,
+                                                                  int* exps, double* X, int64_t ldx) {
+  const int64_t r = blockIdx.x;
+  const float* row = C + (r < n ? r : 0) * ld;
+  unsigned long long mx = 0;
+  if (r < n)
+    for (int64_t k = threadIdx.x; k < n; k += 256) {
+      const unsigned long long m = mag_bits(row[k]);
+      mx = m > mx ? m : mx;
+    }
+  mx = group_max<256>(mx);
+  const bool bad = mx >= mag_inf<float>();
+  const int e = bad ? 0 : mag_exponent<float>(mx);
+  if (threadIdx.x == 0) exps[r] = bad ? kOzBadRow : e;
+  for (int64_t k0 = threadIdx.x * 8; k0 < ldk; k0 += 256 * 8) {
+    long long x[8];
+    float v[8], y[8];
+    load8(row, k0, r < n ? n : 0, true, v);
+    load8(Y + (r < n ? r : 0) * ld, k0, r < n ? n : 0, true, y);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      long long mant;
+      int exp2;
+      bool neg;
+      decompose(v[i], mant, exp2, neg);
+      x[i] = bad ? 0 : fixed_rne(mant, exp2, neg, 15 - e);
+    }
+    write_digits8(x, 2, planes + r * ldk + k0, rows_pad * ldk);
+    if (r < n) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (k0 + i < n) X[r * ldx + k0 + i] = (double)y[i] + (double)ldexpf((float)x[i], e - 15);
     }
   }
 }
@@ -374,51 +554,57 @@ __device__ __forceinline__ void oz_drain(uint32_t taddr, uint32_t dbar, int lane
   }
 }
 
-// The MMAs of one k-step t with r = t mod CKS.  Level l's exact chunks are staggered by l k-steps
-// and chunk k of level l accumulates in TMEM buffer (l + k) mod NB, so at this k-step level l sits
-// in buffer (l + [l >= CKS - r] + cm) mod NB, cm = (t / CKS) mod NB.  Per A slice pa, its
-// partner levels pa .. LV-1 go in runs of up to four levels, split at the level CKS - r that has
-// moved on (fixed by r, so the runs and all shared-memory offsets are compile-time): one MMA with
+// The MMAs of one step t with r = t mod CKS.  Level l's exact chunks are staggered by l steps
+// and chunk k of level l accumulates in TMEM buffer (l + k) mod NB, so at this step level l sits
+// in buffer (l + [l >= CKS - r] + cm) mod NB, cm = (t / CKS) mod NB.  PAT is what that depends on: the level
+// CKS - r that starts a chunk here (all above it have moved on), 0 for r = 0, LV where none does.  Per A
+// slice pa, its partner levels pa .. LV-1 go in runs of up to four levels, split at the level that has
+// moved on (so the runs and all shared-memory offsets are compile-time): one MMA with
 // N = 64 x run takes the adjacent B slices pb .. pb+run-1 into the run's adjacent accumulators; a
 // run whose buffers pass the last one (known from cm at run time) is issued as two MMAs.  The level
-// LS that starts a chunk at this k-step gets its own MMA at pa = 0, the chunk's first, which
-// overwrites the accumulator instead of adding to it (at the first k-step every level starts, and
+// that starts a chunk at this step gets its own MMA at pa = 0, the chunk's first, which
+// overwrites the accumulator instead of adding to it (at the first step every level starts, and
 // all of pa = 0's MMAs overwrite).  `pre` runs after the MMAs of the first A slices, about half
-// of the k-step's work.
-template <int LV, int LA, int BK, int R, typename Pre>
-__device__ __forceinline__ void oz_issue_kstep(bool leader, uint32_t tmem, uint64_t adesc0, uint64_t bdesc0, int cm,
+// of the step's work.
+template <int LV, int LA, int BK, int PAT, typename Pre>
+__device__ __forceinline__ void oz_issue_step(bool leader, uint32_t tmem, uint64_t adesc0, uint64_t bdesc0, int cm,
                                                bool first_step, Pre&& pre) {
   using C = OzCfg<LV, LA, BK>;
-  constexpr int LS = R == 0 ? 0 : C::CKS - R;
-  constexpr int PRE_AFTER = LA >= 5 ? 2 : 1;
+  constexpr int MOVED = PAT == 0 ? LV : PAT;      // levels from here on have moved on
 #pragma unroll
-  for (int pa = 0; pa < LA; ++pa) {
-    if (pa == PRE_AFTER) pre();
-    int l0 = pa;
+  for (int sub = 0; sub < C::SK; ++sub) {
+    // the next 32 bytes of every swizzled row (start address in 16-byte units)
+    const uint64_t as = adesc0 + (uint64_t)(2 * sub), bs = bdesc0 + (uint64_t)(2 * sub);
+    const int LS = sub == 0 ? PAT : LV;           // the level that starts a chunk (LV: none)
 #pragma unroll
-    for (int l = pa + 1; l <= LV; ++l) {
-      if (l == LV || l - l0 == 4 || l == C::CKS - R || (pa == 0 && LS < LV && l == LS + 1)) {
-        const int run = l - l0;
-        const uint32_t acc = (pa == 0 && (first_step || l0 == LS)) ? 0u : 1u;
-        int b = l0 + (l0 >= C::CKS - R ? 1 : 0) + cm;
-        if (b >= C::NB) b -= C::NB;
-        const int first = min(run, C::NB - b);
-        // the start-address field (bits 0-13, 16-byte units) absorbs the in-stage offsets
-        const uint64_t ad = adesc0 + (uint64_t)((pa * C::A_BYTES) >> 4);
-        const uint64_t bd = bdesc0 + (uint64_t)(((l0 - pa) * C::B_BYTES) >> 4);
-        if (leader) {
-          mma_bf16(tmem + (uint32_t)(b * OZ_BN), ad, bd, C::IDESC_M | ((uint32_t)(first * OZ_BN) >> 3 << 17), acc);
-          if (first < run)
-            mma_bf16(tmem, ad, bd + (uint64_t)((first * C::B_BYTES) >> 4),
-                     C::IDESC_M | ((uint32_t)((run - first) * OZ_BN) >> 3 << 17), acc);
+    for (int pa = 0; pa < LA; ++pa) {
+      if (C::SK == 1 ? pa == (LA >= 5 ? 2 : 1) : (sub == C::SK - 1 && pa == 0)) pre();
+      int l0 = pa;
+#pragma unroll
+      for (int l = pa + 1; l <= LV; ++l) {
+        if (l == LV || l - l0 == 4 || l == MOVED || (pa == 0 && LS < LV && l == LS + 1)) {
+          const int run = l - l0;
+          const uint32_t acc = (pa == 0 && sub == 0 && (first_step || l0 == LS)) ? 0u : 1u;
+          int b = l0 + (l0 >= MOVED ? 1 : 0) + cm;
+          if (b >= C::NB) b -= C::NB;
+          const int first = min(run, C::NB - b);
+          // the start-address field (bits 0-13, 16-byte units) absorbs the in-stage offsets
+          const uint64_t ad = as + (uint64_t)((pa * C::A_BYTES) >> 4);
+          const uint64_t bd = bs + (uint64_t)(((l0 - pa) * C::B_BYTES) >> 4);
+          if (leader) {
+            mma_bf16(tmem + (uint32_t)(b * OZ_BN), ad, bd, C::IDESC_M | ((uint32_t)(first * OZ_BN) >> 3 << 17), acc);
+            if (first < run)
+              mma_bf16(tmem, ad, bd + (uint64_t)((first * C::B_BYTES) >> 4),
+                       C::IDESC_M | ((uint32_t)((run - first) * OZ_BN) >> 3 << 17), acc);
+          }
+          l0 = l;
         }
-        l0 = l;
       }
     }
   }
 }
 
-// The gate counter: the number of k-steps whose operands have landed and whose starting level's
+// The gate counter: the number of steps whose operands have landed and whose starting level's
 // buffer has been drained (written by the gate warp with release, read by the MMA warp with acquire).
 __device__ __forceinline__ uint32_t oz_gate_load(uint32_t addr) {
   uint32_t v;
@@ -428,7 +614,7 @@ __device__ __forceinline__ uint32_t oz_gate_load(uint32_t addr) {
 __device__ __forceinline__ void oz_gate_store(uint32_t addr, uint32_t v) {
   asm volatile("st.release.cta.shared::cta.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
-// Bounded wait until the gate passes k-step t; false on timeout or abort.
+// Bounded wait until the gate passes step t; false on timeout or abort.
 __device__ __forceinline__ bool oz_gate_wait(uint32_t addr, uint32_t t, volatile int* abort_flag, uint64_t limit_ns,
                                              uint32_t& gate) {
   gate = oz_gate_load(addr);
@@ -469,7 +655,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(const __grid_con
       reinterpret_cast<uint32_t*>(gbase + C::STAGES * C::STAGE_BYTES + 8 * (2 * C::STAGES + 2 * C::NB + 1));
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   volatile int* skip_flag = reinterpret_cast<volatile int*>(tmem_slot + 2);
-  const uint32_t gate_addr = smem_u32(tmem_slot + 3);  // k-steps released to the MMA warp
+  const uint32_t gate_addr = smem_u32(tmem_slot + 3);  // steps released to the MMA warp
   volatile int never = 0;  // abort flag of the clean-up waits, which must not stop early
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -531,21 +717,20 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(const __grid_con
   } else if (warp == 1) {
     // ---------------- MMA issuer: the whole warp runs the loop, so the stage, buffer and descriptor
     // arithmetic is warp-uniform; one elected lane issues.  TMEM buffer b = columns [64 b, 64 b + 64).
-    // The gate warp tells it which k-steps may start (operands landed, new buffer drained); the
-    // MMA queue is shallow, so the issuer does no barrier test of its own between k-steps: it reads
-    // the gate counter half-way through each k-step's MMAs, and that load's latency overlaps them.
+    // The gate warp tells it which steps may start (operands landed, new buffer drained); the
+    // MMA queue is shallow, so the issuer does no barrier test of its own between steps: it reads
+    // the gate counter half-way through each step's MMAs, and that load's latency overlaps them.
     leader = elect_one();
     bool ok = true;
-    uint32_t gate = 0;  // k-steps released so far (last value read)
+    uint32_t gate = 0;  // steps released so far (last value read)
     const int nks = nk * C::KS;
+    int s = 0, t = 0, r = 0, cm = 0;  // stage, step, step in the chunk, chunk mod NB
     for (int it = 0; it < nk && ok; ++it) {
-      const int s = it % C::STAGES;
       const uint32_t st = base + s * C::STAGE_BYTES;
       const uint64_t adesc_s = smem_desc_sw(st, C::SBO, C::LAYOUT);
       const uint64_t bdesc_s = smem_desc_sw(st + LA * C::A_BYTES, C::SBO, C::LAYOUT);
 #pragma unroll
       for (int j = 0; j < C::KS; ++j) {
-        const int t = it * C::KS + j;  // k-step
         if (gate <= (uint32_t)t) {
           ok = __all_sync(0xffffffffu, oz_gate_wait(gate_addr, (uint32_t)t, abort_flag, a.wait_ns, gate));
           gate = __shfl_sync(0xffffffffu, gate, 0);
@@ -558,46 +743,62 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(const __grid_con
           }
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const int ck = t / C::CKS, r = t - ck * C::CKS, cm = ck % C::NB;
-        auto buf = [&](int l) {  // buffer of level l at this k-step
+        auto buf = [&](int l) {  // buffer of level l at this step
           const int b = l + cm + (l >= C::CKS - r ? 1 : 0);
           return b >= C::NB ? b - C::NB : b;
         };
         uint32_t gate_ahead = gate;
         auto pre = [&]() { gate_ahead = oz_gate_load(gate_addr); };
-        // k-step j reads the next 32 bytes of every swizzled row (start address in 16-byte units)
-        const uint64_t adesc0 = adesc_s + (uint64_t)(2 * j), bdesc0 = bdesc_s + (uint64_t)(2 * j);
-        switch (r) {
-          case 0: oz_issue_kstep<LV, LA, BK, 0>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
-          case 1: oz_issue_kstep<LV, LA, BK, 1>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
-          case 2: oz_issue_kstep<LV, LA, BK, 2>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
-          case 3: oz_issue_kstep<LV, LA, BK, 3>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
-          case 4: oz_issue_kstep<LV, LA, BK, 4>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
-          case 5: oz_issue_kstep<LV, LA, BK, 5>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
-          case 6: oz_issue_kstep<LV, LA, BK, 6>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
-          default: oz_issue_kstep<LV, LA, BK, 7>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
+        const uint64_t adesc0 = adesc_s + (uint64_t)(2 * j * C::SK), bdesc0 = bdesc_s + (uint64_t)(2 * j * C::SK);
+        switch (r == 0 ? 0 : min(C::CKS - r, LV)) {
+          case 0: oz_issue_step<LV, LA, BK, 0>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
+          case 1: oz_issue_step<LV, LA, BK, 1>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
+          case 2: oz_issue_step<LV, LA, BK, 2>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
+          case 3: oz_issue_step<LV, LA, BK, 3>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
+          case 4:
+            if constexpr (LV > 4) oz_issue_step<LV, LA, BK, 4>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre);
+            else oz_issue_step<LV, LA, BK, LV>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre);
+            break;
+          case 5:
+            if constexpr (LV > 5) oz_issue_step<LV, LA, BK, 5>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre);
+            else oz_issue_step<LV, LA, BK, LV>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre);
+            break;
+          case 6:
+            if constexpr (LV > 6) oz_issue_step<LV, LA, BK, 6>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre);
+            else oz_issue_step<LV, LA, BK, LV>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre);
+            break;
+          default: oz_issue_step<LV, LA, BK, LV>(leader, tmem, adesc0, bdesc0, cm, t == 0, pre); break;
         }
         __syncwarp();
         mma_issued = true;
-        if (leader) {  // the level whose chunk ends here (every level at the last k-step) is ready
+        if (leader) {  // the level whose chunk ends here (every level at the last step) is ready
+          if (t == nks - 1) {
 #pragma unroll
-          for (int l = 0; l < LV; ++l)
-            if ((t + l) % C::CKS == C::CKS - 1 || t == nks - 1) mma_commit(ready_bar(buf(l)));
+            for (int l = 0; l < LV; ++l) mma_commit(ready_bar(buf(l)));
+          } else if (C::CKS - 1 - r < LV) {
+            mma_commit(ready_bar(buf(C::CKS - 1 - r)));
+          }
         }
         gate = __shfl_sync(0xffffffffu, max(gate, gate_ahead), 0);
+        ++t;
+        if (++r == C::CKS) {
+          r = 0;
+          if (++cm == C::NB) cm = 0;
+        }
       }
       if (!ok) break;
       if (leader) mma_commit(empty_bar(s));
       __syncwarp();
+      if (++s == C::STAGES) s = 0;
     }
   } else if (warp == OZ_GATE_WARP) {
-    // ---------------- gate: per k-step, wait (bounded) for its stage's operands (at the stage's
-    // first k-step) and, when a level starts a chunk there in a buffer used before, for that
-    // buffer's drain; then release the k-step to the MMA warp.  Level l's exact chunks are
-    // staggered by l k-steps (chunk k covers k-steps [k CKS - l, (k + 1) CKS - l)), so at most one
-    // level starts a chunk per k-step, and chunk k of level l accumulates in buffer (l + k) mod NB.
-    // That buffer last held chunk k - 1 of level l + 1, which ended two k-steps earlier: its drain
-    // has a full k-step of MMAs to finish.
+    // ---------------- gate: per step, wait (bounded) for its stage's operands (at the stage's
+    // first step) and, when a level starts a chunk there in a buffer used before, for that
+    // buffer's drain; then release the step to the MMA warp.  Level l's exact chunks are
+    // staggered by l steps (chunk k covers steps [k CKS - l, (k + 1) CKS - l)), so at most one
+    // level starts a chunk per step, and chunk k of level l accumulates in buffer (l + k) mod NB.
+    // That buffer last held chunk k - 1 of level l + 1, which ended two steps earlier: its drain
+    // has a full step of MMAs to finish.
     uint32_t used = 0, par = 0;  // per buffer: used before; parity of its uses so far
     const int nks = nk * C::KS;
     for (int t = 0; t < nks; ++t) {
@@ -648,13 +849,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_gemm_kernel(const __grid_con
 #pragma unroll
     for (int j = 0; j < (WIDE ? 16 : 1); ++j) hi[j] = 0;
     bool ok = true;
-    // drain events in the MMA issuer's order: at k-step t, the level whose staggered chunk ends
-    // there; at the last k-step, every level
+    // drain events in the MMA issuer's order: at step t, the level whose staggered chunk ends
+    // there; at the last step, every level
     uint32_t rpar = 0;  // per buffer: parity of its drains so far
     const int nks = nk * C::KS;
     for (int t = 0; t < nks && ok; ++t) {
       const bool final_step = t == nks - 1;
-      const int lone = (C::CKS - 1 - t % C::CKS);  // the level whose chunk ends at k-step t
+      const int lone = (C::CKS - 1 - t % C::CKS);  // the level whose chunk ends at step t
       for (int l = final_step ? 0 : lone; l < (final_step ? LV : min(lone + 1, LV)); ++l) {
         const int b = (l + (t + l) / C::CKS) % C::NB;
         const uint32_t ph = (rpar >> b) & 1u;
@@ -967,8 +1168,7 @@ kf_status launch_oz(cudaStream_t s, const OzSlices& A, const OzSlices& B, int M,
   a.M = M;
   a.N = N;
   a.nk = (int)ceil_div(K, BK);
-  // whole exact chunks per split, so chunk boundaries do not depend on the split
-  a.kt_per_split = (int)(ceil_div(ceil_div(K, OZ_KC), splits) * C::CK);
+  a.kt_per_split = (int)(ceil_div(ceil_div(K, OZ_SPLIT_K), splits) * (OZ_SPLIT_K / BK));
   a.partials = splits > 1 && !sums ? partials : nullptr;
   a.sums = sums;
   a.ld_sums = round_up(N, OZ_BN);
@@ -1007,6 +1207,30 @@ kf_status launch_oz(cudaStream_t s, const OzSlices& A, const OzSlices& B, int M,
   return KF_OK;
 }
 
+// One warp per row up to 512 columns (a block's threads would mostly idle), a block per row with the row in
+// registers up to 10240, two passes beyond.
+template <typename T>
+void slice_rows(cudaStream_t s, const T* X, int64_t ld, int64_t rows, int64_t cols, int S, const OzSlices& out) {
+  const unsigned blocks = (unsigned)out.rows_pad;
+#define OZ_SLICE(G, NCH) \
+  oz_slice_kernel<T, G, NCH><<<blocks * G / 256, 256, 0, s>>>(X, ld, rows, cols, S, out.planes, out.rows_pad, out.ldk, out.exps)
+  if (out.ldk <= 256)
+    OZ_SLICE(32, 1);
+  else if (out.ldk <= 512)
+    OZ_SLICE(32, 2);
+  else if (out.ldk <= 2048)
+    OZ_SLICE(256, 1);
+  else if (out.ldk <= 4096)
+    OZ_SLICE(256, 2);
+  else if (out.ldk <= 6144)
+    OZ_SLICE(256, 3);
+  else if (out.ldk <= 10240)
+    OZ_SLICE(256, 5);
+  else
+    OZ_SLICE(256, 0);
+#undef OZ_SLICE
+}
+
 }  // namespace
 
 thread_local TcLaunchTimer* g_oz_timer = nullptr;
@@ -1015,7 +1239,7 @@ thread_local TcLaunchTimer* g_oz_timer = nullptr;
 // 26 tiles; 74 us as one pass over K, 25 us in five splits and 7 us for their sum).  At least two chunks per
 // split: its fixed part (pipeline fill, drain, epilogue, the sum) is worth about three.
 int64_t oz_sums_splits(int64_t M, int64_t N, int64_t K) {
-  const int64_t tiles = ceil_div(M, OZ_BM) * ceil_div(N, OZ_BN), chunks = ceil_div(K, OZ_KC);
+  const int64_t tiles = ceil_div(M, OZ_BM) * ceil_div(N, OZ_BN), chunks = ceil_div(K, OZ_SPLIT_K);
   if (tiles >= 152 || chunks < 4) return 1;
   const int64_t s = std::min<int64_t>(std::min<int64_t>(152 / tiles, chunks / 2), 16);
   if (s < 2) return 1;
@@ -1043,13 +1267,37 @@ kf_status oz_slice(cudaStream_t s, const void* X, int64_t ld, int f64, int64_t r
   out.rows = rows;
   out.filled = S;
   if (f64)
-    oz_slice_kernel<double><<<(unsigned)out.rows_pad, 256, 0, s>>>(static_cast<const double*>(X), ld, rows, cols, S,
-                                                                   out.planes, out.rows_pad, out.ldk, out.exps);
+    slice_rows<double>(s, static_cast<const double*>(X), ld, rows, cols, S, out);
   else
-    oz_slice_kernel<float><<<(unsigned)out.rows_pad, 256, 0, s>>>(static_cast<const float*>(X), ld, rows, cols, S,
-                                                                  out.planes, out.rows_pad, out.ldk, out.exps);
+    slice_rows<float>(s, static_cast<const float*>(X), ld, rows, cols, S, out);
   note_launch();
   return launch_check("oz_slice");
+}
+
+kf_status oz_slice_symmetric(cudaStream_t s, float* X, int64_t ld, int64_t n, OzSlices& out) {
+  if (n < 1 || out.S < 3 || n > out.rows_pad || n > out.ldk || ld < n || ld % 4 || (reinterpret_cast<uintptr_t>(X) & 15))
+    return KF_ERR_ARG;
+  out.rows = n;
+  out.filled = 3;
+  oz_exps_kernel<<<(unsigned)out.rows_pad, 256, 0, s>>>(X, ld, n, out.exps);
+  note_launch();
+  KF_TRY(launch_check("oz_exps"));
+  oz_slice_symmetric_kernel<<<(unsigned)out.rows_pad, 256, 0, s>>>(X, ld, n, out.planes, out.rows_pad, out.ldk, out.exps);
+  note_launch();
+  return launch_check("oz_slice_symmetric");
+}
+
+kf_status oz_slice_correction(cudaStream_t s, const float* C, const float* Y, int64_t ld, int64_t n, double* X,
+                              int64_t ldx, OzSlices& out) {
+  if (n < 1 || out.S < 2 || n > out.rows_pad || n > out.ldk || ld < n || ldx < n || ld % 4 ||
+      (reinterpret_cast<uintptr_t>(C) & 15) || (reinterpret_cast<uintptr_t>(Y) & 15))
+    return KF_ERR_ARG;
+  out.rows = n;
+  out.filled = 2;
+  oz_slice_correction_kernel<<<(unsigned)out.rows_pad, 256, 0, s>>>(C, Y, ld, n, out.planes, out.rows_pad, out.ldk,
+                                                                    out.exps, X, ldx);
+  note_launch();
+  return launch_check("oz_slice_correction");
 }
 
 kf_status oz_gemm(cudaStream_t s, const OzSlices& A, const OzSlices& B, int M, int N, int K, int levels,
@@ -1070,8 +1318,8 @@ kf_status oz_gemm(cudaStream_t s, const OzSlices& A, const OzSlices& B, int M, i
       sums = work.p;
     }
   }
-  // whole exact chunks per split, every split non-empty
-  const int64_t chunks = ceil_div(K, OZ_KC);
+  // whole multiples of OZ_SPLIT_K per split, every split non-empty
+  const int64_t chunks = ceil_div(K, OZ_SPLIT_K);
   splits = (int)std::min<int64_t>(splits, chunks);
   splits = (int)ceil_div(chunks, ceil_div(chunks, splits));
   // the sums of all levels fit 64 bits up to K 2^(8 LV + 6.1) < 2^62
@@ -1083,6 +1331,10 @@ kf_status oz_gemm(cudaStream_t s, const OzSlices& A, const OzSlices& B, int M, i
                          : launch_oz<5, 5, true, kOzBK>(s, A, B, M, N, K, e, splits, partials, sums);
     case 6 * 16 + 6: return launch_oz<6, 6, true, kOzBK>(s, A, B, M, N, K, e, splits, partials, sums);
     case 7 * 16 + 7: return launch_oz<7, 7, true, kOzBK>(s, A, B, M, N, K, e, splits, partials, sums);
+    case 7 * 16 + 3: return launch_oz<7, 3, true, kOzBK>(s, A, B, M, N, K, e, splits, partials, sums);
+    case 5 * 16 + 2:
+      return narrow_sums ? launch_oz<5, 2, false, kOzBK>(s, A, B, M, N, K, e, splits, partials, sums)
+                         : launch_oz<5, 2, true, kOzBK>(s, A, B, M, N, K, e, splits, partials, sums);
   }
   return KF_ERR_ARG;
 }

@@ -46,6 +46,16 @@ void oz_slice_layout(OzSlices& out, void* mem, int64_t rows, int64_t cols, int S
 kf_status oz_slice(cudaStream_t s, const void* X, int64_t ld, int f64, int64_t rows, int64_t cols, int S,
                    OzSlices& out);
 
+// A symmetric n x n float32 X (16-byte aligned, ld a multiple of 4) rounded in place so that it stays
+// symmetric and three slices by rows hold it exactly (each element to 2^-24 of the larger of its two row
+// maxima), and those slices.
+kf_status oz_slice_symmetric(cudaStream_t s, float* X, int64_t ld, int64_t n, OzSlices& out);
+
+// Two slices Cs (2^-16 of the row maxima) of a float32 C, and X = Y + Cs in float64 (Y float32, both n x n with
+// leading dimension ld as above).
+kf_status oz_slice_correction(cudaStream_t s, const float* C, const float* Y, int64_t ld, int64_t n, double* X,
+                              int64_t ldx, OzSlices& out);
+
 // Epilogue of the exact-slice product, float64.  With acc = (A B^T)[i][j]:
 //   v = alpha acc + beta cin[i][j] + (i == j ? delta : 0) + Radd[i][j]
 //   out[i][j] = v,  outf[i][j] = (float) v,  outT[j][i] = v,

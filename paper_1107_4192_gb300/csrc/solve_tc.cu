@@ -197,10 +197,13 @@ kf_status refine_inverse_tc(cudaStream_t s, TcScratch& sc, int n, const void* P,
                             int64_t ldj, double* X2, int64_t ldx, int* status, int step) {
   if (gain_q && q_kind != 0 && q_kind != 1) return KF_ERR_ARG;
   const int64_t ld = rb.ld;
+  float* Y = reinterpret_cast<float*>(rb.X0);  // X_0, then its rounding Y_0
+  float* C = Y + n * ld;
+  double *E = rb.R, *X1 = rb.X1;
   {
-    GemmParams<double> g;  // X0 = W^T W (lower triangle + mirror; row r of W^T is zero for k < r)
+    GemmParams<float> g;  // X_0 = W^T W (lower triangle + mirror; row r of W^T is zero for k < r)
     g.M = n; g.N = n; g.K = n;
-    g.out = rb.X0; g.ldo = ld;
+    g.out = Y; g.ldo = ld;
     g.sym = 1;
     g.tri_a = -1;
     g.tri_b = -1;
@@ -208,41 +211,51 @@ kf_status refine_inverse_tc(cudaStream_t s, TcScratch& sc, int n, const void* P,
     KF_TRY(tc_gemm_ops(s, sc, TcOperand{W, ldw, 0, 1}, TcOperand{W, ldw, 0, 1}, g, 3));
   }
   KF_TRY(oz_slice(s, P, ldp, p_f64, n, n, 7, rb.Ps));
-  const double* X = rb.X0;
-  for (int k = 0; k < 2; ++k) {
-    // R_k = I - P X_k  (X_k symmetric: its rows are the product's columns)
-    KF_TRY(oz_slice(s, X, ld, 1, n, n, k == 0 ? 5 : 7, rb.Xs));
-    OzEpilogue e;
+  KF_TRY(oz_slice_symmetric(s, Y, ld, n, rb.Xs));
+  {
+    OzEpilogue e;  // E_0 = I - Y_0 P (P symmetric: its rows are the product's columns)
     e.alpha = -1.0;
     e.delta = 1.0;
-    e.out = rb.R;
-    e.ldo = ld;
+    e.out = E; e.ldo = ld;
     e.status = status;
     e.step = step;
-    KF_TRY(oz_gemm(s, rb.Ps, rb.Xs, n, n, n, k == 0 ? 5 : 7, e));
-    // X_{k+1} = X_k + X_k R_k;  C = op(A) op(B)^T with op(B) = R_k^T (R_k stored K x N)
-    GemmParams<double> g;
+    KF_TRY(oz_gemm(s, rb.Xs, rb.Ps, n, n, n, 7, e, 1, nullptr, OzSums{}, 3));
+  }
+  {
+    GemmParams<float> g;  // C = E_0 Y_0, symmetric
     g.M = n; g.N = n; g.K = n;
-    g.cin = X; g.ldcin = ld; g.beta = 1.0;
+    g.out = C; g.ldo = ld;
     g.sym = 1;
     g.status = status;
     g.step = step;
-    if (k == 0) {
-      g.out = rb.X1; g.ldo = ld;
-      KF_TRY(tc_gemm_ops(s, sc, TcOperand{X, ld, 1, 0}, TcOperand{rb.R, ld, 1, 1}, g, 3));
-      X = rb.X1;
-    } else if (gain_q) {
-      // the correction is ~1e-9 of X: two bf16 slices (16 bits) leave it accurate to ~1e-14 of X
-      g.gain_q = gain_q; g.gain_q_kind = q_kind;
-      g.out = J64; g.ldo = ldj;
-      g.outf = Jf; g.ldof = ldj;
-      KF_TRY(tc_gemm_ops(s, sc, TcOperand{X, ld, 1, 0}, TcOperand{rb.R, ld, 1, 1}, g, 2));
-    } else {
-      g.out = X2; g.ldo = ldx;
-      KF_TRY(tc_gemm_ops(s, sc, TcOperand{X, ld, 1, 0}, TcOperand{rb.R, ld, 1, 1}, g, 2));
-    }
+    KF_TRY(tc_gemm_ops(s, sc, TcOperand{E, ld, 1, 0}, TcOperand{Y, ld, 0, 0}, g, 2));
   }
-  return KF_OK;
+  KF_TRY(oz_slice_correction(s, C, Y, ld, n, X1, ld, rb.Xs));
+  {
+    OzEpilogue e;  // E_1 = I - X_1 P = E_0 - C_s P
+    e.alpha = -1.0;
+    e.cin = E; e.ldcin = ld; e.beta = 1.0;
+    e.out = E; e.ldo = ld;
+    e.status = status;
+    e.step = step;
+    KF_TRY(oz_gemm(s, rb.Xs, rb.Ps, n, n, n, 5, e, 1, nullptr, OzSums{}, 2));
+  }
+  // X_2 = X_1 + E_1 X_1: the correction is ~1e-9 of X, so two bf16 slices (16 bits) leave it accurate to
+  // ~1e-14 of X, and the asymmetry of X_1 (~1e-10) does not matter in it
+  GemmParams<double> g;
+  g.M = n; g.N = n; g.K = n;
+  g.cin = X1; g.ldcin = ld; g.beta = 1.0;
+  g.sym = 1;
+  g.status = status;
+  g.step = step;
+  if (gain_q) {
+    g.gain_q = gain_q; g.gain_q_kind = q_kind;
+    g.out = J64; g.ldo = ldj;
+    g.outf = Jf; g.ldof = ldj;
+  } else {
+    g.out = X2; g.ldo = ldx;
+  }
+  return tc_gemm_ops(s, sc, TcOperand{E, ld, 1, 0}, TcOperand{X1, ld, 1, 0}, g, 2);
 }
 
 }  // namespace kfm

@@ -24,8 +24,8 @@ kf_status gain_from_inverse_tc(cudaStream_t s, TcScratch& sc, int n, const float
 kf_status gain_identity_tc(cudaStream_t s, TcScratch& sc, int n, const float* W, int64_t ldw, int q_kind,
                            const double* q, float* J, int64_t ldj, int* status);
 
-// Buffers of refine_inverse_tc: three n x ld float64 matrices and the slices
-// of P (7 slices) and of the iterate (7 slices).
+// Buffers of refine_inverse_tc: three n x ld float64 matrices (the first holds the float32 Y_0 and C) and the
+// slices of P (7) and of the iterate (3, then 2; room for 7).
 struct RefineBufs {
   double *X0 = nullptr, *R = nullptr, *X1 = nullptr;
   int64_t ld = 0;
@@ -35,16 +35,19 @@ uint64_t refine_bytes(int64_t n, int64_t ld);
 void refine_layout(RefineBufs& rb, void* mem, int64_t n, int64_t ld);
 
 // Inverse of the symmetric positive definite P (float32, or float64 when p_f64; n x n) to float64
-// accuracy, from W = L^{-1} of its float32-class factor (chol_inverse_tc):
-//   X0 = W^T W;   R_k = I - P X_k;   X_{k+1} = X_k + X_k R_k   (k = 0, 1)
-// (Newton's iteration for the inverse, quadratically convergent from the
-// float32-class X0).  The residuals are exact-slice products (5 slice levels
-// for R_0, 7 for R_1), the corrections split-bf16 products with float64
-// epilogues (X_k R_k is symmetric: lower triangle + mirror).  The last
-// correction is fused into its consumer:
+// accuracy, from W = L^{-1} of its float32-class factor (chol_inverse_tc): Newton's iteration, each residual
+// I - X_k P exact to 2^-51 of the row maxima,
+//   Y_0 = W^T W rounded to 24 bits below its row maxima;   E_0 = I - Y_0 P;
+//   X_1 = Y_0 + C_s, C_s = E_0 Y_0 rounded to 16 bits;     E_1 = I - X_1 P = E_0 - C_s P;
+//   X_2 = X_1 + E_1 X_1.
+// The iterates are rounded so that few slices hold them exactly, and the second residual updates the
+// first: 18 slice products (3 slices of Y_0 against 7 of P, levels below 7) and 9 (2 of C_s against 5,
+// levels below 5), where separate residuals of unrounded iterates took 15 + 28 (N = 8196: 19.6 + 27.9 ms;
+// now 15.8 + 9.4 ms).  The corrections are split-bf16 products (symmetric: lower triangle + mirror).
+// The last correction is fused into its consumer:
 //  - gain_q != NULL (F = I, Q = q I or diagonal): J = I - Q X_2 into J64
 //    (float64) and Jf (float32), X_2 itself never stored;
-//  - gain_q == NULL: X_2 into X2 (float64, n x ldx).
+//  - gain_q == NULL: X_2 into X2 (float64, n x ldx; may be rb.X0).
 kf_status refine_inverse_tc(cudaStream_t s, TcScratch& sc, int n, const void* P, int p_f64, int64_t ldp, const float* W,
                             int64_t ldw, RefineBufs& rb, int q_kind, const double* gain_q, double* J64, float* Jf,
                             int64_t ldj, double* X2, int64_t ldx, int* status, int step);

@@ -254,3 +254,44 @@ def test_filter_products_split_over_k(N, m):
     ref = run_oracle(prob)
     assert rel_err_elementwise(out["diagP_filt"], diag_of(ref["P_filt"])) <= 2.0 ** -35 * N
     assert rel_err_per_step(out["x_filt"], ref["x_filt"]) <= 1e-4
+
+
+@pytest.mark.parametrize("f32", [False, True])
+@pytest.mark.parametrize("K", [8, 250, 257, 500, 513, 2049, 4100, 6145, 10240, 10241])
+def test_slicing_row_lengths(f32, K):
+    """Every way a row is held while it is sliced (a warp or a block per row, one to five parts, two passes),
+    at the edges of their lengths, with an operand whose leading dimension breaks the 16-byte alignment."""
+    rng = np.random.default_rng(K)
+    M, N, lda = 9, 3, K + 1
+    A = np.zeros((M, lda))
+    A[:, :K] = rng.standard_normal((M, K)) * np.exp(rng.uniform(-30, 30, (M, 1)))
+    A[2] = 0.0
+    A[3, 1:] = 0.0
+    Bm = rng.standard_normal((N, K))
+    if f32:
+        A = A.astype(np.float32)
+    dA = torch.from_numpy(A).cuda()
+    C = torch.zeros(M, N, dtype=torch.float64, device="cuda")
+    B.kfx_gemm_exact(6, M, N, K, 1.0, dA, lda, torch.from_numpy(Bm).cuda(), K, 0.0, 0.0, C, N)
+    ref, ea, eb = exact_sliced_product(A[:, :K].astype(np.float64), Bm, 6)
+    assert np.array_equal(C.cpu().numpy(), ref)  # digits, sums and one rounding are exact
+    A[4, K // 2] = np.inf
+    A[5, K - 1] = np.nan
+    C.zero_()
+    B.kfx_gemm_exact(6, M, N, K, 1.0, torch.from_numpy(A).cuda(), lda, torch.from_numpy(Bm).cuda(), K, 0.0, 0.0, C, N)
+    got = C.cpu().numpy()
+    bad = np.isin(np.arange(M), [4, 5])
+    assert np.all(np.isnan(got[bad])) and np.array_equal(got[~bad], ref[~bad])
+
+
+@pytest.mark.parametrize("n", [1, 2, 63, 129, 200, 385])
+def test_refined_inverse_ragged_sizes(n):
+    """The Newton steps on rounded iterates at ragged sizes, against numpy in float64: no worse than the
+    conditioning times float64 rounding (cond 100; the bound of the larger sizes' test)."""
+    A = spd32(n, 100.0 if n > 1 else 1.0, n)
+    X = torch.zeros(n, n, dtype=torch.float64, device="cuda")
+    st, fi = B.kfx_spd_inverse(2, n, torch.from_numpy(A).cuda(), n, X, n)
+    assert st == 0 and fi == -1
+    ref = np.linalg.inv(A.astype(np.float64))
+    assert np.linalg.norm(X.cpu().numpy() - ref) <= 1e-12 * np.linalg.norm(ref)
+    assert torch.equal(X, X.T)
