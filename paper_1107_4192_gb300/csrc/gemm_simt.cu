@@ -19,10 +19,12 @@ template <> struct SimtCfg<double> {
 template <> struct SimtCfg<float> {
   static constexpr int BM = 128, BN = 128, BK = 8, TM = 8, TN = 8, PAD = 4;
 };
-// float64 products too small to fill the GPU with 64 x 64 tiles (the m x m
-// innovation factorisation, its panels): the float64 pipe does about two
-// multiply-adds per clock per SM, so such a product is bound by how many SMs
-// it reaches.  16 x 16 tiles, one output per thread, same summation order.
+// float64 products that do not fill the GPU evenly with 64 x 64 tiles: the float64 pipe does about 1.7
+// multiply-adds per clock and SM whatever the tile, so such a product is bound by the SM with the most
+// tiles.  32 x 32 and 16 x 16 tiles, four and one outputs per thread, same summation order.
+struct SimtCfgMid64 {
+  static constexpr int BM = 32, BN = 32, BK = 16, TM = 2, TN = 2, PAD = 1;
+};
 struct SimtCfgSmall64 {
   static constexpr int BM = 16, BN = 16, BK = 16, TM = 1, TN = 1, PAD = 1;
 };
@@ -64,7 +66,13 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(GemmParams<T> p) {
 #pragma unroll
     for (int j = 0; j < TN; ++j) acc[i][j] = T(0);
 
-  for (int k0 = 0; k0 < p.K; k0 += BK) {
+  // k-range of this tile: triangular operands are zero outside their band
+  int k_lo = 0, k_hi = p.K;
+  if (p.tri_a > 0) k_hi = min(k_hi, m0 + BM);
+  if (p.tri_a < 0) k_lo = max(k_lo, m0);
+  if (p.tri_b > 0) k_hi = min(k_hi, n0 + BN);
+  if (p.tri_b < 0) k_lo = max(k_lo, n0);
+  for (int k0 = k_lo / BK * BK; k0 < k_hi; k0 += BK) {
     // A tile: BM x BK, stored transposed As[kk][row]
 #pragma unroll
     for (int l = 0; l < (BM * BK) / 256; ++l) {
@@ -174,15 +182,35 @@ kf_status gemm_simt(cudaStream_t s, bool transB, const GemmParams<T>& p) {
       if (outs[k] && (!apart(outs[k], es[k], lds[k], p.M, p.N, p.A, sizeof(T), p.lda, p.M, p.K) ||
                       !apart(outs[k], es[k], lds[k], p.M, p.N, p.B, sizeof(T), p.ldb, rB, cB)))
         separate = false;
-    if (separate && (int64_t)grid.x * grid.y < 2 * 152) {
-      const dim3 g2 = grid_for(SimtCfgSmall64::BM, SimtCfgSmall64::BN);
-      if (g2.y <= 65535) {
-        if (transB)
-          gemm_simt_kernel<T, true, SimtCfgSmall64><<<g2, 256, 0, s>>>(p);
-        else
-          gemm_simt_kernel<T, false, SimtCfgSmall64><<<g2, 256, 0, s>>>(p);
-        note_launch();
-        return launch_check("gemm_simt");
+    if (separate) {
+      // The largest tile whose fullest SM has at most 10% more work than with the best tile: small products
+      // are bound by the SM with the most tiles (n = 384: 64 x 64 0.42 ms, 32 x 32 and 16 x 16 0.12 ms; n = 1026:
+      // 2.13, 2.11 and 1.87 ms), large ones by the float64 units in any tile (n = 2048: 14.4, 13.9, 13.9 ms), where
+      // the larger tile reads less.
+      auto fullest = [&](int bm, int bn) {
+        const dim3 g = grid_for(bm, bn);
+        return ceil_div((int64_t)g.x * g.y, 152) * bm * bn;
+      };
+      const int64_t w64 = fullest(64, 64), w32 = fullest(32, 32), w16 = fullest(16, 16);
+      const int64_t best = std::min(std::min(w64, w32), w16);
+      if (w64 * 10 > best * 11) {
+        const bool mid = w32 * 10 <= best * 11;
+        const dim3 g2 = mid ? grid_for(32, 32) : grid_for(16, 16);
+        if (g2.y <= 65535) {
+          if (mid) {
+            if (transB)
+              gemm_simt_kernel<T, true, SimtCfgMid64><<<g2, 256, 0, s>>>(p);
+            else
+              gemm_simt_kernel<T, false, SimtCfgMid64><<<g2, 256, 0, s>>>(p);
+          } else {
+            if (transB)
+              gemm_simt_kernel<T, true, SimtCfgSmall64><<<g2, 256, 0, s>>>(p);
+            else
+              gemm_simt_kernel<T, false, SimtCfgSmall64><<<g2, 256, 0, s>>>(p);
+          }
+          note_launch();
+          return launch_check("gemm_simt");
+        }
       }
     }
   }

@@ -1,5 +1,6 @@
 // Cholesky factor of the innovation covariance (eqn 8), its inverse and the solve of the innovation
-// vector, S = L L^T, L^{-1} and L^{-1} nu, float64, in one launch.
+// vector, S = L L^T, L^{-1} and L^{-1} nu, float64, in one launch.  The float64 path factors and inverts
+// P_{t+1|t} (eqn 11) with it too, up to kInnovFactorMaxM sources.
 //
 // What bounds it: one warp's float64 instruction occupies its SM sub-partition for 64 cycles whatever
 // the number of active lanes (measured; 19 cycles per instruction and SM when all four are busy), so
@@ -29,7 +30,6 @@ namespace {
 
 constexpr int kRowsPerCta = 4;      // row tasks: one warp per SM sub-partition
 constexpr int kIfThreads = 256;     // diagonal tiles use seven warps, the other tasks four
-constexpr int kMaxM = kInnovFactorMaxM;
 constexpr uint64_t kIfWaitNs = WAIT_NS;
 
 struct IfArgs {
@@ -37,11 +37,11 @@ struct IfArgs {
   double* S;
   int64_t lds;
   double* dinv;   // T blocks of 32 x 32: inverses of the diagonal blocks
-  double* Linv;   // m x m, or null
+  double* Linv;   // m x m (row stride m), or null
   double* nu;     // m, or null
   double* W;      // L and the updated diagonal tiles, row stride 32 T
   double* Dt;     // the same, pairs of columns interleaved: D[c][kk] at ((kk / 2) 32 + c) 2 + kk mod 2
-  int* flags;     // ticket, done, diag ready [T], diag rows updated [T], panel rows done [T x T]
+  int* flags;     // ticket, done, diag ready [T], diag rows updated [T], panel rows done [T x T bytes]
   int* status;
   int step;
 };
@@ -52,13 +52,8 @@ struct DiagTile {
   double q[32];       // 1 / L_jj
   int fail;
 };
-struct RowTile {
-  double row[kRowsPerCta][kMaxM + 32];
-};
-struct InvRow {
-  double B[kMaxM + 32];
-  int ready[kMaxM / 32 + 1];  // X_k (in B) is final
-};
+// The other tasks' shared memory: a row CTA holds kRowsPerCta rows of 32 T values; a row of L^{-1} its 32 T
+// values X (as they become final) and T ready flags.
 
 __device__ __forceinline__ int ld_acquire(const int* p) {
   int v;
@@ -76,14 +71,21 @@ __device__ __forceinline__ double2 ld2(const double2* p) {
   return v;
 }
 
-// One warp waits until *flag >= want; false when the wait expired or another task failed.
-__device__ __forceinline__ bool wait_flag(const int* flag, int want, const IfArgs& a, int lane, int sleep_ns) {
+// Rows of tile i whose panel k is done: one byte, four tiles per word.
+__device__ __forceinline__ int* rows_word(const IfArgs& a, int k, int i) {
+  return a.flags + 2 + 2 * a.T + k * ((a.T + 3) / 4) + i / 4;
+}
+
+// One warp waits until the count in *flag (its byte at `shift` with mask 0xff, or the whole word) is at least
+// want; false when the wait expired or another task failed.
+__device__ __forceinline__ bool wait_flag(const int* flag, int want, const IfArgs& a, int lane, int sleep_ns,
+                                          int shift = 0, int mask = -1) {
   int ok = 1;
   if (lane == 0) {
-    if (ld_acquire(flag) < want) {
+    if (((ld_acquire(flag) >> shift) & mask) < want) {
       const uint64_t t0 = globaltimer();
       for (int n = 1;; ++n) {
-        if (ld_acquire(flag) >= want) break;
+        if (((ld_acquire(flag) >> shift) & mask) >= want) break;
         if ((n & 15) == 0) {
           if (status_failed(a.status)) { ok = 0; break; }
           if (globaltimer() - t0 > kIfWaitNs) {
@@ -257,8 +259,8 @@ __device__ void factor_tile(DiagTile& s, const IfArgs& a, int tile, int warp, in
 
 // Wait of a row CTA's four warps: warp 0 polls for all (one poll per warp slowed the data down).
 __device__ __forceinline__ bool wait_flag_rows(const int* flag, int want, const IfArgs& a, volatile int* failed, int warp,
-                                               int lane, int sleep_ns) {
-  if (warp == 0 && !wait_flag(flag, want, a, lane, sleep_ns)) *failed = 1;
+                                               int lane, int sleep_ns, int shift = 0, int mask = -1) {
+  if (warp == 0 && !wait_flag(flag, want, a, lane, sleep_ns, shift, mask)) *failed = 1;
   bar_sync(6, 32 * kRowsPerCta);
   return *failed == 0;
 }
@@ -272,7 +274,6 @@ __device__ void row_task(double* row, const IfArgs& a, volatile int* failed, boo
   const int ncols = live ? (is_nu ? a.m : min(a.m, 32 * (tr + 1))) : 0;
   const int last = is_nu ? a.T - 1 : tr;  // last column tile of the row
   const int* diag_ready = a.flags + 2;
-  int* rows_done = a.flags + 2 + 2 * a.T;
   int bad = -1;
   for (int j = lane; j < 32 * (last + 1); j += 32) {
     const double v = j < ncols ? (is_nu ? a.nu[j] : a.S[(int64_t)r * a.lds + j]) : 0.0;
@@ -298,13 +299,13 @@ __device__ void row_task(double* row, const IfArgs& a, volatile int* failed, boo
       if (!is_nu) {
         a.W[(int64_t)r * ldw + 32 * k + lane] = acc;
         __syncwarp();
-        if (lane == 0) red_release(rows_done + k * a.T + tr, 1);
+        if (lane == 0) red_release(rows_word(a, k, tr), 1 << (8 * (tr & 3)));
         a.S[(int64_t)r * a.lds + 32 * k + lane] = acc;
       }
       __syncwarp();
     }
     for (int i = k + 1; i <= last; ++i) {
-      if (!wait_flag_rows(rows_done + k * a.T + i, min(32, a.m - 32 * i), a, failed, warp, lane, 0)) return;
+      if (!wait_flag_rows(rows_word(a, k, i), min(32, a.m - 32 * i), a, failed, warp, lane, 0, 8 * (i & 3), 0xff)) return;
       if (!live) continue;
       const int c = 32 * i + lane;
       // rows of L beyond m do not exist: those lanes read the tile's first row and drop the result
@@ -337,11 +338,11 @@ __device__ void row_task(double* row, const IfArgs& a, volatile int* failed, boo
 // Row r of L^{-1}, four warps: X_k for the row's tiles k = tr .. 0 with
 // X_j = (0 - X_tr L[tr, j] - .. - X_{j+1} L[j+1, j]) L_jj^{-1}; warp w owns the tiles j = w mod 4 and
 // applies the X_k that are ready while it waits for the last one.
-__device__ void inverse_row(InvRow& s, const IfArgs& a, int r, int warp, int lane) {
+__device__ void inverse_row(double* B, int* ready_flags, const IfArgs& a, int r, int warp, int lane) {
   const int tr = r / 32, ldw = 32 * a.T;
   if (!wait_flag(a.flags + 2 + tr, 2, a, lane, 100)) return;
   double* out = a.Linv + (int64_t)r * a.m;
-  volatile int* ready = s.ready;
+  volatile int* ready = ready_flags;
   for (int j = tr - 1 - ((tr - 1 - warp) & 3); j >= 0; j -= 4) {
     const double* D = a.dinv + (int64_t)j * 1024 + lane;
     double b = 0.0;
@@ -371,7 +372,7 @@ __device__ void inverse_row(InvRow& s, const IfArgs& a, int r, int warp, int lan
         }
         if (!__shfl_sync(0xffffffffu, ok, 0)) return;
         __threadfence_block();
-        X = s.B + 32 * k;
+        X = B + 32 * k;
       }
       double acc = 0.0;
 #pragma unroll
@@ -379,13 +380,13 @@ __device__ void inverse_row(InvRow& s, const IfArgs& a, int r, int warp, int lan
         if (kk < nk) acc = __fma_rn(X[kk], lv[kk], acc);
       b = __dsub_rn(b, acc);
     }
-    s.B[32 * j + lane] = b;
+    B[32 * j + lane] = b;
     __syncwarp();
     double acc = 0.0;
 #pragma unroll
-    for (int kk = 0; kk < 32; ++kk) acc = __fma_rn(s.B[32 * j + kk], dv[kk], acc);
+    for (int kk = 0; kk < 32; ++kk) acc = __fma_rn(B[32 * j + kk], dv[kk], acc);
     __syncwarp();
-    s.B[32 * j + lane] = acc;
+    B[32 * j + lane] = acc;
     __threadfence_block();
     __syncwarp();
     if (lane == 0) ready[j] = 1;
@@ -397,16 +398,14 @@ __device__ void inverse_row(InvRow& s, const IfArgs& a, int r, int warp, int lan
 }
 
 __global__ void __launch_bounds__(kIfThreads) innovation_factor_kernel(const IfArgs a) {
-  __shared__ union {
-    DiagTile d;
-    RowTile r;
-    InvRow v;
-  } sm;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double* rows = reinterpret_cast<double*>(smem_raw);
+  int* ready = reinterpret_cast<int*>(rows + 32 * a.T);
   __shared__ int ticket_s, failed_s;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   if (threadIdx.x == 0) ticket_s = status_failed(a.status) ? -1 - atomicAdd(a.flags, 1) : atomicAdd(a.flags, 1);
   if (threadIdx.x == 0) failed_s = 0;
-  if (threadIdx.x <= kMaxM / 32) sm.v.ready[threadIdx.x] = 0;
+  for (int e = threadIdx.x; e < a.T; e += kIfThreads) ready[e] = 0;
   __syncthreads();
   const int ticket = ticket_s;
   // tickets: per tile its row CTAs, then its diagonal tile; then the innovation; then the rows of L^{-1}
@@ -418,15 +417,15 @@ __global__ void __launch_bounds__(kIfThreads) innovation_factor_kernel(const IfA
       const int tile = min(ticket / full, a.T - 1), u = ticket - tile * full;
       const int units = tile == a.T - 1 ? last_units : full;
       if (u == units - 1) {
-        factor_tile(sm.d, a, tile, warp, lane);
+        factor_tile(*reinterpret_cast<DiagTile*>(smem_raw), a, tile, warp, lane);
       } else if (warp < kRowsPerCta) {
-        row_task(sm.r.row[warp], a, &failed_s, false, 32 * tile + kRowsPerCta * u + warp, warp, lane);
+        row_task(rows + warp * 32 * a.T, a, &failed_s, false, 32 * tile + kRowsPerCta * u + warp, warp, lane);
       }
     } else if (a.nu && ticket == nfac) {
-      if (warp < kRowsPerCta) row_task(sm.r.row[warp], a, &failed_s, true, a.m, warp, lane);
+      if (warp < kRowsPerCta) row_task(rows + warp * 32 * a.T, a, &failed_s, true, a.m, warp, lane);
     } else if (warp < 4) {
       const int r = ticket - nfac - (a.nu ? 1 : 0);
-      inverse_row(sm.v, a, r, warp, lane);
+      inverse_row(rows, ready, a, r, warp, lane);
     }
   }
   __syncthreads();
@@ -437,24 +436,21 @@ __global__ void __launch_bounds__(kIfThreads) innovation_factor_kernel(const IfA
   __syncthreads();
   if (ticket_s) {  // every other CTA has finished: clear the flags for the next launch
     __threadfence();
-    for (int e = threadIdx.x; e < 2 + 2 * a.T + a.T * a.T; e += kIfThreads) a.flags[e] = 0;
+    for (int e = threadIdx.x; e < 2 + 2 * a.T + a.T * ((a.T + 3) / 4); e += kIfThreads) a.flags[e] = 0;
   }
 }
 
 }  // namespace
 
-size_t innovation_factor_work(int64_t m) {
-  const int64_t T = ceil_div(m, 32);
-  return (size_t)(m * 32 * T + T * 1024);
-}
 size_t innovation_factor_flags(int64_t m) {
   const int64_t T = ceil_div(m, 32);
-  return (size_t)(2 + 2 * T + T * T);
+  return (size_t)(2 + 2 * T + T * ((T + 3) / 4));
 }
 
 kf_status innovation_factor(cudaStream_t s, int m, double* S, int64_t lds, double* dinv, double* Linv, double* nu,
-                            double* work, int* flags, int* status, int step) {
-  if (m < 1 || m > kInnovFactorMaxM || !S || !dinv || !work || !flags) return KF_ERR_ARG;
+                            double* W, double* Dt, int* flags, int* status, int step) {
+  if (m < 1 || m > kInnovFactorMaxM || !S || !dinv || !W || !Dt || !flags) return KF_ERR_ARG;
+  if ((reinterpret_cast<uintptr_t>(W) | reinterpret_cast<uintptr_t>(Dt)) & 15) return KF_ERR_ARG;
   IfArgs a;
   a.m = m;
   a.T = (int)ceil_div(m, 32);
@@ -463,15 +459,19 @@ kf_status innovation_factor(cudaStream_t s, int m, double* S, int64_t lds, doubl
   a.dinv = dinv;
   a.Linv = Linv;
   a.nu = nu;
-  a.W = work;
-  a.Dt = work + (int64_t)m * 32 * a.T;
+  a.W = W;
+  a.Dt = Dt;
   a.flags = flags;
   a.status = status;
   a.step = step;
   const int full = 32 / kRowsPerCta + 1;
   const int last_units = (int)ceil_div(m - 32 * (a.T - 1), kRowsPerCta) + 1;
   const int grid = full * (a.T - 1) + last_units + (nu ? 1 : 0) + (Linv ? m : 0);
-  innovation_factor_kernel<<<grid, kIfThreads, 0, s>>>(a);
+  const size_t smem = std::max(sizeof(DiagTile), (size_t)kRowsPerCta * 32 * a.T * sizeof(double));
+  static_assert(kRowsPerCta >= 2, "a row of the inverse and its flags fit");
+  KF_CUDA_TRY(smem_limit_per_device((const void*)innovation_factor_kernel,
+                                    kRowsPerCta * (kInnovFactorMaxM + 32) * (int)sizeof(double)));
+  innovation_factor_kernel<<<grid, kIfThreads, smem, s>>>(a);
   note_launch();
   return launch_check("innovation_factor");
 }

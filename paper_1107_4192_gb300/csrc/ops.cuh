@@ -47,7 +47,7 @@ struct GemmParams {
   // Tensor-core path only: transA = 1 means A is stored K x M (row-major) and
   // is used transposed.  tri_a / tri_b: +1 when row r of the operand as used
   // (A: M x K, op(B): N x K) is zero for k > r, -1 when zero for k < r, so
-  // k-tiles outside the band are skipped; 0 = dense.
+  // k-tiles outside the band are skipped; 0 = dense (every kernel).
   int transA = 0;
   int tri_a = 0, tri_b = 0;
   // Smoother gain from an inverse (J = I - Q P^{-1}, F = I): when gain_q is
@@ -96,17 +96,16 @@ kf_status trsm_right(cudaStream_t s, bool trans, int M, int n, const T* L, int64
                      const T* dinv, int nb, T* B, int64_t ldb, int* status);
 
 // S = L L^T for the m x m innovation covariance (lower triangle, in place), the inverses of its 32 x 32
-// diagonal blocks (dinv: ceil(m / 32) blocks of 1024), L^{-1} (m x m with zeros above the diagonal, when
-// not null) and nu <- L^{-1} nu (when not null), float64, one launch; bit for bit what potrf and
-// trsm_right give with 32-wide blocks.  m <= kInnovFactorMaxM.  work: innovation_factor_work(m)
-// doubles (16-byte aligned); flags: innovation_factor_flags(m) ints, zero before the first launch (every
-// launch leaves them zero), both used by one stream at a time.  A bad pivot sets KF_ERR_NOT_PD
-// (step, pivot), a non-finite nu KF_ERR_NUMERIC (after the factor).
-constexpr int kInnovFactorMaxM = 960;
-size_t innovation_factor_work(int64_t m);
+// diagonal blocks (dinv: ceil(m / 32) blocks of 1024), L^{-1} (m x m, row stride m, zeros above the diagonal;
+// when not null) and nu <- L^{-1} nu (when not null), float64, one launch; bit for bit what potrf and
+// trsm_right give with 32-wide blocks.  m <= kInnovFactorMaxM.  Work space, 16-byte aligned: W of
+// m * round_up(m, 32) and Dt of 32 * round_up(m, 32) doubles; flags: innovation_factor_flags(m) ints,
+// zero before the first launch (every launch leaves them zero); all used by one stream at a time.  A bad
+// pivot sets KF_ERR_NOT_PD (step, pivot), a non-finite nu KF_ERR_NUMERIC (after the factor).
+constexpr int kInnovFactorMaxM = 1536;
 size_t innovation_factor_flags(int64_t m);
 kf_status innovation_factor(cudaStream_t s, int m, double* S, int64_t lds, double* dinv, double* Linv, double* nu,
-                            double* work, int* flags, int* status, int step);
+                            double* W, double* Dt, int* flags, int* status, int step);
 
 // ---------------------------------------------------------------- small ops
 

@@ -65,7 +65,7 @@ struct kf_plan_s {
   char *P = nullptr, *Ut = nullptr, *Zb = nullptr, *KV = nullptr, *VK = nullptr, *Hb = nullptr, *tmpN = nullptr;
   char *Fb = nullptr, *S0b = nullptr;
   double *S = nullptr, *S0 = nullptr, *Sdinv = nullptr, *partials = nullptr;
-  int* Sflags = nullptr;  // task flags of innovation_factor
+  int *Sflags = nullptr, *Lflags = nullptr;  // task flags of innovation_factor for S and for P_{t+1|t}
   char *Sl = nullptr, *Sldinv = nullptr;
   char *Lb = nullptr, *Ldinv = nullptr, *Jb = nullptr;
   float* Wi = nullptr;    // L^{-1} for the tensor-core solve (mixed mode, float32 solve)
@@ -120,7 +120,7 @@ size_t cov_count(int kind, int64_t n) { return kind == 0 ? 1 : kind == 1 ? (size
 // the work space of its factorisation.
 size_t partials_count(int64_t m) {
   const size_t split = (size_t)kSplitsS * m * m;
-  return m <= kInnovFactorMaxM ? std::max(split, innovation_factor_work(m)) : split;
+  return m <= kInnovFactorMaxM ? std::max(split, (size_t)((m + 32) * round_up(m, 32))) : split;
 }
 
 struct Sizes {
@@ -166,7 +166,7 @@ Sizes sizes_for(const kf_desc* d) {
   w += cov_count(d->q_kind, N) * 8 + m * N * 8 + cov_count(d->r_kind, m) * 8;
   // split planes: rows up to max(N, m), k up to max(ldN, 2 ldm) (the Joseph product's rank 2m)
   if (d->prec == KF_PREC_MIXED_BF16X3) w += tc_scratch_bytes(std::max(N, m), std::max(ldN, 2 * ldm));
-  w += 4096;  // status word, flags of innovation_factor (at most 3.8 KB)
+  w += 4096;  // status word, flags of innovation_factor (T (T / 4 + 2) words, T = m / 32 and N / 32: at most 2.8 KB)
   z.workspace = w;
   return z;
 }
@@ -365,16 +365,16 @@ constexpr int kSBlock = 32;
 
 // S = L L^T in place with the inverses of its diagonal blocks (Sdinv), L^{-1} into Linv (when not null)
 // and, when y != NULL, nu <- L^{-1} (y - H x_{t|t-1}), all float64.  One launch up to kInnovFactorMaxM
-// sensors (its row buffers in shared memory; a whole mixed filter step at N = 1000 takes 1.9 ms with
-// m = 960, and 7.6 ms with the block kernels at m = 961), block kernels above.
+// sensors (its row buffers in shared memory; a whole mixed filter step at N = 1000, m = 960 takes 1.9 ms, and
+// 7.6 ms with the block kernels), block kernels above.
 kf_status factor_innovation(kf_plan_s* p, int64_t t, const double* y, double* Linv) {
   cudaStream_t s = p->s;
   const int m = (int)p->m;
   if (m <= kInnovFactorMaxM) {
     // a non-finite nu is reported by the factorisation, after a bad pivot of S
     if (y) KF_TRY(innovation(s, m, p->N, p->H, p->xpred + t * p->N, y, p->nu, nullptr, (int)t));
-    return innovation_factor(s, m, p->S, m, p->Sdinv, Linv, y ? p->nu : nullptr, p->partials, p->Sflags, p->status,
-                             (int)t);
+    return innovation_factor(s, m, p->S, m, p->Sdinv, Linv, y ? p->nu : nullptr, p->partials,
+                             p->partials + m * round_up(m, 32), p->Sflags, p->status, (int)t);
   }
   KF_TRY(potrf<double>(s, p->S, m, m, p->Sdinv, kSBlock, p->status, (int)t));
   if (Linv) {  // I L^{-1}
@@ -415,7 +415,10 @@ kf_status filter_step(kf_plan_s* p, int64_t t, const double* y, double* diag_out
   const bool joseph = p->d.joseph_every > 0 && (t % p->d.joseph_every) == 0;
   if (joseph) KF_CUDA_TRY(cudaMemcpyAsync(p->S0, p->S, (size_t)m * m * 8, cudaMemcpyDeviceToDevice, s));
   const int nbS = kSBlock;
-  KF_TRY(factor_innovation(p, t, y, nullptr));
+  // float64: L^{-1} with the factor, so that the N x m solves become products (their many small launches
+  // took longer than the twofold arithmetic)
+  const bool inverse = sizeof(B) == sizeof(double);
+  KF_TRY(factor_innovation(p, t, y, inverse ? (double*)p->Sl : nullptr));
   const B* L = (const B*)p->S;
   const B* Ld = (const B*)p->Sdinv;
   if (sizeof(B) != sizeof(double)) {
@@ -429,8 +432,19 @@ kf_status filter_step(kf_plan_s* p, int64_t t, const double* y, double* diag_out
   // solve and is conditioned like L (the square root of cond(S)); the m-sized
   // solve L^{-1} nu of the mean update runs in float64.
   B* Z = (B*)p->Zb;
-  KF_TRY((copy2d<B, B>(s, Z, ldm, Ut, ldm, N, m)));
-  KF_TRY(trsm_right<B>(s, true, N, m, L, m, Ld, nbS, Z, ldm, p->status));
+  GemmParams<B> zi;  // products with L^{-1} (rows zero above the diagonal)
+  zi.M = N; zi.N = m; zi.K = m;
+  zi.B = (const B*)p->Sl; zi.ldb = m;
+  zi.status = p->status;
+  if (inverse) {
+    zi.A = Ut; zi.lda = ldm;
+    zi.tri_b = 1;
+    zi.out = Z; zi.ldo = ldm;
+    KF_TRY(gemm_simt<B>(s, true, zi));
+  } else {
+    KF_TRY((copy2d<B, B>(s, Z, ldm, Ut, ldm, N, m)));
+    KF_TRY(trsm_right<B>(s, true, N, m, L, m, Ld, nbS, Z, ldm, p->status));
+  }
   if (y) KF_TRY(gemv<B>(s, N, m, Z, ldm, p->nu, p->xpred + t * N, 1.0, p->xfilt + t * N));
   const bool ident = p->d.f_kind == KF_F_IDENTITY;
   B* dst = (B*)p->slot_ptr(t);
@@ -452,8 +466,15 @@ kf_status filter_step(kf_plan_s* p, int64_t t, const double* y, double* diag_out
   if (joseph) {
     // Joseph form (I - KH) P (I - KH)^T + K R K^T = P - K V^T - V K^T with
     // K = Z L^{-1} and V = U^T - K S / 2: one rank-2m product [K V][V K]^T.
-    KF_TRY((copy2d<B, B>(s, KV, ldkv, Z, ldm, N, m)));
-    KF_TRY(trsm_right<B>(s, false, N, m, L, m, Ld, nbS, KV, ldkv, p->status));
+    if (inverse) {
+      zi.A = Z; zi.lda = ldm;
+      zi.tri_b = -1;
+      zi.out = KV; zi.ldo = ldkv;
+      KF_TRY(gemm_simt<B>(s, false, zi));
+    } else {
+      KF_TRY((copy2d<B, B>(s, KV, ldkv, Z, ldm, N, m)));
+      KF_TRY(trsm_right<B>(s, false, N, m, L, m, Ld, nbS, KV, ldkv, p->status));
+    }
     KF_TRY((copy2d<B, double>(s, (B*)p->S0b, m, p->S0, m, m, m)));
     GemmParams<B> v;
     v.M = N; v.N = m; v.K = m;
@@ -838,6 +859,11 @@ kf_status run_smoother(kf_plan_s* p, double* x_smooth, double* diagP_smooth, dou
   B* Jm = sizeof(V) == sizeof(B) ? (B*)p->Jb : (B*)p->Jm;
   // a float64 solve in the mixed path: one float64 definition of P_{t+1|t} and of the mean (above)
   const bool fp64sv = p->bulk == BULK_BF16X3 && (sizeof(V) == 8 || p->refine || p->mean_refine);
+  // float64 throughout and N within the one-launch factorisation: it also gives L^{-1} (into the working
+  // covariance, which only the recomputation of skipped steps uses here), and the two solves of N rows become
+  // triangular products (N = 384: factor and gain 2.6 -> 0.9 ms)
+  const bool direct = sizeof(B) == 8 && p->Lflags != nullptr;
+  double* Linv = (double*)p->P;
   // t = T: smoothed = filtered
   KF_CUDA_TRY(cudaMemcpyAsync(p->xs + T * N, p->xfilt + T * N, N * 8, cudaMemcpyDeviceToDevice, s));
   const B* PT;
@@ -878,6 +904,9 @@ kf_status run_smoother(kf_plan_s* p, double* x_smooth, double* diagP_smooth, dou
         Prof pf(p, KF_KC_SOLVE_FACTOR);
         if (tc_solve)
           KF_TRY(chol_inverse_step(p, (float*)Lb, (int)(t + 1)));
+        else if (direct)
+          KF_TRY(innovation_factor(s, (int)N, (double*)Lb, ldN, (double*)p->Ldinv, Linv, nullptr, (double*)Wb,
+                                   (double*)p->Ldinv + 32 * round_up(N, 32), p->Lflags, p->status, (int)(t + 1)));
         else
           KF_TRY(potrf<V>(s, Lb, ldN, (int)N, (V*)p->Ldinv, nbs, p->status, (int)(t + 1)));
       }
@@ -945,6 +974,20 @@ kf_status run_smoother(kf_plan_s* p, double* x_smooth, double* diagP_smooth, dou
         }
         KF_TRY(gain_from_inverse_tc(s, p->tc, (int)N, (const float*)Bm, ldN, p->Wi, ldN, (float*)p->tmpN, ldN,
                                     (float*)Jb, ldN, p->status));
+      } else if (direct) {
+        // J = (Bm L^{-T}) L^{-1}: two triangular products
+        GemmParams<B> z;
+        z.M = (int)N; z.N = (int)N; z.K = (int)N;
+        z.A = Bm; z.lda = ldN;
+        z.B = (const B*)Linv; z.ldb = N;
+        z.tri_b = 1;
+        z.out = (B*)Lb; z.ldo = ldN;
+        z.status = p->status;
+        KF_TRY(gemm_simt<B>(s, true, z));
+        z.A = (const B*)Lb;
+        z.tri_b = -1;
+        z.out = (B*)Jb;
+        KF_TRY(gemm_simt<B>(s, false, z));
       } else {
         KF_TRY((copy2d<V, B>(s, Jb, ldN, Bm, ldN, N, N)));
         KF_TRY(trsm_right<V>(s, true, (int)N, (int)N, Lb, ldN, (const V*)p->Ldinv, nbs, Jb, ldN, p->status));
@@ -1121,6 +1164,7 @@ kf_status kf_plan(kf_plan_t* out, const kf_desc* d) {
   A(&p->Sdinv, round_up(m, 64) * 64 * 8);
   A(&p->partials, partials_count(m) * 8);
   if (m <= kInnovFactorMaxM) A(&p->Sflags, innovation_factor_flags(m) * sizeof(int));
+  if (p->bulk == BULK_F64 && N <= kInnovFactorMaxM) A(&p->Lflags, innovation_factor_flags(N) * sizeof(int));
   A(&p->Sl, m * m * b);
   A(&p->Sldinv, round_up(m, 64) * 64 * b);
   A(&p->S0b, m * m * b);

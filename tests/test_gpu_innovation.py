@@ -59,3 +59,35 @@ def test_failure_in_a_later_tile_then_recovery(prec, solve):
         assert st == B.KF_ERR_NUMERIC and step == 2
         st, step, x1 = _filter(plan, good, T, N)
         assert st == B.KF_OK and torch.equal(x0, x1)
+
+
+@pytest.mark.parametrize("N,m,T,mesh", [(33, 5, 3, True), (320, 40, 3, False), (1536, 20, 2, False), (1537, 20, 2, False)])
+def test_float64_gain_on_both_sides_of_the_direct_size(N, m, T, mesh):
+    """Float64 smoother with the one-launch factor and inverse of P_{t+1|t} and, above 1536 sources, with the
+    block kernels; Joseph form every second step."""
+    prob = synth.mesh_problem(N, m, T, seed=N, identity_F=not mesh)
+    out, ref = solver.run(prob, prec=B.KF_PREC_FP64, joseph_every=2), run_oracle(prob)
+    for k, tol in (("x_filt", 1e-10), ("x_smooth", 1e-10)):
+        assert rel_err_per_step(out[k], ref[k]) <= tol
+    for k, r in (("diagP_filt", "P_filt"), ("diagP_smooth", "P_smooth")):
+        assert rel_err_elementwise(out[k], diag_of(ref[r])) <= 1e-10
+
+
+def test_float64_gain_reports_a_singular_prediction():
+    """P_{t+1|t} singular (Q = 0, P0 of low rank): the smoother's factor reports the step, and the plan works again."""
+    N, m, T = 100, 8, 3
+    prob = synth.random_walk_problem(N, m, T, seed=3)
+    good = solver.upload(prob)
+    with solver.Plan.for_inputs(good, N, m, T) as plan:
+        st, _, _ = _filter(plan, good, T, N)
+        x0 = plan.smooth()[0]
+        bad = solver.upload(prob)
+        bad.Q = torch.zeros_like(bad.Q)
+        bad.P0 = torch.diag(torch.cat([torch.ones(70), torch.full((N - 70,), 1e-300)]).double()).cuda()
+        bad.P0[80:, :] = 0
+        st, step, x = _filter(plan, bad, T, N)
+        if st == B.KF_OK:
+            st, step = B.fis_smooth(plan.handle, x, raise_on_error=False)
+        assert st in (B.KF_ERR_NOT_PD, B.KF_ERR_NUMERIC)
+        st, _, _ = _filter(plan, good, T, N)
+        assert st == B.KF_OK and torch.equal(plan.smooth()[0], x0)

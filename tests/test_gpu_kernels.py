@@ -282,3 +282,21 @@ def test_tc_wait_limit_timeout_then_recovery():
     B.kfx_gemm(3, 1, 0, M, N, K, 1.0, dA, K, dB, K, 0.0, dC, N)
     full = A.astype(np.float64) @ Bm.astype(np.float64).T
     assert np.linalg.norm(dC.double().cpu().numpy() - full) <= 2e-6 * np.linalg.norm(full)
+
+
+@pytest.mark.parametrize("M,N,K,transB,sym", [(16, 16, 40, 1, 0), (17, 33, 5, 0, 0), (32, 31, 64, 1, 0), (65, 64, 16, 0, 0),
+                                              (96, 800, 20, 1, 0), (800, 96, 20, 0, 0), (400, 400, 33, 1, 1),
+                                              (801, 801, 17, 1, 1), (1700, 1500, 9, 0, 0), (2500, 2500, 7, 1, 1)])
+def test_gemm_float64_tiles(M, N, K, transB, sym):
+    """Float64 products around the sizes where the dispatch changes between 16-, 32- and 64-wide tiles."""
+    rng = np.random.default_rng(M + N + K)
+    A = rng.standard_normal((M, K))
+    Bm = A if sym else rng.standard_normal((N, K) if transB else (K, N))
+    dA, dB = _dev(A, 0), _dev(Bm, 0)
+    dC = torch.zeros(M, N, dtype=torch.float64, device="cuda")
+    B.kfx_gemm(0, transB, sym, M, N, K, 1.0, dA, K, dB, K if transB else N, 0.0, dC, N)
+    ref = A @ (Bm.T if transB else Bm)
+    got = dC.cpu().numpy()
+    assert np.abs(got - ref).max() <= 1e-13 * np.abs(ref).max() * max(1, np.sqrt(K) / 4)
+    if sym:
+        assert np.array_equal(got, got.T)
