@@ -91,3 +91,27 @@ def test_float64_gain_reports_a_singular_prediction():
         assert st in (B.KF_ERR_NOT_PD, B.KF_ERR_NUMERIC)
         st, _, _ = _filter(plan, good, T, N)
         assert st == B.KF_OK and torch.equal(plan.smooth()[0], x0)
+
+
+@pytest.mark.parametrize("N,m,T,sensors,sources", [(300, 20, 5, 0, 0), (700, 64, 40, 6, 0), (130, 129, 3, 0, 8),
+                                                   (900, 120, 60, 4, 4), (40, 1537, 3, 0, 0)])
+def test_mne_with_sensors_and_sources_in_different_units(N, m, T, sensors, sources):
+    """The minimum-norm products on slices keep float64 accuracy when sensors (rows) or sources (columns) are
+    scaled apart by up to e^12 and e^16; per-source error, 1e-11 for the conditioning of G."""
+    rng = np.random.default_rng(N + m)
+    u, c = np.exp(rng.uniform(-sensors, sensors, m)), np.exp(rng.uniform(-sources, sources, N))
+    H = rng.standard_normal((m, N)) * u[:, None] / np.sqrt(c)
+    R, Y = rng.uniform(0.5, 2, m) * u ** 2, rng.standard_normal((T, m)) * u
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    X = torch.empty(T, N, dtype=torch.float64, device="cuda")
+    B.mne_solve(t(H), t(c), 1, t(R), 1, t(Y), N, m, T, 1.3, X)
+    # the reference in extended precision: float64 solves of the balanced system, refined (with m much larger than
+    # N a float64 solve alone is off by the tolerance)
+    Hl = H.astype(np.longdouble) / u[:, None]
+    G = 1.3 * (Hl * c) @ Hl.T + np.diag(R / u ** 2).astype(np.longdouble)
+    rhs, V = (Y / u).T.astype(np.longdouble), np.zeros((m, T), np.longdouble)
+    for _ in range(4):
+        V = V + np.linalg.solve(G.astype(np.float64), (rhs - G @ V).astype(np.float64))
+    ref = (1.3 * V.T @ (Hl * c)).astype(np.float64)
+    err = np.linalg.norm(X.cpu().numpy() - ref, axis=0) / np.linalg.norm(ref, axis=0)
+    assert err.max() <= 1e-11
