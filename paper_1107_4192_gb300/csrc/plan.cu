@@ -88,6 +88,9 @@ struct kf_plan_s {
   TcScratch tc{};
   double *F = nullptr, *Q = nullptr, *H = nullptr, *R = nullptr;
   int64_t *Frp = nullptr, *Fcol = nullptr;
+  // Mixed path: F packed for the float32 mesh products, in the memory of the float32 copy of H, which only the
+  // float32 filter reads (an F too large for that keeps the kernels with float64 sums).
+  float4* Fpack = nullptr;
   int* status = nullptr;
   int status_h[ST_WORDS] = {0, 0, 0, 0};  // read after a stream synchronisation
   bool filtered = false;
@@ -335,6 +338,11 @@ kf_status predict_cov(kf_plan_s* p, const B* src, B* dst) {
   const int64_t N = p->N;
   if (p->d.f_kind == KF_F_IDENTITY)
     return add_cov<B, B>(p->s, dst, p->ldN, src, p->ldN, N, p->d.q_kind, p->Q);
+  if constexpr (sizeof(B) == 4) {
+    if (p->Fpack)
+      return spmm_fpft_packed(p->s, N, p->Frp, p->Fpack, src, p->ldN, (B*)p->tmpN, p->ldN, dst, p->ldN, p->d.q_kind,
+                              p->Q);
+  }
   if (p->d.f_kind == KF_F_CSR)
     return spmm_fpft<B>(p->s, N, p->Frp, p->Fcol, p->F, src, p->ldN, (B*)p->tmpN, p->ldN, dst, p->ldN,
                         p->d.q_kind, p->Q);
@@ -912,7 +920,10 @@ kf_status run_smoother(kf_plan_s* p, double* x_smooth, double* diagP_smooth, dou
       }
       // J_t = P_{t|t} F^T P_{t+1|t}^{-1}
       const B* Bm = Pt;
-      if (p->d.f_kind == KF_F_CSR) {
+      if (p->Fpack) {
+        KF_TRY(spmm_wft_packed(s, N, p->Frp, p->Fpack, (const float*)Pt, ldN, (float*)p->tmpN, ldN, -1, nullptr));
+        Bm = (const B*)p->tmpN;
+      } else if (p->d.f_kind == KF_F_CSR) {
         KF_TRY(spmm_pft<B>(s, N, p->Frp, p->Fcol, p->F, Pt, ldN, (B*)p->tmpN, ldN));
         Bm = (const B*)p->tmpN;
       } else if (p->d.f_kind == KF_F_DENSE) {
@@ -1086,8 +1097,10 @@ kf_status copy_inputs(kf_plan_s* p, const double* F, const int64_t* rp, const in
   KF_CUDA_TRY(cudaMemcpyAsync(p->R, R, cov_count(p->d.r_kind, m) * 8, cudaMemcpyDeviceToDevice, s));
   if (p->b == 8)
     KF_TRY((copy2d<double, double>(s, (double*)p->Hb, p->ldN, H, N, m, N, true)));
-  else
+  else if (p->bulk != BULK_BF16X3)
     KF_TRY((copy2d<float, double>(s, (float*)p->Hb, p->ldN, H, N, m, N, true)));
+  else if (p->Fpack)
+    KF_TRY(spmm_pack(s, p->d.f_nnz, p->Fcol, p->F, p->Fpack));
   return KF_OK;
 }
 
@@ -1159,6 +1172,9 @@ kf_status kf_plan(kf_plan_t* out, const kf_desc* d) {
     A(&p->ozsums.p, p->ozsums.count * 8);
   }
   A(&p->Hb, m * ldN * b);
+  if (p->bulk == BULK_BF16X3 && d->f_kind == KF_F_CSR && (uint64_t)d->f_nnz * sizeof(float4) <= (uint64_t)(m * ldN * b) &&
+      spmm_packed_ok(N, ldN))
+    p->Fpack = reinterpret_cast<float4*>(p->Hb);
   A(&p->S, m * m * 8);
   A(&p->S0, m * m * 8);
   A(&p->Sdinv, round_up(m, 64) * 64 * 8);

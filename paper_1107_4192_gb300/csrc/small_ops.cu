@@ -233,21 +233,45 @@ kf_status gemv_f64acc(cudaStream_t s, int64_t rows, int64_t cols, const float* A
   return launch_check("gemv_f64acc");
 }
 
-// y = ybase + sign A^T x: one thread per column, consecutive threads read consecutive columns.
-__global__ void gemv_t_kernel(int64_t rows, int64_t cols, const double* A, int64_t lda, const double* x,
-                              const double* ybase, double sign, double* y) {
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < cols; j += (int64_t)gridDim.x * blockDim.x) {
+// y = ybase + sign A^T x: a block owns 32 columns; its 32 warps take the rows w, w + 32, .. (256-byte row
+// pieces, eight in flight per warp) and their sums are added in warp order.  One thread per column and all its
+// rows left most SMs idle behind one dependent chain each (N = 5124: 0.85 ms, now 0.09 ms).
+__global__ void __launch_bounds__(1024) gemv_t_kernel(int64_t rows, int64_t cols, const double* A, int64_t lda,
+                                                      const double* x, const double* ybase, double sign, double* y) {
+  __shared__ double part[32][33];
+  const int lane = threadIdx.x % 32, w = threadIdx.x / 32;
+  for (int64_t j0 = blockIdx.x * (int64_t)32; j0 < cols; j0 += (int64_t)gridDim.x * 32) {
+    const int64_t j = j0 + lane;
     double acc = 0.0;
-    for (int64_t i = 0; i < rows; ++i) acc = fma(A[i * lda + j], x[i], acc);
-    y[j] = ybase ? ybase[j] + sign * acc : acc;
+    if (j < cols) {
+      const double* a = A + j;
+      int64_t i = w;
+      for (; i + 7 * 32 < rows; i += 8 * 32) {
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = a[(i + 32 * u) * lda];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc = fma(v[u], x[i + 32 * u], acc);
+      }
+      for (; i < rows; i += 32) acc = fma(a[i * lda], x[i], acc);
+    }
+    part[w][lane] = acc;
+    __syncthreads();
+    if (w == 0 && j < cols) {
+      double sum = 0.0;
+#pragma unroll
+      for (int k = 0; k < 32; ++k) sum += part[k][lane];
+      y[j] = ybase ? ybase[j] + sign * sum : sum;
+    }
+    __syncthreads();
   }
 }
 
 kf_status gemv_t(cudaStream_t s, int64_t rows, int64_t cols, const double* A, int64_t lda, const double* x,
                  const double* ybase, double sign, double* y) {
   if (cols <= 0) return KF_OK;
-  gemv_t_kernel<<<(unsigned)std::min<int64_t>(ceil_div(cols, 128), 1024), 128, 0, s>>>(rows, cols, A, lda, x, ybase,
-                                                                                   sign, y);
+  gemv_t_kernel<<<(unsigned)std::min<int64_t>(ceil_div(cols, 32), 4096), 1024, 0, s>>>(rows, cols, A, lda, x, ybase, sign,
+                                                                                   y);
   note_launch();
   return launch_check("gemv_t");
 }
@@ -307,28 +331,31 @@ kf_status vsub(cudaStream_t s, int64_t n, const double* a, const double* b, doub
   return launch_check("vsub");
 }
 
-__global__ void innovation_kernel(int64_t m, int64_t N, const double* H, const double* x, const double* y,
-                                  double* nu, int* status, int step) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t i = warp; i < m; i += nwarps) {
+// One row of H per block of four warps, the lane sums added in lane and warp order (a warp per row and eight rows
+// per block left the float64 work of 306 rows to 39 SMs: N = 5124 42 us, now 13 us).
+__global__ void __launch_bounds__(128) innovation_kernel(int64_t m, int64_t N, const double* H, const double* x,
+                                                         const double* y, double* nu, int* status, int step) {
+  __shared__ double part[4];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int64_t i = blockIdx.x; i < m; i += gridDim.x) {
     double acc = 0.0;
-    for (int64_t j = lane; j < N; j += 32) acc = fma(H[i * N + j], x[j], acc);
+    for (int64_t j = threadIdx.x; j < N; j += 128) acc = fma(H[i * N + j], x[j], acc);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) {
-      double v = y[i] - acc;
+    if (lane == 0) part[w] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      const double v = y[i] - (((part[0] + part[1]) + part[2]) + part[3]);
       nu[i] = v;
       if (!isfinite(v)) status_set(status, KF_ERR_NUMERIC, step, (int)i);
     }
+    __syncthreads();
   }
 }
 
 kf_status innovation(cudaStream_t s, int64_t m, int64_t N, const double* H, const double* x,
                      const double* y, double* nu, int* status, int step) {
-  unsigned blocks = (unsigned)std::min<int64_t>(ceil_div(m * 32, 256), 1024);
-  innovation_kernel<<<blocks, 256, 0, s>>>(m, N, H, x, y, nu, status, step);
+  innovation_kernel<<<(unsigned)std::min<int64_t>(m, 65535), 128, 0, s>>>(m, N, H, x, y, nu, status, step);
   note_launch();
   return launch_check("innovation");
 }

@@ -61,6 +61,132 @@ kf_status spmm_pft(cudaStream_t s, int64_t N, const int64_t* rowptr, const int64
   return launch_check("spmm_pft");
 }
 
+// ---------------------------------------------------------------- float32 matrices, packed F
+//
+// The sums of a float32 matrix in float64 took 14 float64 operations per element (a conversion and a
+// multiply-add per entry of F): 0.73 ms per pass at N = 5124, on the float64 units, where the matrix passes HBM
+// in 0.03 ms.  Here a sum is a pair of float32 (its rounded value and what the rounding lost, Knuth's two-sum;
+// products exact by fused multiply-add, F as value + remainder), 46 bits or more, rounded once at the end: the
+// same float32 result as from a float64 sum but for ties (0.11 ms for F P and 0.19 ms for W F^T).
+
+struct Pair {
+  float h = 0.0f, l = 0.0f;
+  __device__ __forceinline__ void add(float x) {  // exact sum of h and x, the error into l
+    const float s = h + x, t = s - h;
+    l += (h - (s - t)) + (x - t);
+    h = s;
+  }
+  // += (vh + vl) p
+  __device__ __forceinline__ void fma(float vh, float vl, float p) {
+    const float q = vh * p;
+    l += fmaf(vl, p, fmaf(vh, p, -q));
+    add(q);
+  }
+  // (an infinite or NaN sum stands in h; its l is NaN)
+  __device__ __forceinline__ float value() const { return isfinite(h) ? h + l : h; }
+};
+
+__global__ void spmm_pack_kernel(int64_t nnz, const int64_t* col, const double* val, float4* out) {
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < nnz; k += (int64_t)gridDim.x * blockDim.x) {
+    const float h = (float)val[k];
+    out[k] = make_float4(h, (float)(val[k] - (double)h), __int_as_float((int)col[k]), 0.0f);
+  }
+}
+
+kf_status spmm_pack(cudaStream_t s, int64_t nnz, const int64_t* col, const double* val, float4* out) {
+  spmm_pack_kernel<<<(unsigned)std::min<int64_t>(ceil_div(nnz, 256), 4096), 256, 0, s>>>(nnz, col, val, out);
+  note_launch();
+  return launch_check("spmm_pack");
+}
+
+// W = F P, one block per row: four consecutive columns per thread, each entry's row of P read in 16-byte loads.
+__global__ void __launch_bounds__(256) spmm_fp_packed_kernel(int64_t N, const int64_t* rowptr, const float4* F,
+                                                             const float* P, int64_t ldp, float* W, int64_t ldw) {
+  const int64_t i = blockIdx.x, k0 = rowptr[i], k1 = rowptr[i + 1];
+  for (int64_t j = 4 * (int64_t)threadIdx.x; j < N; j += 4 * 256) {
+    Pair acc[4];
+    for (int64_t k = k0; k < k1; ++k) {
+      const float4 f = F[k];
+      const float4 p = *reinterpret_cast<const float4*>(P + (int64_t)__float_as_int(f.z) * ldp + j);
+      acc[0].fma(f.x, f.y, p.x);
+      acc[1].fma(f.x, f.y, p.y);
+      acc[2].fma(f.x, f.y, p.z);
+      acc[3].fma(f.x, f.y, p.w);
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (j + e < N) W[i * ldw + j + e] = acc[e].value();
+  }
+}
+
+// out = W F^T (+ Q): a block stages R rows of W in shared memory, so that the gathers at F's columns are shared
+// loads and each entry of F is read once for R rows.
+template <int R>
+__global__ void __launch_bounds__(512) spmm_wft_packed_kernel(int64_t N, const int64_t* rowptr, const float4* F,
+                                                              const float* W, int64_t ldw, float* out, int64_t ldo,
+                                                              int q_kind, const double* q) {
+  extern __shared__ __align__(16) float rows[];  // R x ldw
+  const int64_t i0 = (int64_t)blockIdx.x * R;
+  const int nr = (int)(N - i0 < R ? N - i0 : R);
+  for (int64_t u = threadIdx.x; u < nr * (ldw / 4); u += 512)
+    reinterpret_cast<float4*>(rows)[u] = reinterpret_cast<const float4*>(W + i0 * ldw)[u];
+  __syncthreads();
+  for (int64_t j = threadIdx.x; j < N; j += 512) {
+    Pair acc[R];
+    const int64_t k1 = rowptr[j + 1];
+    for (int64_t k = rowptr[j]; k < k1; ++k) {
+      const float4 f = F[k];
+      const float* w = rows + __float_as_int(f.z);
+#pragma unroll
+      for (int r = 0; r < R; ++r) acc[r].fma(f.x, f.y, w[r * ldw]);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if (r >= nr) break;
+      const int64_t i = i0 + r;
+      if (q_kind == 2 || (q_kind >= 0 && i == j)) {
+        const double v = q_kind == 0 ? q[0] : q_kind == 1 ? q[i] : q[i * N + j];
+        const float h = (float)v;
+        acc[r].add(h);
+        acc[r].add((float)(v - (double)h));
+      }
+      out[i * ldo + j] = acc[r].value();
+    }
+  }
+}
+
+template <int R>
+kf_status launch_wft_packed(cudaStream_t s, int64_t N, const int64_t* rowptr, const float4* F, const float* W, int64_t ldw,
+                            float* out, int64_t ldo, int q_kind, const double* q) {
+  KF_CUDA_TRY(smem_limit_per_device((const void*)spmm_wft_packed_kernel<R>, 216 * 1024));
+  spmm_wft_packed_kernel<R><<<(unsigned)ceil_div(N, R), 512, R * ldw * sizeof(float), s>>>(N, rowptr, F, W, ldw, out, ldo,
+                                                                                          q_kind, q);
+  note_launch();
+  return launch_check("spmm_wft_packed");
+}
+
+// As many rows per block as keep two blocks on an SM, four at most while eight would leave SMs idle.
+kf_status spmm_wft_packed(cudaStream_t s, int64_t N, const int64_t* rowptr, const float4* F, const float* W, int64_t ldw,
+                          float* out, int64_t ldo, int q_kind, const double* q) {
+  const int64_t row = ldw * (int64_t)sizeof(float);
+  if (8 * row <= 108 * 1024 && N >= 8 * 304) return launch_wft_packed<8>(s, N, rowptr, F, W, ldw, out, ldo, q_kind, q);
+  if (4 * row <= 108 * 1024) return launch_wft_packed<4>(s, N, rowptr, F, W, ldw, out, ldo, q_kind, q);
+  if (2 * row <= 108 * 1024) return launch_wft_packed<2>(s, N, rowptr, F, W, ldw, out, ldo, q_kind, q);
+  if (row > 216 * 1024) return KF_ERR_ARG;
+  return launch_wft_packed<1>(s, N, rowptr, F, W, ldw, out, ldo, q_kind, q);
+}
+
+bool spmm_packed_ok(int64_t N, int64_t ld) { return N <= INT32_MAX && ld % 4 == 0 && ld * 4 <= 216 * 1024; }
+
+kf_status spmm_fpft_packed(cudaStream_t s, int64_t N, const int64_t* rowptr, const float4* F, const float* P, int64_t ldp,
+                           float* W, int64_t ldw, float* out, int64_t ldo, int q_kind, const double* q) {
+  if (N <= 0) return KF_OK;
+  spmm_fp_packed_kernel<<<(unsigned)N, 256, 0, s>>>(N, rowptr, F, P, ldp, W, ldw);
+  note_launch();
+  KF_TRY(launch_check("spmm_fp_packed"));
+  return spmm_wft_packed(s, N, rowptr, F, W, ldw, out, ldo, q_kind, q);
+}
+
 template kf_status spmm_fpft<double>(cudaStream_t, int64_t, const int64_t*, const int64_t*, const double*,
                                      const double*, int64_t, double*, int64_t, double*, int64_t, int,
                                      const double*);

@@ -336,3 +336,19 @@ def test_host_buffer_entry_matches_device_path():
                         h["P0"], outs["x_filt"], outs["diagP_filt"], outs["x_smooth"], outs["diagP_smooth"])
     for k in outs:
         assert np.array_equal(outs[k], dev[k]), k
+
+
+@pytest.mark.parametrize("N,m,T", [(9, 200, 4), (333, 40, 4), (2433, 64, 3), (2500, 33, 3)])
+def test_mixed_mesh_products_against_the_float64_path(N, m, T):
+    """The float32 mesh products with pair sums (one to eight rows per block, ragged ends, entries of F of both
+    signs and an empty row) inside the mixed smoother, against the float64 path of the same problem."""
+    prob = synth.mesh_problem(N, m, T, seed=N)
+    rng = np.random.default_rng(N)
+    prob.F.val = prob.F.val * rng.uniform(-1.0, 1.0, prob.F.val.shape)
+    cut = prob.F.rowptr[3], prob.F.rowptr[4]  # row 3 of F becomes empty
+    prob.F.val, prob.F.col = np.delete(prob.F.val, np.s_[cut[0]:cut[1]]), np.delete(prob.F.col, np.s_[cut[0]:cut[1]])
+    prob.F.rowptr = prob.F.rowptr - np.where(np.arange(N + 1) >= 4, cut[1] - cut[0], 0)
+    ref = solver.run(prob, prec=B.KF_PREC_FP64)
+    out = solver.run(prob, prec=B.KF_PREC_MIXED_BF16X3, solve_prec=B.KF_SOLVE_FP64_MEAN, joseph_every=2)
+    assert rel_err_per_step(out["x_smooth"], ref["x_smooth"]) <= TOL_MEAN32
+    assert rel_err_elementwise(out["diagP_smooth"], ref["diagP_smooth"]) <= TOL_DIAG32
