@@ -107,6 +107,15 @@ size_t innovation_factor_flags(int64_t m);
 kf_status innovation_factor(cudaStream_t s, int m, double* S, int64_t lds, double* dinv, double* Linv, double* nu,
                             double* W, double* Dt, int* flags, int* status, int step);
 
+// L (n x n float32, lower triangle, in place) <- chol(L) and W <- L^{-1} (lower triangle and the zeros above the
+// diagonal of its 32 x 32 diagonal tiles) in one launch, n <= kCholDirectMaxN.  L and W 16-byte aligned with
+// row strides in multiples of 4; scratch: chol_direct_scratch(n) bytes, cleared by the call.  base: index of
+// the first pivot in a bad pivot's report.
+constexpr int kCholDirectMaxN = 2048;
+size_t chol_direct_scratch(int n);
+kf_status chol_inverse_direct(cudaStream_t s, int n, float* L, int64_t ldl, float* W, int64_t ldw, void* scratch,
+                              int* status, int step, int base);
+
 // ---------------------------------------------------------------- small ops
 
 // dst[i, j] = (Tdst) src[i, j] for i < rows, j < cols; pad columns cols..ld_dst-1 zeroed

@@ -2,16 +2,14 @@
 //
 // J_t = P_{t|t} F^T P_{t+1|t}^{-1} (eqn 11) is formed as
 //   P_{t+1|t} = L L^T,   W = L^{-1},   J_t = ((P_{t|t} F^T) W^T) W,
-// so that, apart from the nb x nb diagonal blocks, all O(N^3) work is large
+// so that, apart from the diagonal blocks, all O(N^3) work is large
 // products that run as three-way split-bf16 GEMMs (six bf16 products with
 // float32 accumulation, float32-class accuracy) on the tensor cores:
 //  - Cholesky, recursive on halves:  L11 = chol(A11);  L21 = A21 W11^T;
 //    A22 <- A22 - L21 L21^T;  L22 = chol(A22);
 //  - triangular inverse on the same halves: W21 = -W22 (L21 W11);
-//  - the diagonal blocks (nb = 128) are factored and inverted by one CTA each.
-// Products with a triangular operand skip the k-tiles outside its band.  The
-// small products near the leaves run in float32 on the CUDA cores, where
-// their latency is a fraction of a tensor-core launch.
+//  - the diagonal blocks (up to kDirectMax rows) are factored and inverted by one launch each (chol_direct.cu).
+// Products with a triangular operand skip the k-tiles outside its band.
 // This replaces the two triangular solves with N right-hand sides by a
 // triangular inverse and two triangular products (2.67 N^3 instead of
 // 2.33 N^3 flops), in exchange for large, fully parallel products only.
@@ -45,32 +43,21 @@ struct Ctx {
 
 int split_point(int n, int nb) { return (int)round_up((n + 1) / 2, nb); }
 
-// Products up to about 640^3 are latency-bound on the tensor-core path (an
-// operand split plus the tensor-core kernel cost ~30 us at any size below
-// 512^3); they run as pipelined float32 CUDA-core products instead.
-constexpr int64_t kSmallWork = int64_t(1) << 28;
-
 kf_status gemm(Ctx& c, const GemmParams<float>& g, bool transB) {
-  if ((int64_t)g.M * g.N * g.K <= kSmallWork) {
-    if (gemm_small_ok(transB, g)) return gemm_small(c.s, transB, g);
-    if (gemm_small_alias(transB, g) == SmallAlias::kOther && g.A != c.T && g.B != c.T && !g.cin && !g.csub) {
-      // in place wider than one tile (L21 = A21 W11^T): through the scratch T
-      GemmParams<float> t = g;
-      t.out = c.T;
-      t.ldo = c.ldt;
-      if (gemm_small_ok(transB, t)) {
-        KF_TRY(gemm_small(c.s, transB, t));
-        return copy2d<float, float>(c.s, g.out, g.ldo, c.T, c.ldt, g.M, g.N);
-      }
-    }
-  }
-  // the tensor-core path splits both operands into scratch first, so in place is safe there
+  // both operands are split into scratch first, so in place is safe
   return tc_gemm_split(c.s, *c.sc, g, 3, transB);
 }
 
+// Matrices up to this size are factored and inverted by one launch (chol_direct.cu); above it the products
+// between the halves are large enough for the tensor cores.  Whole smoothing calls with the line at 1024 / 1536 /
+// 2048: N = 1501 8.97 / 8.60 / 8.62 ms, N = 2048 12.56 / 12.48 / 14.00 ms, N = 5124 (leaves of 1281) 23.4 / 22.4 /
+// 22.5 ms, N = 8196 (leaves of 1025) 136.4 / 135.8 / 137.5 ms.
+constexpr int kDirectMax = 1536;
+static_assert(kDirectMax <= kCholDirectMaxN, "leaf size");
+
 kf_status trtri_rec(Ctx& c, int off, int n) {
   if (c.done.count({off, n})) return KF_OK;
-  if (n <= c.nb) return KF_ERR_ARG;  // leaves come from potrf_diag
+  if (n <= kDirectMax) return KF_ERR_ARG;  // leaves come from potrf_rec
   const int n1 = split_point(n, c.nb), n2 = n - n1;
   KF_TRY(trtri_rec(c, off, n1));
   KF_TRY(trtri_rec(c, off + n1, n2));
@@ -98,9 +85,9 @@ kf_status trtri_rec(Ctx& c, int off, int n) {
 }
 
 kf_status potrf_rec(Ctx& c, int off, int n) {
-  if (n <= c.nb) {
-    KF_TRY(potrf_diag<float>(c.s, c.L + (int64_t)off * c.ldl + off, c.ldl, n, c.W + (int64_t)off * c.ldw + off,
-                             c.ldw, c.status, c.step, off));
+  if (n <= kDirectMax) {
+    KF_TRY(chol_inverse_direct(c.s, n, c.L + (int64_t)off * c.ldl + off, c.ldl, c.W + (int64_t)off * c.ldw + off,
+                               c.ldw, c.sc->a[0], c.status, c.step, off));
     c.done.insert({off, n});
     return KF_OK;
   }

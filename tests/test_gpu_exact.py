@@ -295,3 +295,21 @@ def test_refined_inverse_ragged_sizes(n):
     ref = np.linalg.inv(A.astype(np.float64))
     assert np.linalg.norm(X.cpu().numpy() - ref) <= 1e-12 * np.linalg.norm(ref)
     assert torch.equal(X, X.T)
+
+
+@pytest.mark.parametrize("n,bad", [(1, (0,)), (31, (30,)), (32, (0, 31)), (33, (32,)), (64, (31, 32)), (65, (64,)),
+                                   (1024, (500,)), (1535, (1534,)), (1536, (767,)), (1537, (895, 896, 1536))])
+def test_one_launch_factor_and_inverse(n, bad):
+    """The float32 factor and triangular inverse around its 32-wide tiles and at the size above which it runs on
+    halves: X = W^T W against numpy (float32 sums of 32 terms, 32 x 6e-8 x cond 100 = 2e-4), and the index of the
+    first bad pivot (a zero row and column) in either half."""
+    A = spd32(n, 100.0 if n > 1 else 1.0, n)
+    X = torch.zeros(n, n, dtype=torch.float64, device="cuda")
+    for i in bad:
+        Z = A.copy()
+        Z[i, :] = 0.0
+        Z[:, i] = 0.0
+        assert B.kfx_spd_inverse(1, n, torch.from_numpy(Z).cuda(), n, X, n) == (B.KF_ERR_NOT_PD, i)
+    assert B.kfx_spd_inverse(1, n, torch.from_numpy(A).cuda(), n, X, n) == (0, -1)
+    ref = np.linalg.inv(A.astype(np.float64))
+    assert np.linalg.norm(X.cpu().numpy() - ref) <= 2e-4 * np.linalg.norm(ref)
