@@ -10,12 +10,13 @@
 // smoother's W = J D and P + W J^T (eqn 13), the innovation U^T = P H^T
 // (eqn 8) and the update P - K U (eqn 10).
 //
-// Kernel structure (one 128 x BN output tile per CTA, 6 warps):
+// Kernel structure (one 128 x BN output tile per CTA, 10 warps):
 //   warp 0  one lane issues TMA loads (cp.async.bulk.tensor, 128-byte
-//           swizzle) of the four operand tiles of a 64-wide k-slice into a
-//           shared-memory stage and arms the stage's "full" mbarrier;
-//   warp 1  allocates TMEM; one lane waits for "full", issues the 12
-//           tcgen05.mma (3 products x 4 k16 steps) and commits them to the
+//           swizzle) of the 2 S operand tiles of a 64-wide k-slice (128 x 256
+//           with S = 3: 32-wide, 64-byte swizzle, two stages per k-tile) into
+//           a shared-memory stage and arms the stage's "full" mbarrier;
+//   warp 1  allocates TMEM; one lane waits for "full", issues its tcgen05.mma
+//           (3 or 6 products per k16 step) and commits them to the
 //           stage's "empty" mbarrier, which hands the stage back to the TMA
 //           lane when the MMAs have read it; at the end it commits to the
 //           "accumulator ready" barrier;
@@ -48,26 +49,27 @@ constexpr int NUM_THREADS = 320;  // TMA warp, MMA warp, 8 epilogue warps
 
 template <int BN, int S>  // S = bf16 slices per operand: 2 -> 3 products, 3 -> 6 products
 struct TcCfg {
-  static constexpr int A_BYTES = BM * BK * 2;   // one plane
-  static constexpr int B_BYTES = BN * BK * 2;
+  // k-elements per stage: half a k-tile where a whole one would leave no room for a second stage
+  static constexpr int SK = S * (BM + BN) * BK * 2 > 100 * 1024 ? BK / 2 : BK;
+  static constexpr int SUB = BK / SK;           // stages per k-tile
+  static constexpr uint32_t SBO = 8 * SK * 2;   // 8-row swizzle atom
+  static constexpr uint32_t LAYOUT = SK == 64 ? kLayoutSw128 : kLayoutSw64;
+  static constexpr int A_BYTES = BM * SK * 2;   // one plane
+  static constexpr int B_BYTES = BN * SK * 2;
   static constexpr int STAGE_BYTES = S * A_BYTES + S * B_BYTES;
-  static constexpr int STAGES = (200 * 1024) / STAGE_BYTES;
+  static constexpr int STAGES = (216 * 1024) / STAGE_BYTES;
   static_assert(STAGES >= 2, "need a double-buffered pipeline");
-  static constexpr int TMEM_COLS = 2 * BN;      // two float32 accumulators (ping-pong between chunks)
+  static constexpr int TMEM_COLS = 2 * BN;      // two float32 accumulators (ping-pong between k-tiles)
   static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024 /*align*/ + 256 /*barriers*/;
   // instruction descriptor: D = f32, A = B = bf16, both K-major, N >> 3, M >> 4
   static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
                                     ((uint32_t)(BM >> 4) << 24);
 };
 
-// 128-byte swizzled K-major operand tile: 8-row x 128-byte atoms stacked every 1024 bytes.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr) { return smem_desc_sw(addr, 1024, kLayoutSw128); }
-
 struct TcMaps {
   CUtensorMap a[3], b[3];  // bf16 planes of A and B, most significant first
 };
 
-constexpr int KC = 1;  // k-tiles accumulated in TMEM before promotion to registers
 constexpr int GROUP = 16;  // row tiles per rasterisation group
 
 // Epilogue threads: warps 2..9.  Warp w reads TMEM lanes 32*(w%4)..+31 (its
@@ -87,7 +89,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   const int grp = blockIdx.x / per_group, first_m = grp * GROUP;
   const int gsize = min(tiles_m - first_m, GROUP);
   const int local = blockIdx.x - grp * per_group;
-  const int tm = first_m + local % gsize, tn = local / gsize;
+  int tm = first_m + local % gsize, tn = local / gsize;
+  // triangular operands whose k-range grows with the row or column: the long tiles first, so that the last wave
+  // is of short ones
+  if (p.tri_a > 0) tm = tiles_m - 1 - tm;
+  if (p.tri_b > 0) tn = tiles_n - 1 - tn;
   const int m0 = tm * BM, n0 = tn * BN;
   if (p.sym && m0 + BM - 1 < n0) return;  // tile entirely above the diagonal
 
@@ -137,7 +143,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   if (p.tri_b > 0) kt1 = min(kt1, (n0 + BN + BK - 1) / BK);
   if (p.tri_b < 0) kt0 = max(kt0, n0 / BK);
   const int nk = kt1 > kt0 ? kt1 - kt0 : 0;
-  const int nchunks = (nk + KC - 1) / KC;
+  const int nit = nk * C::SUB;  // stages; each k-tile is accumulated in TMEM, then promoted to registers
   bool mma_issued = false;
 
   if (skip) {
@@ -145,8 +151,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   } else if (warp == 0 && lane == 0) {
     // ---------------- TMA producer
     int last_round[8] = {-1, -1, -1, -1, -1, -1, -1, -1};
-    for (int it = 0; it < nk; ++it) {
-      const int kt = kt0 + it;
+    for (int it = 0; it < nit; ++it) {
       const int s = it % C::STAGES;
       const uint32_t ph = (uint32_t)(it / C::STAGES) & 1u;
       if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, wait_ns)) {
@@ -156,7 +161,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       }
       const uint32_t st = base + s * C::STAGE_BYTES;
       mbar_expect_tx(full_bar(s), C::STAGE_BYTES);
-      const int x = kt * BK;
+      const int x = kt0 * BK + it * C::SK;
 #pragma unroll
       for (int i = 0; i < S; ++i) tma_load_2d(st + i * C::A_BYTES, &maps.a[i], x, m0, full_bar(s));
 #pragma unroll
@@ -168,10 +173,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         if (last_round[s] >= 0) mbar_wait(full_bar(s), (uint32_t)last_round[s] & 1u, &never);
     }
   } else if (warp == 1 && lane == 0) {
-    // ---------------- MMA issuer: chunk c accumulates into TMEM buffer c & 1
-    for (int it = 0; it < nk; ++it) {
-      const int c = it / KC, buf = c & 1;
-      if (it % KC == 0 && !mbar_wait(acce_bar(buf), ((uint32_t)(c >> 1) & 1u) ^ 1u, abort_flag, wait_ns)) {
+    // ---------------- MMA issuer: k-tile c accumulates into TMEM buffer c & 1
+    for (int it = 0; it < nit; ++it) {
+      const int c = it / C::SUB, buf = c & 1;
+      if (it % C::SUB == 0 && !mbar_wait(acce_bar(buf), ((uint32_t)(c >> 1) & 1u) ^ 1u, abort_flag, wait_ns)) {
         *abort_flag = 1;
         status_set(p.status, KF_ERR_TIMEOUT, p.step, 4);
         break;
@@ -186,9 +191,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t st = base + s * C::STAGE_BYTES;
       const uint32_t dacc = tmem + (uint32_t)(buf * BN);
-      const bool first_of_chunk = (it % KC) == 0;
+      const bool first_of_tile = it % C::SUB == 0;
 #pragma unroll
-      for (int k = 0; k < BK / UMMA_K; ++k) {
+      for (int k = 0; k < C::SK / UMMA_K; ++k) {
         const uint32_t off = k * UMMA_K * 2;  // bytes along K inside the swizzle atom
         // products of slice levels i + j < S, least significant first
 #pragma unroll
@@ -196,25 +201,25 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 #pragma unroll
           for (int i = 0; i <= lvl; ++i) {
             const int j = lvl - i;
-            const uint32_t acc = (!first_of_chunk || k > 0 || lvl != S - 1 || i != 0) ? 1u : 0u;
-            mma_bf16(dacc, smem_desc(st + i * C::A_BYTES + off), smem_desc(st + S * C::A_BYTES + j * C::B_BYTES + off),
-                     C::IDESC, acc);
+            const uint32_t acc = (!first_of_tile || k > 0 || lvl != S - 1 || i != 0) ? 1u : 0u;
+            mma_bf16(dacc, smem_desc_sw(st + i * C::A_BYTES + off, C::SBO, C::LAYOUT),
+                     smem_desc_sw(st + S * C::A_BYTES + j * C::B_BYTES + off, C::SBO, C::LAYOUT), C::IDESC, acc);
           }
         }
       }
       mma_issued = true;
       mma_commit(empty_bar(s));
-      if (it % KC == KC - 1 || it == nk - 1) mma_commit(accf_bar(buf));
+      if (it % C::SUB == C::SUB - 1) mma_commit(accf_bar(buf));
     }
   } else if (warp >= 2) {
-    // ---------------- epilogue: promote each chunk into float32 registers, then store
+    // ---------------- epilogue: promote each k-tile into float32 registers, then store
     const int q = warp % 4, h = (warp - 2) / 4;
     const int gi = m0 + 32 * q + lane;
     float acc[HALF];
 #pragma unroll
     for (int j = 0; j < HALF; ++j) acc[j] = 0.0f;
     bool ok = true;
-    for (int c = 0; c < nchunks && ok; ++c) {
+    for (int c = 0; c < nk && ok; ++c) {
       const int buf = c & 1;
       if (!mbar_wait(accf_bar(buf), (uint32_t)(c >> 1) & 1u, abort_flag, wait_ns)) {
         if (!*abort_flag) {
@@ -237,7 +242,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(acce_bar(buf)) : "memory");
     }
     // Stage the tile in shared memory (the operand stages are idle once the
-    // last chunk has been promoted), one column half at a time, then sweep it
+    // last k-tile has been promoted), one column half at a time, then sweep it
     // by rows for the direct outputs and by columns for the mirrored ones, so
     // that every global access of a warp covers consecutive addresses.
     constexpr int PITCH = HALF + 1;  // odd pitch: row and column sweeps are both conflict-free
@@ -333,28 +338,13 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// rows x cols bf16 plane with leading dimension ld (elements), box = 64 x box_rows.
-kf_status make_map(CUtensorMap* map, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
-  EncodeTiledFn enc = encode_fn();
-  if (!enc) return KF_ERR_UNSUPPORTED;
-  if ((reinterpret_cast<uintptr_t>(ptr) & 15) || ((ld * 2) & 15) || cols % BK) return KF_ERR_ARG;
-  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-  cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)box_rows};
-  cuuint32_t estr[2] = {1, 1};
-  CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? KF_OK : KF_ERR_CUDA;
-}
-
 template <int BN, int S, typename TE>
 kf_status launch(cudaStream_t s, const GemmParams<TE>& g, const TcScratch& sc, int64_t ldk, bool b_is_a) {
   using C = TcCfg<BN, S>;
   TcMaps maps;
   for (int i = 0; i < S; ++i) {
-    KF_TRY(make_map(&maps.a[i], sc.a[i], g.M, ldk, ldk, BM));
-    KF_TRY(make_map(&maps.b[i], b_is_a ? sc.a[i] : sc.b[i], g.N, ldk, ldk, BN));
+    KF_TRY(tma_map_bf16(&maps.a[i], sc.a[i], g.M, ldk, ldk, C::SK, BM, 2 * C::SK));
+    KF_TRY(tma_map_bf16(&maps.b[i], b_is_a ? sc.a[i] : sc.b[i], g.N, ldk, ldk, C::SK, BN, 2 * C::SK));
   }
   KF_CUDA_TRY(smem_limit_per_device((const void*)tc_gemm_kernel<BN, S, TE>, (int)C::SMEM));
   const dim3 grid((unsigned)(ceil_div(g.N, BN) * ceil_div(g.M, BM)));
@@ -365,6 +355,13 @@ kf_status launch(cudaStream_t s, const GemmParams<TE>& g, const TcScratch& sc, i
   note_launch();
   return launch_check("tc_gemm");
 }
+
+// Three slices: tiles of 128 x 256 from this many tiles on (about one and a half per SM), 128 x 128 below.  A
+// tile's operands pass shared memory once to be stored and once per product, and that, not the tensor cores, sets
+// the pace: 2300 cycles per k-tile against 1540 of MMAs at 128 x 128, 3460 against 3070 at 128 x 256.  Both give the
+// same bits.  Full triangular products of N = 5124 (861 wide tiles): 692 us at 128, 643 at 256 wide; halves of
+// 2562 rows (220) 141 and 149 us; N = 2048 (64) 65 and 85 us.
+constexpr int64_t kWideTiles = 240;
 
 template <typename TE>
 kf_status run_split(cudaStream_t s, TcScratch& sc, const TcOperand& A, const TcOperand& B, const GemmParams<TE>& g,
@@ -391,6 +388,8 @@ kf_status run_split(cudaStream_t s, TcScratch& sc, const TcOperand& A, const TcO
   if (b_is_a) ob.rows = 0;
   KF_TRY(split_bf16_pair(s, oa, ob, slices, ldk));
   if (slices == 2) return launch<256, 2, TE>(s, g, sc, ldk, b_is_a);
+  const int64_t wide = ceil_div(g.M, BM) * ceil_div(g.N, 256);
+  if ((g.sym ? wide / 2 : wide) >= kWideTiles) return launch<256, 3, TE>(s, g, sc, ldk, b_is_a);
   return launch<128, 3, TE>(s, g, sc, ldk, b_is_a);
 }
 

@@ -216,6 +216,26 @@ def _split3_ref(X):
     return out
 
 
+@pytest.mark.parametrize("M,N,K,sym", [(3841, 2100, 130, 0), (5000, 5000, 65, 1), (7681, 1025, 1, 0)])
+def test_tc_bf16x6_wide_tiles(M, N, K, sym):
+    """Products with many tiles take 128 x 256 tiles with half k-tiles per stage: the same bits as the narrow tiles,
+    which a product of few rows takes (a whole block of rows, or of a mirrored product's lower triangle)."""
+    rng = np.random.default_rng(M)
+    dA = torch.from_numpy(rng.standard_normal((M, K)).astype(np.float32)).cuda()
+    dB = torch.from_numpy(rng.standard_normal((N, K)).astype(np.float32)).cuda()
+    C0 = torch.from_numpy(rng.standard_normal((M, N)).astype(np.float32)).cuda()
+    dC = C0.clone()
+    B.kfx_gemm(3, 1, sym, M, N, K, -1.5, dA, K, dB, K, 0.5, dC, N)
+    assert not sym or torch.equal(dC, dC.T)
+    for r0 in range(0, M, 1024):
+        r = min(1024, M - r0)
+        n = r0 + r if sym else N
+        part = C0[r0:r0 + r, :n].clone()
+        B.kfx_gemm(3, 1, 0, r, n, K, -1.5, dA[r0:], K, dB, K, 0.5, part, n)
+        got = dC[r0:r0 + r, :n]
+        assert torch.equal(got.tril(r0), part.tril(r0)) if sym else torch.equal(got, part)
+
+
 @pytest.mark.parametrize("transB", [1, 0])
 @pytest.mark.parametrize("M,N,K", [(128, 128, 64), (300, 257, 130), (70, 513, 384)])
 def test_tc_bf16x6_gemm(transB, M, N, K):
