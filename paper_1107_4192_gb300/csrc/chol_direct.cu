@@ -1,14 +1,17 @@
 // Cholesky factor and triangular inverse of a float32 matrix of up to kCholDirectMaxN rows in one launch: the
 // leaves of the smoother-gain factorisation P_{t+1|t} = L L^T, W = L^{-1} (eqn 11).
 //
-// What bounds it: the chain of n pivots (about 200 cycles each) and, per 32-wide tile column, two trips through
-// L2 (the inverse of the diagonal tile to the panel below it, the panel to the next diagonal tile).  As a
+// What bounds it: the chain of n pivots (6.1 us per tile column: about 200 cycles per pivot, and the trip of the
+// diagonal tile's inverse through L2 to the tile below it), and from about 1200 rows on the tiles' loads.  As a
 // recursion of launches a matrix of 1024 rows took eight 128-wide leaves on one SM each (30 us) and about 40
-// small products (5 to 23 us), about 0.5 ms together; this launch takes 0.24 ms (1501 rows: 0.43 ms).
+// small products (5 to 23 us), about 0.5 ms together; this launch takes 0.21 ms (n = 128: 25 us, 512: 97 us, 1281:
+// 0.29 ms, 1501: 0.38 ms).  With the diagonal tiles on CTAs of their own, a trip through L2 more per column, and a
+// look at two flags before each tile it was 0.24 ms, and 0.43 ms for 1501 rows.  Subtracting a column's products one
+// column later, behind the next pivot, gave nothing (0.21 and 0.39 ms).
 //
 // Layout: 32 x 32 tiles, a CTA per tile of L and of W, in dataflow order with a flag per tile.
 //   L(i, j), i > j: starts from A(i, j), subtracts L(i, k) L(j, k)^T for k < j, then multiplies by D_j^T
-//   (D_j = L_jj^{-1});  diagonal tiles factor and invert theirs after the subtractions;
+//   (D_j = L_jj^{-1});  the CTA of L(j + 1, j) goes on with diagonal tile j + 1, which it factors and inverts;
 //   W(i, j), i > j: sums L(i, k) W(k, j) for j <= k < i and multiplies by -D_i;  W(j, j) = D_j.
 // Tickets go by tile column j of L, then row j of W, so that every CTA waits only for lower tickets and the
 // launch progresses however many CTAs are resident.  Waits are bounded; they end when the status word reports a
@@ -122,21 +125,57 @@ __device__ __forceinline__ void cd_add(const float (&part)[4], float (&total)[4]
   }
 }
 
+// Tiles k, k + 1, .. of two rows of flags: waits for both flags of tile k and returns how many tiles up to k1 are ready
+// in a row (at most 32; 0 when the wait expired or another tile failed).  One look at the flags for a run of tiles: a
+// CTA that starts behind the others passes the finished columns at the pace of its loads.
+__device__ __forceinline__ int cd_ready(const int* f, const int* g, int k, int k1, int* count, const CdArgs& a) {
+  if (threadIdx.x < 32) {
+    const int kk = k + (int)threadIdx.x;
+    const uint64_t t0 = globaltimer();
+    int run = 0;
+    for (int n = 1; run == 0; ++n) {
+      int ready = 0;
+      if (kk < k1) {
+        const int x = cd_acquire(f + kk), y = cd_acquire(g + kk);
+        ready = x != 0 && y != 0;
+      }
+      run = __ffs(~__ballot_sync(0xffffffffu, ready)) - 1;
+      if (run < 0) run = 32;
+      if (run == 0 && (n & 15) == 0) {
+        int stop = 0;
+        if (threadIdx.x == 0) {
+          stop = status_failed(a.status);
+          if (!stop && globaltimer() - t0 > WAIT_NS) {
+            status_set(a.status, KF_ERR_TIMEOUT, a.step, 23);
+            stop = 1;
+          }
+        }
+        if (__shfl_sync(0xffffffffu, stop, 0)) break;
+      }
+    }
+    if (threadIdx.x == 0) *count = run;
+  }
+  __syncthreads();
+  return *count;
+}
+
 struct CdSmem {
-  float A[32][kPad], B[32][kPad];
-  float col[2][kPad];  // a finished column of the diagonal tile, and its 1 / pivot in [32]
-  int fail;
+  float A[2][32][kPad], B[2][32][kPad], C[2][32][kPad];
+  float col[32][kPad];  // the finished columns of the diagonal tile, each with its 1 / pivot in [32]
+  int fail, run;
 };
 
-// Diagonal tile in s.A (by rows): warp 0 factors it (lane = row, the row in registers), warp 1 forms the inverse one
-// column behind (lane = column of the inverse); on return s.A holds L and s.B the inverse, both by rows.
-__device__ void cd_factor(CdSmem& s, const CdArgs& a, int tile) {
+// Diagonal tile in s.A[0] (by rows): warp 0 factors it (lane = row, the row in registers), warp 1 forms the inverse four
+// columns behind (lane = column of the inverse); on return s.A[0] holds L and s.B[0] the inverse, both by rows.  Warp 0
+// announces every fourth column at a barrier of its own and waits for nothing.  Not inlined: with the caller's
+// registers live the columns spill.
+__device__ __noinline__ void cd_factor(CdSmem& s, const CdArgs& a, int tile) {
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int m = min(32, a.n - 32 * tile);
   if (warp == 0) {
     float r[32];
 #pragma unroll
-    for (int k = 0; k < 32; ++k) r[k] = lane < m && k < m ? s.A[lane][k] : (lane == k ? 1.0f : 0.0f);
+    for (int k = 0; k < 32; ++k) r[k] = lane < m && k < m ? s.A[0][lane][k] : (lane == k ? 1.0f : 0.0f);
     int bad = -1;
     float d = __shfl_sync(0xffffffffu, r[0], 0);
 #pragma unroll
@@ -147,10 +186,11 @@ __device__ void cd_factor(CdSmem& s, const CdArgs& a, int tile) {
       const float l = lane > j ? r[j] * q : (lane == j ? d * q : 0.0f);
       // the next pivot ahead of this column's round trip through shared memory
       if (j < 31) d = __shfl_sync(0xffffffffu, fmaf(-l, l, r[j + 1]), j + 1);
-      float* col = s.col[j & 1];
+      float* col = s.col[j];
       col[lane] = l;
       if (lane == 0) col[32] = q;
-      asm volatile("bar.sync 1, 64;" ::: "memory");
+      __syncwarp();
+      if (j % 4 == 3) asm volatile("bar.arrive %0, 64;" ::"r"(1 + j / 4) : "memory");
       r[j] = l;
 #pragma unroll
       for (int g = (j + 1) / 4; g < 8; ++g) {
@@ -166,15 +206,15 @@ __device__ void cd_factor(CdSmem& s, const CdArgs& a, int tile) {
       if (bad >= 0) status_set(a.status, KF_ERR_NOT_PD, a.step, a.base + 32 * tile + bad);
     }
 #pragma unroll
-    for (int k = 0; k < 32; ++k) s.A[lane][k] = k <= lane ? r[k] : 0.0f;
+    for (int k = 0; k < 32; ++k) s.A[0][lane][k] = k <= lane ? r[k] : 0.0f;
   } else if (warp == 1) {
     float x[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) x[i] = i == lane ? 1.0f : 0.0f;
 #pragma unroll
     for (int j = 0; j < 32; ++j) {
-      asm volatile("bar.sync 1, 64;" ::: "memory");
-      const float* col = s.col[j & 1];
+      if (j % 4 == 0) asm volatile("bar.sync %0, 64;" ::"r"(1 + j / 4) : "memory");
+      const float* col = s.col[j];
       const float xj = x[j] * col[32];
       x[j] = xj;
 #pragma unroll
@@ -187,12 +227,13 @@ __device__ void cd_factor(CdSmem& s, const CdArgs& a, int tile) {
       }
     }
 #pragma unroll
-    for (int i = 0; i < 32; ++i) s.B[i][lane] = i >= lane ? x[i] : 0.0f;
+    for (int i = 0; i < 32; ++i) s.B[0][i][lane] = i >= lane ? x[i] : 0.0f;
   }
   __syncthreads();
 }
 
-__global__ void __launch_bounds__(kCdThreads) chol_direct_kernel(const CdArgs a) {
+// Two CTAs per SM: with three the columns of a diagonal tile spill (1024 rows 0.23 ms).
+__global__ void __launch_bounds__(kCdThreads, 2) chol_direct_kernel(const CdArgs a) {
   __shared__ __align__(16) CdSmem s;
   __shared__ int ticket_s;
   if (threadIdx.x == 0) {
@@ -214,72 +255,113 @@ __global__ void __launch_bounds__(kCdThreads) chol_direct_kernel(const CdArgs a)
     dst[c + 3][r] = v.w;
   };
   float total[4] = {0.f, 0.f, 0.f, 0.f}, low[4] = {0.f, 0.f, 0.f, 0.f};
+  auto minus = [](const float4& v, const float (&t)[4], const float (&l)[4]) {
+    return make_float4((v.x - t[0]) - l[0], (v.y - t[1]) - l[1], (v.z - t[2]) - l[2], (v.w - t[3]) - l[3]);
+  };
   if (u < T - j) {
-    // ---- L(i, j)
+    // ---- L(i, j); the CTA of L(j + 1, j) goes on with diagonal tile j + 1
     const int i = j + u;
-    const float4 a0 = cd_load(a.L, a.ldl, n, i, j, r, c);
-    for (int k = 0; k < j; ++k) {
-      if (!cd_wait(fl + i * T + k, a)) return;
-      const float4 x = cd_load(a.L, a.ldl, n, i, k, r, c);
-      float4 y = x;
-      if (i != j) {
-        if (!cd_wait(fl + j * T + k, a)) return;
-        y = cd_load(a.L, a.ldl, n, j, k, r, c);
+    if (u == 0 && j > 0) return;  // factored by the CTA of L(j, j - 1)
+    const bool next = u == 1;
+    if (u == 0) {
+      put(s.A[0], cd_load(a.L, a.ldl, n, 0, 0, r, c));
+      __syncthreads();
+    } else {
+      const float4 a0 = cd_load(a.L, a.ldl, n, i, j, r, c);
+      const float4 d0 = next ? cd_load(a.L, a.ldl, n, i, i, r, c) : a0;
+      float dtotal[4] = {0.f, 0.f, 0.f, 0.f}, dlow[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int k = 0; k < j;) {
+        const int end = k + cd_ready(fl + i * T, fl + j * T, k, j, &s.run, a);
+        if (end == k) return;
+        float4 x = cd_load(a.L, a.ldl, n, i, k, r, c), y = cd_load(a.L, a.ldl, n, j, k, r, c);
+#pragma unroll 1
+        for (; k < end; ++k) {
+          const int b = k & 1;
+          put(s.A[b], x);
+          put_t(s.B[b], y);
+          if (next) put_t(s.C[b], x);
+          __syncthreads();
+          if (k + 1 < end) {
+            x = cd_load(a.L, a.ldl, n, i, k + 1, r, c);
+            y = cd_load(a.L, a.ldl, n, j, k + 1, r, c);
+          }
+          float part[4] = {0.f, 0.f, 0.f, 0.f};
+          cd_mul(s.A[b], s.B[b], r, c, part);
+          cd_add(part, total, low);
+          if (next) {
+            float dpart[4] = {0.f, 0.f, 0.f, 0.f};
+            cd_mul(s.A[b], s.C[b], r, c, dpart);
+            cd_add(dpart, dtotal, dlow);
+          }
+        }
       }
-      put(s.A, x);
-      put_t(s.B, y);
+      __syncthreads();
+      put(s.A[0], minus(a0, total, low));
+      if (!cd_wait(fl + j * T + j, a)) return;
+      put_t(s.B[0], cd_load(a.W, a.ldw, n, j, j, r, c));  // (D_j)^T
+      __syncthreads();
+      float acc[4] = {0.f, 0.f, 0.f, 0.f};
+      cd_mul(s.A[0], s.B[0], r, c, acc);
+      cd_store(a.L, a.ldl, n, i, j, r, c, acc);
+      if (!next) {
+        cd_publish(fl + i * T + j);
+        return;
+      }
+      __syncthreads();
+      const float4 l = make_float4(acc[0], acc[1], acc[2], acc[3]);
+      put(s.A[0], l);
+      put_t(s.B[0], l);
       __syncthreads();
       float part[4] = {0.f, 0.f, 0.f, 0.f};
-      cd_mul(s.A, s.B, r, c, part);
-      cd_add(part, total, low);
+      cd_mul(s.A[0], s.B[0], r, c, part);
+      cd_add(part, dtotal, dlow);
       __syncthreads();
+      put(s.A[0], minus(d0, dtotal, dlow));
+      __syncthreads();
+      // L(i, j) published by a warp that has no part in the factorisation
+      if (threadIdx.x == kCdThreads - 1)
+        asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(fl + i * T + j) : "memory");
     }
-    put(s.A, make_float4((a0.x - total[0]) - low[0], (a0.y - total[1]) - low[1], (a0.z - total[2]) - low[2],
-                         (a0.w - total[3]) - low[3]));
-    __syncthreads();
-    if (i == j) {
-      cd_factor(s, a, j);
-      if (s.fail) return;
-      float d[4];
+    cd_factor(s, a, i);
+    if (s.fail) return;
+    float d[4];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) d[e] = s.B[r][c + e];
-      cd_store(a.W, a.ldw, n, j, j, r, c, d);
-      cd_publish(fl + j * T + j);
+    for (int e = 0; e < 4; ++e) d[e] = s.B[0][r][c + e];
+    cd_store(a.W, a.ldw, n, i, i, r, c, d);
+    cd_publish(fl + i * T + i);
 #pragma unroll
-      for (int e = 0; e < 4; ++e)  // the lower triangle of L
-        if (c + e <= r && 32 * j + r < n) a.L[(int64_t)(32 * j + r) * a.ldl + 32 * j + c + e] = s.A[r][c + e];
-      return;
-    }
-    if (!cd_wait(fl + j * T + j, a)) return;
-    put_t(s.B, cd_load(a.W, a.ldw, n, j, j, r, c));  // (D_j)^T
-    __syncthreads();
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    cd_mul(s.A, s.B, r, c, acc);
-    cd_store(a.L, a.ldl, n, i, j, r, c, acc);
-    cd_publish(fl + i * T + j);
+    for (int e = 0; e < 4; ++e)  // the lower triangle of L
+      if (c + e <= r && 32 * i + r < n) a.L[(int64_t)(32 * i + r) * a.ldl + 32 * i + c + e] = s.A[0][r][c + e];
     return;
   }
   // ---- W(i, jw) with i = j
   const int i = j, jw = u - (T - j);
-  for (int k = jw; k < i; ++k) {
-    if (!cd_wait(fl + i * T + k, a)) return;                     // L(i, k)
-    const float4 x = cd_load(a.L, a.ldl, n, i, k, r, c);
-    if (!cd_wait(k == jw ? fl + k * T + k : fl + jw * T + k, a)) return;  // W(k, jw)
-    const float4 y = cd_load(a.W, a.ldw, n, k, jw, r, c);
-    put(s.A, x);
-    put(s.B, y);
-    __syncthreads();
-    float part[4] = {0.f, 0.f, 0.f, 0.f};
-    cd_mul(s.A, s.B, r, c, part);
-    cd_add(part, total, low);
-    __syncthreads();
+  for (int k = jw; k < i;) {
+    const int end = k + cd_ready(fl + i * T, fl + jw * T, k, i, &s.run, a);  // L(i, k) and W(k, jw)
+    if (end == k) return;
+    float4 x = cd_load(a.L, a.ldl, n, i, k, r, c), y = cd_load(a.W, a.ldw, n, k, jw, r, c);
+#pragma unroll 1
+    for (; k < end; ++k) {
+      const int b = k & 1;
+      put(s.A[b], x);
+      put(s.B[b], y);
+      __syncthreads();
+      if (k + 1 < end) {
+        x = cd_load(a.L, a.ldl, n, i, k + 1, r, c);
+        y = cd_load(a.W, a.ldw, n, k + 1, jw, r, c);
+      }
+      float part[4] = {0.f, 0.f, 0.f, 0.f};
+      cd_mul(s.A[b], s.B[b], r, c, part);
+      cd_add(part, total, low);
+    }
   }
+  __syncthreads();
   if (!cd_wait(fl + i * T + i, a)) return;  // D_i
-  put(s.A, cd_load(a.W, a.ldw, n, i, i, r, c));
-  put(s.B, make_float4(-(total[0] + low[0]), -(total[1] + low[1]), -(total[2] + low[2]), -(total[3] + low[3])));
+  put(s.A[0], cd_load(a.W, a.ldw, n, i, i, r, c));
+  put(s.B[0], make_float4(-(total[0] + low[0]), -(total[1] + low[1]), -(total[2] + low[2]), -(total[3] + low[3])));
   __syncthreads();
   float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  cd_mul(s.A, s.B, r, c, acc);
+  cd_mul(s.A[0], s.B[0], r, c, acc);
   cd_store(a.W, a.ldw, n, i, jw, r, c, acc);
   cd_publish(fl + jw * T + i);
 }

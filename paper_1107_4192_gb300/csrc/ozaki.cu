@@ -16,7 +16,7 @@
 //           issues, per stage, the MMAs of every slice pair: per A slice, its
 //           partner levels in runs of up to four whose buffers are adjacent,
 //           one MMA of N = 64 x run each; after the last k-slice of a level's
-//           128-wide chunk it commits the level's buffer to its "ready"
+//           chunk it commits the level's buffer to its "ready"
 //           barrier, and a level's next chunk starts (overwriting) in a buffer
 //           the epilogue has drained;
 //   warp 2  the gate: waits for each step's operands and drained buffer and releases it to warp 1;

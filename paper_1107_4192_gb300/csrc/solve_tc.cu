@@ -50,8 +50,8 @@ kf_status gemm(Ctx& c, const GemmParams<float>& g, bool transB) {
 
 // Matrices up to this size are factored and inverted by one launch (chol_direct.cu); above it the products
 // between the halves are large enough for the tensor cores.  Whole smoothing calls with the line at 1024 / 1536 /
-// 2048: N = 1501 8.97 / 8.60 / 8.62 ms, N = 2048 12.56 / 12.48 / 14.00 ms, N = 5124 (leaves of 1281) 23.4 / 22.4 /
-// 22.5 ms, N = 8196 (leaves of 1025) 136.4 / 135.8 / 137.5 ms.
+// 2048: N = 1501 8.71 / 8.38 / 8.38 ms, N = 2048 12.17 / 12.12 / 13.54 ms, N = 5124 (leaves of 1281) 22.7 / 21.6 /
+// 21.6 ms, N = 8196 (leaves of 1025) 134.8 / 134.4 / 136.2 ms.
 constexpr int kDirectMax = 1536;
 static_assert(kDirectMax <= kCholDirectMaxN, "leaf size");
 
