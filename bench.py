@@ -395,33 +395,33 @@ def main():
              9: "refine_exact_kernel"}
     roof_smoother = roof
     # With the float64-accurate solve the dominant kernel is the exact-slice residual product
-    # (I - P X_0 with 5 slice levels = 15 bf16 products, then I - P X_1 with 7 levels = 28), each
-    # launch timed alone (class 9).  Its tensor work is the bf16 products it issues; the float64
-    # product it delivers (2 N^3 per launch) is reported beside it against the float64 peak.
+    # (I - Y_0 P with Y_0 in 3 and P in 7 slices = 18 bf16 products, then E_0 - C_s P with C_s in 2
+    # and P in 5 slices = 9), each launch timed alone (class 9).  Its tensor work is the bf16
+    # products it issues; the float64 product it delivers (2 N^3 per launch) is reported beside it
+    # against the float64 peak.
     if prof[9][0] > 0 and prof[9][1] > prof[7][1]:
         n_x, ms_x = prof[9]
-        pairs_per_step, launches_per_step = 15 + 28, 2
+        pairs_per_step, launches_per_step = 18 + 9, 2
         steps_x = n_x / launches_per_step
         issued = pairs_per_step * 2 * N ** 3 * steps_x
         t_x = ms_x / 1e3
-        roof = {"bound": "tensor", "kernel": "oz_gemm_kernel<5>, oz_gemm_kernel<7> (exact-slice I - P X)",
+        roof = {"bound": "tensor", "kernel": "oz_gemm_kernel<7,3>, oz_gemm_kernel<5,2> (exact-slice I - X P)",
                 "achieved": issued / t_x / 1e12, "peak": peaks["bf16_tflops_sustained"], "unit": "TFLOP/s",
                 "peak_source": peak_src,
                 "peak_note": "bf16_tflops_sustained (measured): the products are bf16 slice products",
-                # DRAM bytes of one oz_gemm_kernel<7> launch at N = 8196 (dram__bytes_read.sum +
-                # dram__bytes_write.sum, one ncu capture of the T = 3 run: 38.14e9 read + 0.56e9
-                # written); the 5-level launch streams 5/7 of the slice planes
-                "traffic": 38.70e9 if N == 8196 else None,
-                "traffic_note": "per oz_gemm_kernel<7> launch; the operand planes are re-read from DRAM by "
-                                "every 8-row-tile group (20x the 1.9 GB of planes), at 23% of HBM bandwidth",
+                # DRAM bytes of one oz_gemm_kernel<7,3> launch at N = 8196 (dram__bytes_read.sum +
+                # dram__bytes_write.sum, one ncu capture of a refined inverse)
+                "traffic": 14.85e9 if N == 8196 else None,
+                "traffic_note": "per oz_gemm_kernel<7,3> launch (14.29e9 read, 0.56e9 written); the operand planes "
+                                "are re-read from DRAM by every 8-row-tile group, at 14% of HBM bandwidth",
                 "launches": n_x, "avg_launch_ms": ms_x / max(n_x, 1),
-                "work_per_launch": f"(15 or 28) x 2 N^3 bf16 flops, N = {N} (levels 5 and 7)",
+                "work_per_launch": f"(18 or 9) x 2 N^3 bf16 flops, N = {N}",
                 "fp64_equivalent_tflops": launches_per_step * 2 * N ** 3 * steps_x / t_x / 1e12,
                 "fp64_equivalent_note": "2 N^3 float64-accurate flops per launch, vs 1.25 TFLOP/s nominal "
                                         "float64 of this GPU",
                 "mma_shape_note": "per k-step and A slice, one 128 x (64 run) x 16 MMA per run of up to four "
-                                  "slice levels whose TMEM accumulators are adjacent (13.5 MMAs per k-step at "
-                                  "7 levels); probe: N = 64 runs at 67% of the bf16 rate, N = 256 at 100%"}
+                                  "slice levels whose TMEM accumulators are adjacent; probe: N = 64 runs at "
+                                  "67% of the bf16 rate, N = 256 at 100%"}
         roof["frac"] = roof["achieved"] / roof["peak"]
 
     line = {"metric": METRIC, "value": value, "unit": "timesteps/s", "n_gpus": world, "steps": args.steps,
