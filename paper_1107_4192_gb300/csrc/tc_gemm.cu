@@ -13,7 +13,7 @@
 // Kernel structure (one 128 x BN output tile per CTA, 10 warps):
 //   warp 0  one lane issues TMA loads (cp.async.bulk.tensor, 128-byte
 //           swizzle) of the 2 S operand tiles of a 64-wide k-slice (128 x 256
-//           with S = 3: 32-wide, 64-byte swizzle, two stages per k-tile) into
+//           tiles: 32-wide, 64-byte swizzle, two stages per k-tile) into
 //           a shared-memory stage and arms the stage's "full" mbarrier;
 //   warp 1  allocates TMEM; one lane waits for "full", issues its tcgen05.mma
 //           (3 or 6 products per k16 step) and commits them to the
@@ -49,8 +49,10 @@ constexpr int NUM_THREADS = 320;  // TMA warp, MMA warp, 8 epilogue warps
 
 template <int BN, int S>  // S = bf16 slices per operand: 2 -> 3 products, 3 -> 6 products
 struct TcCfg {
-  // k-elements per stage: half a k-tile where a whole one would leave no room for a second stage
-  static constexpr int SK = S * (BM + BN) * BK * 2 > 100 * 1024 ? BK / 2 : BK;
+  // k-elements per stage: half a k-tile for 128 x 256 tiles (three slices: a whole one leaves no room for a second
+  // stage; two: four half stages, the 8196^3 product 1645 us, two whole ones 1752 us), a whole one for 128 x 128
+  // (halves: 46.9 us per solve product, whole 44.3)
+  static constexpr int SK = BN == 256 ? BK / 2 : BK;
   static constexpr int SUB = BK / SK;           // stages per k-tile
   static constexpr uint32_t SBO = 8 * SK * 2;   // 8-row swizzle atom
   static constexpr uint32_t LAYOUT = SK == 64 ? kLayoutSw128 : kLayoutSw64;
