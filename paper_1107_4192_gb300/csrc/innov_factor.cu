@@ -21,6 +21,7 @@
 // Every element gets the operations of the blocked right-looking algorithm of chol.cu with 32-wide
 // blocks (potrf and trsm_right) in the same order: a sum over the 32 columns of a block from zero in
 // increasing order, subtracted once; so L, L^{-1} and L^{-1} nu have the same bits.
+#include "flag_ptx.cuh"
 #include "ops.cuh"
 #include "tc_ptx.cuh"
 
@@ -55,22 +56,6 @@ struct DiagTile {
 // The other tasks' shared memory: a row CTA holds kRowsPerCta rows of 32 T values; a row of L^{-1} its 32 T
 // values X (as they become final) and T ready flags.
 
-__device__ __forceinline__ int ld_acquire(const int* p) {
-  int v;
-  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void red_release(int* p, int v) {
-  asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
-// A load that stays where it is written: the loads of a block are issued together, ahead of its chain.
-__device__ __forceinline__ double2 ld2(const double2* p) {
-  double2 v;
-  asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p) : "memory");
-  return v;
-}
-
 // Rows of tile i whose panel k is done: one byte, four tiles per word.
 __device__ __forceinline__ int* rows_word(const IfArgs& a, int k, int i) {
   return a.flags + 2 + 2 * a.T + k * ((a.T + 3) / 4) + i / 4;
@@ -98,7 +83,9 @@ __device__ __forceinline__ bool wait_flag(const int* flag, int want, const IfArg
       }
     }
   }
-  return __shfl_sync(0xffffffffu, ok, 0) != 0;
+  ok = __shfl_sync(0xffffffffu, ok, 0);
+  __syncwarp();  // orders the other lanes' reads after lane 0's acquire; the exchange alone does not
+  return ok != 0;
 }
 
 __device__ __forceinline__ double half_of(double x) {  // x / 2 for a normal x, without the float64 unit
@@ -135,11 +122,6 @@ __device__ __forceinline__ void pivot_warp(double d, int lane, double& q, double
   }
   const double e2 = __fma_rn(-l, q0, 1.0);
   q = __fma_rn(e2, q0, q0);
-}
-
-__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-__device__ __forceinline__ void bar_arrive(int id, int n) {
-  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
 // Diagonal tile: warp 0 runs the pivot chain alone on its sub-partition; warps 1-3 hold the tile's
@@ -337,13 +319,15 @@ __device__ void row_task(double* row, const IfArgs& a, volatile int* failed, boo
 
 // Row r of L^{-1}, four warps: X_k for the row's tiles k = tr .. 0 with
 // X_j = (0 - X_tr L[tr, j] - .. - X_{j+1} L[j+1, j]) L_jj^{-1}; warp w owns the tiles j = w mod 4 and
-// applies the X_k that are ready while it waits for the last one.
+// applies the X_k that are ready while it waits for the last one.  Of tile j it needs the second count: the rows of
+// tile tr have waited for the first alone, which does not cover dinv.
 __device__ void inverse_row(double* B, int* ready_flags, const IfArgs& a, int r, int warp, int lane) {
   const int tr = r / 32, ldw = 32 * a.T;
   if (!wait_flag(a.flags + 2 + tr, 2, a, lane, 100)) return;
   double* out = a.Linv + (int64_t)r * a.m;
   volatile int* ready = ready_flags;
   for (int j = tr - 1 - ((tr - 1 - warp) & 3); j >= 0; j -= 4) {
+    if (!wait_flag(a.flags + 2 + j, 2, a, lane, 0)) return;
     const double* D = a.dinv + (int64_t)j * 1024 + lane;
     double b = 0.0;
     double dv[32];
@@ -363,6 +347,10 @@ __device__ void inverse_row(double* B, int* ready_flags, const IfArgs& a, int r,
         if (lane == 0 && !ready[k]) {
           const uint64_t t0 = globaltimer();
           while (!ready[k]) {
+            if (status_failed(a.status)) {  // another warp of the row may have stopped at it
+              ok = 0;
+              break;
+            }
             if (globaltimer() - t0 > kIfWaitNs) {
               status_set(a.status, KF_ERR_TIMEOUT, a.step, 22);
               ok = 0;
@@ -371,6 +359,7 @@ __device__ void inverse_row(double* B, int* ready_flags, const IfArgs& a, int r,
           }
         }
         if (!__shfl_sync(0xffffffffu, ok, 0)) return;
+        __syncwarp();
         __threadfence_block();
         X = B + 32 * k;
       }
