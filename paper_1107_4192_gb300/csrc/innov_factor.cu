@@ -239,18 +239,19 @@ __device__ void factor_tile(DiagTile& s, const IfArgs& a, int tile, int warp, in
   if (threadIdx.x == 0) red_release(a.flags + 2 + tile, 1);
 }
 
-// Wait of a row CTA's four warps: warp 0 polls for all (one poll per warp slowed the data down).
-__device__ __forceinline__ bool wait_flag_rows(const int* flag, int want, const IfArgs& a, volatile int* failed, int warp,
-                                               int lane, int sleep_ns, int shift = 0, int mask = -1) {
-  if (warp == 0 && !wait_flag(flag, want, a, lane, sleep_ns, shift, mask)) *failed = 1;
-  bar_sync(6, 32 * kRowsPerCta);
-  return *failed == 0;
+// Wait of a row CTA's four warps: warp 0 polls for all (one poll per warp slowed the data down), and the barrier
+// itself carries its result: a flag in shared memory could already be the next wait's when a late warp reads it, and
+// that warp would leave the others at their barrier for good.
+__device__ __forceinline__ bool wait_flag_rows(const int* flag, int want, const IfArgs& a, int warp, int lane, int sleep_ns,
+                                               int shift = 0, int mask = -1) {
+  const bool failed = warp == 0 && !wait_flag(flag, want, a, lane, sleep_ns, shift, mask);
+  return !bar_or(6, 32 * kRowsPerCta, failed);
 }
 
 // Four rows of one tile of S, a row per warp (or the innovation as row m, warp 0): for each panel k left
 // of the rows' diagonal tile, L[r, k] = A[r, k] L_kk^{-T}, then A[r, i] -= L[r, k] L[i, k]^T for the
 // tiles i > k of the row.
-__device__ void row_task(double* row, const IfArgs& a, volatile int* failed, bool is_nu, int r, int warp, int lane) {
+__device__ void row_task(double* row, const IfArgs& a, bool is_nu, int r, int warp, int lane) {
   const bool live = is_nu ? warp == 0 : r < a.m;
   const int tr = is_nu ? a.T : r / 32, ldw = 32 * a.T;
   const int ncols = live ? (is_nu ? a.m : min(a.m, 32 * (tr + 1))) : 0;
@@ -264,7 +265,7 @@ __device__ void row_task(double* row, const IfArgs& a, volatile int* failed, boo
   }
   __syncwarp();
   for (int k = 0; k < tr; ++k) {
-    if (!wait_flag_rows(diag_ready + k, 1, a, failed, warp, lane, 20)) return;
+    if (!wait_flag_rows(diag_ready + k, 1, a, warp, lane, 20)) return;
     const double2* D = reinterpret_cast<const double2*>(a.Dt + (int64_t)k * 1024) + lane;
     double2 dv[16];  // row `lane` of L_kk^{-1}
 #pragma unroll
@@ -287,7 +288,7 @@ __device__ void row_task(double* row, const IfArgs& a, volatile int* failed, boo
       __syncwarp();
     }
     for (int i = k + 1; i <= last; ++i) {
-      if (!wait_flag_rows(rows_word(a, k, i), min(32, a.m - 32 * i), a, failed, warp, lane, 0, 8 * (i & 3), 0xff)) return;
+      if (!wait_flag_rows(rows_word(a, k, i), min(32, a.m - 32 * i), a, warp, lane, 0, 8 * (i & 3), 0xff)) return;
       if (!live) continue;
       const int c = 32 * i + lane;
       // rows of L beyond m do not exist: those lanes read the tile's first row and drop the result
@@ -390,10 +391,9 @@ __global__ void __launch_bounds__(kIfThreads) innovation_factor_kernel(const IfA
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double* rows = reinterpret_cast<double*>(smem_raw);
   int* ready = reinterpret_cast<int*>(rows + 32 * a.T);
-  __shared__ int ticket_s, failed_s;
+  __shared__ int ticket_s;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   if (threadIdx.x == 0) ticket_s = status_failed(a.status) ? -1 - atomicAdd(a.flags, 1) : atomicAdd(a.flags, 1);
-  if (threadIdx.x == 0) failed_s = 0;
   for (int e = threadIdx.x; e < a.T; e += kIfThreads) ready[e] = 0;
   __syncthreads();
   const int ticket = ticket_s;
@@ -408,10 +408,10 @@ __global__ void __launch_bounds__(kIfThreads) innovation_factor_kernel(const IfA
       if (u == units - 1) {
         factor_tile(*reinterpret_cast<DiagTile*>(smem_raw), a, tile, warp, lane);
       } else if (warp < kRowsPerCta) {
-        row_task(rows + warp * 32 * a.T, a, &failed_s, false, 32 * tile + kRowsPerCta * u + warp, warp, lane);
+        row_task(rows + warp * 32 * a.T, a, false, 32 * tile + kRowsPerCta * u + warp, warp, lane);
       }
     } else if (a.nu && ticket == nfac) {
-      if (warp < kRowsPerCta) row_task(rows + warp * 32 * a.T, a, &failed_s, true, a.m, warp, lane);
+      if (warp < kRowsPerCta) row_task(rows + warp * 32 * a.T, a, true, a.m, warp, lane);
     } else if (warp < 4) {
       const int r = ticket - nfac - (a.nu ? 1 : 0);
       inverse_row(rows, ready, a, r, warp, lane);

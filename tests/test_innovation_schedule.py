@@ -22,7 +22,7 @@ def host_source(text):
         text = text.replace(old, new)
 
     swap("extern __shared__ __align__(16) unsigned char smem_raw[];", "unsigned char* smem_raw = emu::shared_memory();")
-    swap("__shared__ int ticket_s, failed_s;", "int &ticket_s = emu::shared_int(0), &failed_s = emu::shared_int(1);")
+    swap("__shared__ int ticket_s;", "int& ticket_s = emu::shared_int(0);")
     lines = [ln for ln in text.splitlines() if not ln.startswith("#include")]
     text = "\n".join(lines)
     cut = text.index("kf_status innovation_factor(")
@@ -55,3 +55,9 @@ def test_every_read_is_ordered_after_its_write(program, m):
     """Warps held back where they have released a flag: what they store after it must have a wait of its own (the
     inverse of a diagonal tile by rows, which the rows of L^{-1} read)."""
     run(program, m, 12, release=0.2)
+
+
+@pytest.mark.parametrize("bad", [0, 40])
+def test_a_failure_ends_every_wait(program, bad):
+    """A bad pivot while warps are held back after a barrier: every CTA ends and the first pivot is reported."""
+    run(program, 70, 16, bad=bad, barrier=0.01)
