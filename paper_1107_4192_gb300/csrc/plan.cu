@@ -169,7 +169,10 @@ Sizes sizes_for(const kf_desc* d) {
   w += cov_count(d->q_kind, N) * 8 + m * N * 8 + cov_count(d->r_kind, m) * 8;
   // split planes: rows up to max(N, m), k up to max(ldN, 2 ldm) (the Joseph product's rank 2m)
   if (d->prec == KF_PREC_MIXED_BF16X3) w += tc_scratch_bytes(std::max(N, m), std::max(ldN, 2 * ldm));
-  w += 4096;  // status word, flags of innovation_factor (T (T / 4 + 2) words, T = m / 32 and N / 32: at most 2.8 KB)
+  // status word and the flags of innovation_factor, for S and (float64) for P_{t+1|t}
+  uint64_t flags = m <= kInnovFactorMaxM ? innovation_factor_flags(m) : 0;
+  if (d->prec == KF_PREC_FP64 && N <= kInnovFactorMaxM) flags += innovation_factor_flags(N);
+  w += std::max<uint64_t>(4096, 1024 + flags * sizeof(int));
   z.workspace = w;
   return z;
 }

@@ -200,3 +200,25 @@ def test_charge_respects_the_arena_largest_free_block(built, monkeypatch):
     assert serve.plan_bytes(prob, req, budget)[1] <= int(0.7 * full)
     monkeypatch.setattr(B, "kf_arena_stats", lambda: (10 * full, 0, 1000))
     assert srv._charge(prob, req)[0] is None                      # nothing fits now: wait
+
+
+@pytest.mark.gpu
+def test_footprint_covers_the_flags_of_large_factors(built):
+    """N = m = 1536, the largest size of the one-launch factorisations, on the float64 path: the plan takes no more
+    from the arena than kf_plan_footprint says (its buffers are multiples of the arena's 256 bytes there, but for a few
+    counted with the spare bytes)."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1107_4192_gb300 import solver
+    n = 1536
+    prob = synth.random_walk_problem(n, n, 2, seed=1)
+    B.kf_arena_reserve(4 * 10 ** 9)
+    try:
+        d = solver.upload(prob)
+        with solver.Plan.for_inputs(d, n, n, 2, prec=B.KF_PREC_FP64) as plan:
+            _, used, _ = B.kf_arena_stats()
+            _, w, s, _ = B.kf_plan_footprint(plan.desc)
+            assert 0.9 * (w + s) <= used <= w + s
+    finally:
+        B.kf_arena_release()
