@@ -14,6 +14,9 @@ __device__ __forceinline__ int ld_acquire(const int* p) {
 __device__ __forceinline__ void red_release(int* p, int v) {
   asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
+__device__ __forceinline__ void or_release(int* p, int v) {
+  asm volatile("red.release.gpu.global.or.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
 
 // A load that stays where it is written: the loads of a block are issued together, ahead of its chain.
 __device__ __forceinline__ double2 ld2(const double2* p) {

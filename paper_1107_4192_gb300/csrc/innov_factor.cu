@@ -14,7 +14,8 @@
 // row's panel products and updates in global dataflow order, one CTA per diagonal tile factors and
 // inverts it, one CTA per row of L^{-1} forms it from the right, one warp does nu as an additional
 // row below S.  Work is handed out by a ticket, and every task waits only on tasks with lower
-// tickets, so the launch makes progress however many CTAs are resident.  Waits are bounded (2 s, then
+// tickets (a row, for its own tile, on the rows above it alone: the diagonal tile is lower triangular),
+// so the launch makes progress however many CTAs are resident.  Waits are bounded (2 s, then
 // KF_ERR_TIMEOUT), and end when the status word reports a failure; the last CTA to finish clears the
 // flags for the next launch.
 //
@@ -42,7 +43,7 @@ struct IfArgs {
   double* nu;     // m, or null
   double* W;      // L and the updated diagonal tiles, row stride 32 T
   double* Dt;     // the same, pairs of columns interleaved: D[c][kk] at ((kk / 2) 32 + c) 2 + kk mod 2
-  int* flags;     // ticket, done, diag ready [T], diag rows updated [T], panel rows done [T x T bytes]
+  int* flags;     // ticket, done, diag ready [T], diag rows updated [T], panel rows done [T x T]
   int* status;
   int step;
 };
@@ -56,21 +57,20 @@ struct DiagTile {
 // The other tasks' shared memory: a row CTA holds kRowsPerCta rows of 32 T values; a row of L^{-1} its 32 T
 // values X (as they become final) and T ready flags.
 
-// Rows of tile i whose panel k is done: one byte, four tiles per word.
-__device__ __forceinline__ int* rows_word(const IfArgs& a, int k, int i) {
-  return a.flags + 2 + 2 * a.T + k * ((a.T + 3) / 4) + i / 4;
-}
+// Rows of tile i whose panel k is done, a bit per row.
+__device__ __forceinline__ int* rows_word(const IfArgs& a, int k, int i) { return a.flags + 2 + 2 * a.T + k * a.T + i; }
 
-// One warp waits until the count in *flag (its byte at `shift` with mask 0xff, or the whole word) is at least
-// want; false when the wait expired or another task failed.
-__device__ __forceinline__ bool wait_flag(const int* flag, int want, const IfArgs& a, int lane, int sleep_ns,
-                                          int shift = 0, int mask = -1) {
+// One warp waits until *flag has reached want (a count), or holds all of want's bits (BITS); false when the wait
+// expired or another task failed.
+template <bool BITS = false>
+__device__ __forceinline__ bool wait_flag(const int* flag, int want, const IfArgs& a, int lane, int sleep_ns) {
+  auto reached = [&](int v) { return BITS ? (v & want) == want : v >= want; };
   int ok = 1;
   if (lane == 0) {
-    if (((ld_acquire(flag) >> shift) & mask) < want) {
+    if (!reached(ld_acquire(flag))) {
       const uint64_t t0 = globaltimer();
       for (int n = 1;; ++n) {
-        if (((ld_acquire(flag) >> shift) & mask) >= want) break;
+        if (reached(ld_acquire(flag))) break;
         if ((n & 15) == 0) {
           if (status_failed(a.status)) { ok = 0; break; }
           if (globaltimer() - t0 > kIfWaitNs) {
@@ -242,9 +242,9 @@ __device__ void factor_tile(DiagTile& s, const IfArgs& a, int tile, int warp, in
 // Wait of a row CTA's four warps: warp 0 polls for all (one poll per warp slowed the data down), and the barrier
 // itself carries its result: a flag in shared memory could already be the next wait's when a late warp reads it, and
 // that warp would leave the others at their barrier for good.
-__device__ __forceinline__ bool wait_flag_rows(const int* flag, int want, const IfArgs& a, int warp, int lane, int sleep_ns,
-                                               int shift = 0, int mask = -1) {
-  const bool failed = warp == 0 && !wait_flag(flag, want, a, lane, sleep_ns, shift, mask);
+template <bool BITS = false>
+__device__ __forceinline__ bool wait_flag_rows(const int* flag, int want, const IfArgs& a, int warp, int lane, int sleep_ns) {
+  const bool failed = warp == 0 && !wait_flag<BITS>(flag, want, a, lane, sleep_ns);
   return !bar_or(6, 32 * kRowsPerCta, failed);
 }
 
@@ -282,17 +282,21 @@ __device__ void row_task(double* row, const IfArgs& a, bool is_nu, int r, int wa
       if (!is_nu) {
         a.W[(int64_t)r * ldw + 32 * k + lane] = acc;
         __syncwarp();
-        if (lane == 0) red_release(rows_word(a, k, tr), 1 << (8 * (tr & 3)));
+        if (lane == 0) or_release(rows_word(a, k, tr), (int)(1u << (r & 31)));
         a.S[(int64_t)r * a.lds + 32 * k + lane] = acc;
       }
       __syncwarp();
     }
     for (int i = k + 1; i <= last; ++i) {
-      if (!wait_flag_rows(rows_word(a, k, i), min(32, a.m - 32 * i), a, warp, lane, 0, 8 * (i & 3), 0xff)) return;
+      // the tile's rows; of the rows' own tile those up to the CTA's last one (r - warp is its first)
+      const int rows = min(min(32, a.m - 32 * i), i == tr ? (r - warp) % 32 + kRowsPerCta : 32);
+      if (!wait_flag_rows<true>(rows_word(a, k, i), rows == 32 ? -1 : (1 << rows) - 1, a, warp, lane, 0)) return;
       if (!live) continue;
       const int c = 32 * i + lane;
-      // rows of L beyond m do not exist: those lanes read the tile's first row and drop the result
-      const double2* Lc = reinterpret_cast<const double2*>(a.W + (int64_t)(c < a.m ? c : 32 * i) * ldw + 32 * k);
+      // rows of L beyond m do not exist, and those below r do not matter to it: their lanes read the tile's first row
+      // and drop the result
+      const bool mine = c < a.m && c <= r;
+      const double2* Lc = reinterpret_cast<const double2*>(a.W + (int64_t)(mine ? c : 32 * i) * ldw + 32 * k);
       double2 lv[16];
 #pragma unroll
       for (int kk = 0; kk < 16; ++kk) lv[kk] = ld2(Lc + kk);
@@ -302,7 +306,7 @@ __device__ void row_task(double* row, const IfArgs& a, bool is_nu, int r, int wa
         s = __fma_rn(row[32 * k + 2 * kk], lv[kk].x, s);
         s = __fma_rn(row[32 * k + 2 * kk + 1], lv[kk].y, s);
       }
-      if (c < a.m) row[c] = __dsub_rn(row[c], s);
+      if (mine) row[c] = __dsub_rn(row[c], s);
     }
     __syncwarp();
   }
@@ -425,7 +429,7 @@ __global__ void __launch_bounds__(kIfThreads) innovation_factor_kernel(const IfA
   __syncthreads();
   if (ticket_s) {  // every other CTA has finished: clear the flags for the next launch
     __threadfence();
-    for (int e = threadIdx.x; e < 2 + 2 * a.T + a.T * ((a.T + 3) / 4); e += kIfThreads) a.flags[e] = 0;
+    for (int e = threadIdx.x; e < 2 + 2 * a.T + a.T * a.T; e += kIfThreads) a.flags[e] = 0;
   }
 }
 
@@ -433,7 +437,7 @@ __global__ void __launch_bounds__(kIfThreads) innovation_factor_kernel(const IfA
 
 size_t innovation_factor_flags(int64_t m) {
   const int64_t T = ceil_div(m, 32);
-  return (size_t)(2 + 2 * T + T * ((T + 3) / 4));
+  return (size_t)(2 + 2 * T + T * T);
 }
 
 kf_status innovation_factor(cudaStream_t s, int m, double* S, int64_t lds, double* dinv, double* Linv, double* nu,

@@ -286,5 +286,6 @@ inline int ld_acquire(const int* p) {
 }
 // Whoever is held back here has told the others to go on.
 inline void red_release(int* p, int v) { *p += v; emu::sched.yield(emu::sched.hold_release); }
+inline void or_release(int* p, int v) { *p |= v; emu::sched.yield(emu::sched.hold_release); }
 inline double2 ld2(const double2* p) { return *p; }
 inline uint64_t globaltimer() { emu::sched.poll(); return (uint64_t)emu::sched.steps * 10; }

@@ -61,3 +61,9 @@ def test_every_read_is_ordered_after_its_write(program, m):
 def test_a_failure_ends_every_wait(program, bad):
     """A bad pivot while warps are held back after a barrier: every CTA ends and the first pivot is reported."""
     run(program, 70, 16, bad=bad, barrier=0.01)
+
+
+@pytest.mark.parametrize("resident", [1, 3])
+def test_progress_with_few_resident_ctas(program, resident):
+    """A task waits only for tasks handed out before it: one resident CTA at a time is enough."""
+    run(program, 70, 2, resident=resident)
