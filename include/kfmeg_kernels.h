@@ -60,6 +60,15 @@ kf_status kfx_gemm_exact(int32_t levels, int64_t M, int64_t N, int64_t K, double
 kf_status kfx_spd_inverse(int32_t mode, int64_t n, const float* A, int64_t lda, double* X, int64_t ldx,
                           int64_t* fail_index, void* stream);
 
+/* S = L L^T (lower triangle, in place, m x m) for the innovation covariance of
+ * eqn 8, Linv = L^{-1} (m x m, row stride m, zeros above the diagonal) and nu <-
+ * L^{-1} nu, float64; Linv and nu may be NULL.  blocks = 0: one launch (m <= 1536,
+ * larger m returns KF_ERR_ARG), as kf_filter runs it; blocks = 1: the block kernels that kf_filter uses for
+ * larger m.  Both give the same bits.  A non-positive pivot returns KF_ERR_NOT_PD
+ * with *fail_index (else -1), a non-finite nu KF_ERR_NUMERIC.  Allocates its work space for the call. */
+kf_status kfx_innovation_factor(int32_t blocks, int64_t m, double* S, int64_t lds, double* Linv, double* nu,
+                                int64_t* fail_index, void* stream);
+
 /* Limit, in nanoseconds of the GPU's global timer, of every pipeline wait
  * (an mbarrier phase a warp of the tensor-core kernels waits for: operands
  * landed, accumulator ready, stage free) in kernels launched after this call;

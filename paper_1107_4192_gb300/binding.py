@@ -71,6 +71,7 @@ _SIGS = {
     "kfx_gemm_exact": (ctypes.c_int, [_I32, _I64, _I64, _I64, _D, _P, _I64, _I32, _P, _I64, _I32, _D, _D, _P, _I64,
                                       _P]),
     "kfx_spd_inverse": (ctypes.c_int, [_I32, _I64, _P, _I64, _P, _I64, ctypes.POINTER(_I64), _P]),
+    "kfx_innovation_factor": (ctypes.c_int, [_I32, _I64, _P, _I64, _P, _P, ctypes.POINTER(_I64), _P]),
     "kfx_tc_wait_limit": (ctypes.c_int, [ctypes.c_uint64, ctypes.POINTER(ctypes.c_uint64)]),
     "kfx_posv_right": (ctypes.c_int, [_I32, _I64, _P, _I64, _I64, _P, _I64, ctypes.POINTER(_I64), _P]),
     "kfx_posv_right_static": (ctypes.c_int, [_I32, _I64, _P, _I64, _I64, _P, _I64, ctypes.POINTER(_I64), _P]),
@@ -260,6 +261,13 @@ def kfx_spd_inverse(mode, n, A, lda, X, ldx, stream=None):
     """X = A^{-1} (float32 SPD A, float64 X); mode 1 float32-class, 2 float64-accurate."""
     fi = _I64()
     st = lib().kfx_spd_inverse(mode, n, _ptr(A), lda, _f64(X), ldx, ctypes.byref(fi), _stream(stream))
+    return st, fi.value
+
+
+def kfx_innovation_factor(blocks, m, S, lds, Linv=None, nu=None, stream=None):
+    """S = L L^T in place, Linv = L^{-1}, nu <- L^{-1} nu; blocks 0: one launch, 1: block kernels."""
+    fi = _I64()
+    st = lib().kfx_innovation_factor(blocks, m, _f64(S), lds, _f64(Linv), _f64(nu), ctypes.byref(fi), _stream(stream))
     return st, fi.value
 
 

@@ -185,6 +185,42 @@ kf_status kfx_spd_inverse(int32_t mode, int64_t n, const float* A, int64_t lda, 
   return (kf_status)h[ST_CODE];
 }
 
+kf_status kfx_innovation_factor(int32_t blocks, int64_t m, double* S, int64_t lds, double* Linv, double* nu,
+                                int64_t* fail_index, void* stream) {
+  if (fail_index) *fail_index = -1;
+  if (m < 1 || m > (blocks ? (1 << 20) : kInnovFactorMaxM) || !S || lds < m) return KF_ERR_ARG;
+  cudaStream_t s = (cudaStream_t)stream;
+  constexpr int nb = 32;
+  const int64_t mp = round_up(m, nb);
+  // flags and the status word (zero), then the work space, which needs no initial value: poisoned, so that a read
+  // before its write shows
+  const size_t head = round_up((int64_t)(innovation_factor_flags(m) + ST_WORDS) * 4, 256);
+  const size_t work = (size_t)(mp * nb + m * mp + nb * mp) * 8;
+  char* mem = nullptr;
+  KF_CUDA_TRY(cudaMalloc((void**)&mem, head + work));
+  int *status = reinterpret_cast<int*>(mem), *flags = status + ST_WORDS;
+  double* dinv = reinterpret_cast<double*>(mem + head);
+  kf_status r = KF_OK;
+  if (cudaMemsetAsync(mem, 0, head, s) != cudaSuccess || cudaMemsetAsync(dinv, 0xff, work, s) != cudaSuccess) r = KF_ERR_CUDA;
+  if (!blocks) {
+    if (r == KF_OK)
+      r = innovation_factor(s, (int)m, S, lds, dinv, Linv, nu, dinv + mp * nb, dinv + mp * nb + m * mp, flags, status, 0);
+  } else {
+    if (r == KF_OK) r = potrf<double>(s, S, lds, (int)m, dinv, nb, status, 0);
+    if (r == KF_OK && Linv) r = eye(s, m, Linv, m);
+    if (r == KF_OK && Linv) r = trsm_right<double>(s, false, (int)m, (int)m, S, lds, dinv, nb, Linv, m, status);
+    if (r == KF_OK && nu) r = trsm_right<double>(s, true, 1, (int)m, S, lds, dinv, nb, nu, m, status);
+  }
+  int h[ST_WORDS] = {0, 0, 0, 0};
+  cudaMemcpyAsync(h, status, sizeof(h), cudaMemcpyDeviceToHost, s);
+  cudaError_t e = cudaStreamSynchronize(s);
+  cudaFree(mem);
+  if (e != cudaSuccess) return KF_ERR_CUDA;
+  if (r != KF_OK) return r;
+  if (h[ST_CODE] && fail_index) *fail_index = h[ST_INDEX];
+  return (kf_status)h[ST_CODE];
+}
+
 kf_status kfx_tc_wait_limit(uint64_t ns, uint64_t* previous) {
   const uint64_t prev = g_tc_wait_ns.exchange(ns == 0 ? kTcDefaultWaitNs : ns);
   if (previous) *previous = prev;

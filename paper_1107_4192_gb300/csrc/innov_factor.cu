@@ -21,7 +21,8 @@
 //
 // Every element gets the operations of the blocked right-looking algorithm of chol.cu with 32-wide
 // blocks (potrf and trsm_right) in the same order: a sum over the 32 columns of a block from zero in
-// increasing order, subtracted once; so L, L^{-1} and L^{-1} nu have the same bits.
+// increasing order, subtracted once; so L, L^{-1} and L^{-1} nu have the same bits (compared through
+// kfx_innovation_factor).
 #include "flag_ptx.cuh"
 #include "ops.cuh"
 #include "tc_ptx.cuh"
