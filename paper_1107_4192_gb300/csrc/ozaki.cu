@@ -46,6 +46,7 @@ constexpr int OZ_GROUP = 8;     // row tiles per rasterisation group (operand re
 constexpr int OZ_ROW_PAD = 128;
 constexpr int kOzBK = 32;       // k per pipeline stage of the launched kernels (two MMA k-steps)
 constexpr int kOzBadRow = 0x7fffffff;  // exponent marking a row that holds an infinity or NaN
+constexpr int kOzScaleMax = 80;        // of a balancing exponent: float32 diagonals stay within it
 
 // LV slice levels, LA <= LV slices of A and LV of B; BK values of k per pipeline stage, one swizzled row
 // of bf16 (16: 32-byte swizzle, one MMA k-step; 32: 64-byte swizzle, two k-steps, half the stages and wider
@@ -323,6 +324,46 @@ __device__ __forceinline__ void load8(const T* row, int64_t k0, int64_t cols, bo
   }
 }
 
+// Eight consecutive values of a 16-byte aligned row from k0 on, up to cols.
+__device__ __forceinline__ void store8(float* row, int64_t k0, int64_t cols, const float (&v)[8]) {
+  if (k0 + 8 <= cols) {
+    reinterpret_cast<float4*>(row + k0)[0] = make_float4(v[0], v[1], v[2], v[3]);
+    reinterpret_cast<float4*>(row + k0)[1] = make_float4(v[4], v[5], v[6], v[7]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (k0 + i < cols) row[k0 + i] = v[i];
+  }
+}
+
+// The exponent e of x 2^w, 2^(e-1) <= |x| 2^w < 2^e; kOzZero for zero, kOzBadRow for an infinity or NaN.
+constexpr int kOzZero = -0x7fffffff;
+__device__ __forceinline__ int exponent_of(double x, int w) {
+  const unsigned long long m = mag_bits(x);
+  const int E = (int)(m >> 52);
+  if (E == 0x7ff) return kOzBadRow;
+  return E > 0 ? E - 1022 + w : m == 0 ? kOzZero : 63 - __clzll((long long)m) - 1073 + w;
+}
+__device__ __forceinline__ int exponent_of(float x, int w) {
+  const unsigned m = __float_as_uint(x) & 0x7fffffffu;
+  const int E = (int)(m >> 23);
+  if (E == 0xff) return kOzBadRow;
+  return E > 0 ? E - 126 + w : m == 0 ? kOzZero : 31 - __clz((int)m) - 148 + w;
+}
+
+// Eight weights sign scale[0..7], 16-byte aligned.
+__device__ __forceinline__ void weights8(const int* scale, int sign, int (&w)[8]) {
+  const int4 a = reinterpret_cast<const int4*>(scale)[0], b = reinterpret_cast<const int4*>(scale)[1];
+  const int v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+  for (int i = 0; i < 8; ++i) w[i] = sign * v[i];
+}
+
+// q 2^k for an integer |q| <= 2^24, rounded like ldexpf.
+__device__ __forceinline__ float scaled(int q, int k) {
+  return (unsigned)(k + 126) <= 252u ? (float)q * __int_as_float((k + 127) << 23) : ldexpf((float)q, k);
+}
+
 // Signed base-256 digits of eight integers |x| <= 2^(8S - 1), written as bf16 to S planes (16-byte stores).
 // Digit p is q_p = Q_p - 256 Q_{p-1} with Q_p = x / 2^(8(S-1-p)) rounded to nearest, ties to even: the
 // successive rounding of the remainders, since a remainder differs from x by multiples of 256 2^(8(S-1-p)).
@@ -353,8 +394,10 @@ __device__ __forceinline__ void write_digits8(const long long (&x)[8], int S, __
   }
 }
 
+// w: a power of two for each value.
 template <typename T>
-__device__ __forceinline__ void slice8(const T (&v)[8], int shift, bool bad, int S, __nv_bfloat16* dst, int64_t pstride) {
+__device__ __forceinline__ void slice8(const T (&v)[8], const int (&w)[8], int shift, bool bad, int S, __nv_bfloat16* dst,
+                                       int64_t pstride) {
   long long x[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
@@ -362,21 +405,21 @@ __device__ __forceinline__ void slice8(const T (&v)[8], int shift, bool bad, int
     int exp2;
     bool neg;
     decompose(v[i], mant, exp2, neg);
-    x[i] = bad ? 0 : fixed_rne(mant, exp2, neg, shift);
+    x[i] = bad ? 0 : fixed_rne(mant, exp2 + w[i], neg, shift);
   }
   write_digits8(x, S, dst, pstride);
 }
 
 // Maximum over the warp (kGroup 32) or the 256-thread block, to all its threads.
-template <int kGroup>
-__device__ __forceinline__ unsigned long long group_max(unsigned long long mx) {
+template <int kGroup, typename V>
+__device__ __forceinline__ V group_max(V mx) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long v = __shfl_xor_sync(0xffffffffu, mx, o);
+    const V v = __shfl_xor_sync(0xffffffffu, mx, o);
     mx = v > mx ? v : mx;
   }
   if constexpr (kGroup == 256) {
-    __shared__ unsigned long long red[8];
+    __shared__ V red[8];
     if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = mx;
     __syncthreads();
 #pragma unroll
@@ -390,37 +433,66 @@ __device__ __forceinline__ unsigned long long group_max(unsigned long long mx) {
 // 256-thread block) holds its row in registers, 8 NCH values per thread, so a row is read once: HBM-bound from
 // a few thousand columns on (5124 x 5124 float64, 5 slices: 246 us with the digits in 64-bit arithmetic and two
 // reads, 85 us now; 1664 x 128: 14.5 us and 5 us).  NCH = 0: two passes, for rows too long for that.
-template <typename T, int kGroup, int NCH>
+//
+// WEIGH: the slices of X[r][k] 2^(sign scale[k]) (below; scale is readable up to ldk).
+template <typename T, int kGroup, int NCH, bool WEIGH>
 __global__ void __launch_bounds__(256) oz_slice_kernel(const T* X, int64_t ld, int64_t rows, int64_t cols, int S,
                                                        __nv_bfloat16* planes, int64_t rows_pad, int64_t ldk,
-                                                       int* exps) {
+                                                       int* exps, const int* scale, int sign) {
   constexpr int kRows = 256 / kGroup;
   const int64_t r = (int64_t)blockIdx.x * kRows + threadIdx.x / kGroup;  // rows_pad is a multiple of kRows
   const int t = threadIdx.x % kGroup;
   const T* row = X + (r < rows ? r : 0) * ld;
   const int64_t n = r < rows ? cols : 0;  // rows beyond the matrix are zero
   const bool vec = (reinterpret_cast<uintptr_t>(X) & 15) == 0 && (ld * sizeof(T)) % 16 == 0;
-  unsigned long long mx = 0;
   T v[NCH > 0 ? NCH : 1][8];
+  int w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  bool bad;  // an infinity or NaN: zero slices, marked exponent
+  int e;     // max |X[r]| < 2^e
   if constexpr (NCH > 0) {
 #pragma unroll
     for (int c = 0; c < NCH; ++c) load8(row, (int64_t)(c * kGroup + t) * 8, n, vec, v[c]);
+  }
+  if constexpr (WEIGH) {
+    int mx = kOzZero;
+    auto take = [&](int64_t k0, const T (&x)[8]) {
+      if (k0 >= ldk) return;
+      weights8(scale + k0, sign, w);
 #pragma unroll
-    for (int c = 0; c < NCH; ++c)
+      for (int i = 0; i < 8; ++i) mx = max(mx, exponent_of(x[i], w[i]));
+    };
+    if constexpr (NCH > 0) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const unsigned long long m = mag_bits(v[c][i]);
+      for (int c = 0; c < NCH; ++c) take((int64_t)(c * kGroup + t) * 8, v[c]);
+    } else {
+      for (int64_t k0 = (int64_t)t * 8; k0 < ldk; k0 += kGroup * 8) {
+        load8(row, k0, n, vec, v[0]);
+        take(k0, v[0]);
+      }
+    }
+    mx = group_max<kGroup>(mx);
+    bad = mx == kOzBadRow;
+    e = bad || mx == kOzZero ? 0 : mx;
+  } else {
+    unsigned long long mx = 0;
+    if constexpr (NCH > 0) {
+#pragma unroll
+      for (int c = 0; c < NCH; ++c)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const unsigned long long m = mag_bits(v[c][i]);
+          mx = m > mx ? m : mx;
+        }
+    } else {
+      for (int64_t k = t; k < n; k += kGroup) {
+        const unsigned long long m = mag_bits(row[k]);
         mx = m > mx ? m : mx;
       }
-  } else {
-    for (int64_t k = t; k < n; k += kGroup) {
-      const unsigned long long m = mag_bits(row[k]);
-      mx = m > mx ? m : mx;
     }
+    mx = group_max<kGroup>(mx);
+    bad = mx >= mag_inf<T>();
+    e = bad ? 0 : mag_exponent<T>(mx);
   }
-  mx = group_max<kGroup>(mx);
-  const bool bad = mx >= mag_inf<T>();  // an infinity or NaN: zero slices, marked exponent
-  const int e = bad ? 0 : mag_exponent<T>(mx);  // max |X[r]| < 2^e
   if (t == 0) exps[r] = bad ? kOzBadRow : e;
   const int shift = 7 + 8 * (S - 1) - e;
   const int64_t pstride = rows_pad * ldk;
@@ -429,103 +501,128 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(const T* X, int64_t ld, i
 #pragma unroll
     for (int c = 0; c < NCH; ++c) {
       const int64_t k0 = (int64_t)(c * kGroup + t) * 8;
-      if (k0 < ldk) slice8(v[c], shift, bad, S, dst + k0, pstride);
+      if (k0 >= ldk) continue;
+      if constexpr (WEIGH) weights8(scale + k0, sign, w);
+      slice8(v[c], w, shift, bad, S, dst + k0, pstride);
     }
   } else {
     for (int64_t k0 = (int64_t)t * 8; k0 < ldk; k0 += kGroup * 8) {
       load8(row, k0, n, vec, v[0]);
-      slice8(v[0], shift, bad, S, dst + k0, pstride);
+      if constexpr (WEIGH) weights8(scale + k0, sign, w);
+      slice8(v[0], w, shift, bad, S, dst + k0, pstride);
     }
   }
 }
 
-// Row exponents alone (float32), as oz_slice_kernel finds them.
-__global__ void __launch_bounds__(256) oz_exps_kernel(const float* X, int64_t ld, int64_t n, int* exps) {
-  const int64_t r = blockIdx.x;
-  unsigned long long mx = 0;
-  const float* row = X + r * ld;
-  if (r < n)
-    for (int64_t k = threadIdx.x * 4; k < n; k += 1024) {  // ld is a multiple of 4 and rows are 16-byte aligned
-      const float4 f = *reinterpret_cast<const float4*>(row + k);
-      const float v[4] = {f.x, f.y, f.z, f.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const unsigned long long m = k + i < n ? mag_bits(v[i]) : 0;
-        mx = m > mx ? m : mx;
-      }
-    }
-  mx = group_max<256>(mx);
-  if (threadIdx.x == 0) exps[r] = mx >= mag_inf<float>() ? kOzBadRow : mag_exponent<float>(mx);
+// ---- slices of a refined inverse's operands, balanced
+//
+// The refinement rounds iterates to few digits below their row maxima, which is harmless only when P has rows of one
+// scale.  So it works on D P D with D_i = 2^(s_i), s_i = -round(log2(P_ii) / 2), whose diagonal lies in [1/2, 2), and
+// on D^{-1} X D^{-1}.  All of that stays in the slices: a row's own factor belongs to its exponent, and the slices of
+// row i of X hold X[i][k] 2^(-s_k), those of row j of P hold P[j][k] 2^(s_k), so the product is X P as it stands.
+
+// s_i from the diagonal (0 for one that is not positive and finite, which the factorisation reports), zero up to ldk.
+__global__ void oz_balance_kernel(const void* P, int f64, int64_t ld, int64_t n, int64_t ldk, int* scale) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ldk; i += (int64_t)gridDim.x * blockDim.x) {
+    int e = 0;
+    if (i < n)
+      e = f64 ? exponent_of(static_cast<const double*>(P)[i * ld + i], 0)
+              : exponent_of(static_cast<const float*>(P)[i * ld + i], 0);
+    scale[i] = e == kOzZero || e == kOzBadRow ? 0 : max(-kOzScaleMax, min(kOzScaleMax, -(e >> 1)));
+  }
 }
 
-// A symmetric float32 matrix rounded so that three slices hold it exactly and it stays symmetric: element
-// (i, j) to the nearest multiple of 2^(max(e_i, e_j) - 23), written back, with its three slices by rows.
-__global__ void __launch_bounds__(256) oz_slice_symmetric_kernel(float* X, int64_t ld, int64_t n, __nv_bfloat16* planes,
-                                                                 int64_t rows_pad, int64_t ldk, const int* exps) {
+// Exponents alone of the rows of a float32 X[r][k] 2^(-scale[k]).
+__global__ void __launch_bounds__(256) oz_exps_kernel(const float* X, int64_t ld, int64_t n, int64_t ldk, const int* scale,
+                                                      int* exps) {
   const int64_t r = blockIdx.x;
-  const int er = exps[r];
-  const bool live = r < n && er != kOzBadRow;
+  const int64_t cols = r < n ? n : 0;
+  const float* row = X + (r < n ? r : 0) * ld;
+  int mx = kOzZero, w[8];
+  for (int64_t k0 = threadIdx.x * 8; k0 < ldk; k0 += 256 * 8) {
+    float v[8];
+    load8(row, k0, cols, true, v);  // ld is a multiple of 4 and rows are 16-byte aligned
+    weights8(scale + k0, -1, w);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) mx = max(mx, exponent_of(v[i], w[i]));
+  }
+  mx = group_max<256>(mx);
+  if (threadIdx.x == 0) exps[r] = mx == kOzZero ? 0 : mx;
+}
+
+// A symmetric float32 matrix rounded so that three slices of its weighed rows hold it exactly and it stays symmetric:
+// with b_i = exps[i] - scale[i] the exponents of the balanced rows, element (i, j) of the balanced matrix to the
+// nearest multiple of 2^(max(b_i, b_j) - 23), written back, with its three slices by rows.
+__global__ void __launch_bounds__(256) oz_slice_symmetric_kernel(float* X, int64_t ld, int64_t n, const int* scale,
+                                                                 __nv_bfloat16* planes, int64_t rows_pad, int64_t ldk,
+                                                                 const int* exps) {
+  const int64_t r = blockIdx.x;
+  const bool live = r < n && exps[r] != kOzBadRow;
+  const int sr = r < n ? scale[r] : 0, br = live ? exps[r] - sr : 0;
   float* row = X + (r < n ? r : 0) * ld;
   for (int64_t k0 = threadIdx.x * 8; k0 < ldk; k0 += 256 * 8) {
     long long x[8];
     float v[8];
+    int sk[8], ek[8];
     load8(row, k0, live ? n : 0, true, v);
+    weights8(scale + k0, 1, sk);
+    weights8(exps + k0, 1, ek);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int ek = k0 + i < n ? exps[k0 + i] : er;
-      const int g = ek == kOzBadRow ? er : max(er, ek);
+      const int g = k0 + i >= n || ek[i] == kOzBadRow ? br : max(br, ek[i] - sk[i]);
       long long mant;
       int exp2;
       bool neg;
       decompose(v[i], mant, exp2, neg);
-      const long long q = fixed_rne(mant, exp2, neg, 23 - g);
-      x[i] = q << min(g - er, 40);  // |x| <= 2^23: the grid only gets coarser as g - er grows
-      v[i] = ldexpf((float)q, g - 23);
+      const long long q = fixed_rne(mant, exp2 - sr - sk[i], neg, 23 - g);
+      x[i] = q << min(g - br, 40);  // |x| <= 2^23: the grid only gets coarser as g - br grows
+      v[i] = scaled((int)q, g - 23 + sr + sk[i]);
     }
     write_digits8(x, 3, planes + r * ldk + k0, rows_pad * ldk);
-    if (live) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-        if (k0 + i < n) row[k0 + i] = v[i];
-    }
+    if (live) store8(row, k0, n, v);
   }
 }
 
-// Two slices Cs of the rows of a float32 correction C (rounded to nearest), and X = Y + Cs in float64 for a
-// float32 Y.
+// Two slices of the weighed rows of a float32 correction C (rounded to nearest), and X = Y + Cs in float64 for a
+// float32 Y and the correction Cs that the slices hold.
 __global__ void __launch_bounds__(256) oz_slice_correction_kernel(const float* C, const float* Y, int64_t ld, int64_t n,
-                                                                  __nv_bfloat16* planes, int64_t rows_pad, int64_t ldk,
-                                                                  int* exps, double* X, int64_t ldx) {
+                                                                  const int* scale, __nv_bfloat16* planes, int64_t rows_pad,
+                                                                  int64_t ldk, int* exps, double* X, int64_t ldx) {
   const int64_t r = blockIdx.x;
-  const float* row = C + (r < n ? r : 0) * ld;
-  unsigned long long mx = 0;
-  if (r < n)
-    for (int64_t k = threadIdx.x; k < n; k += 256) {
-      const unsigned long long m = mag_bits(row[k]);
-      mx = m > mx ? m : mx;
-    }
+  const int64_t cols = r < n ? n : 0;
+  const float *row = C + (r < n ? r : 0) * ld, *yrow = Y + (r < n ? r : 0) * ld;
+  int mx = kOzZero, w[8];
+  for (int64_t k0 = threadIdx.x * 8; k0 < ldk; k0 += 256 * 8) {
+    float v[8];
+    load8(row, k0, cols, true, v);
+    weights8(scale + k0, -1, w);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) mx = max(mx, exponent_of(v[i], w[i]));
+  }
   mx = group_max<256>(mx);
-  const bool bad = mx >= mag_inf<float>();
-  const int e = bad ? 0 : mag_exponent<float>(mx);
+  const bool bad = mx == kOzBadRow;
+  const int e = bad || mx == kOzZero ? 0 : mx;
   if (threadIdx.x == 0) exps[r] = bad ? kOzBadRow : e;
   for (int64_t k0 = threadIdx.x * 8; k0 < ldk; k0 += 256 * 8) {
     long long x[8];
     float v[8], y[8];
-    load8(row, k0, r < n ? n : 0, true, v);
-    load8(Y + (r < n ? r : 0) * ld, k0, r < n ? n : 0, true, y);
+    load8(row, k0, cols, true, v);
+    load8(yrow, k0, cols, true, y);
+    weights8(scale + k0, -1, w);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       long long mant;
       int exp2;
       bool neg;
       decompose(v[i], mant, exp2, neg);
-      x[i] = bad ? 0 : fixed_rne(mant, exp2, neg, 15 - e);
+      x[i] = bad ? 0 : fixed_rne(mant, exp2 + w[i], neg, 15 - e);
+      v[i] = scaled((int)x[i], e - 15 - w[i]);
     }
     write_digits8(x, 2, planes + r * ldk + k0, rows_pad * ldk);
     if (r < n) {
 #pragma unroll
       for (int i = 0; i < 8; ++i)
-        if (k0 + i < n) X[r * ldx + k0 + i] = (double)y[i] + (double)ldexpf((float)x[i], e - 15);
+        if (k0 + i < n) X[r * ldx + k0 + i] = (double)y[i] + (double)v[i];
     }
   }
 }
@@ -1209,11 +1306,13 @@ kf_status launch_oz(cudaStream_t s, const OzSlices& A, const OzSlices& B, int M,
 
 // One warp per row up to 512 columns (a block's threads would mostly idle), a block per row with the row in
 // registers up to 10240, two passes beyond.
-template <typename T>
-void slice_rows(cudaStream_t s, const T* X, int64_t ld, int64_t rows, int64_t cols, int S, const OzSlices& out) {
+template <typename T, bool WEIGH>
+void slice_rows(cudaStream_t s, const T* X, int64_t ld, int64_t rows, int64_t cols, int S, const OzSlices& out,
+                const int* scale = nullptr, int sign = 0) {
   const unsigned blocks = (unsigned)out.rows_pad;
-#define OZ_SLICE(G, NCH) \
-  oz_slice_kernel<T, G, NCH><<<blocks * G / 256, 256, 0, s>>>(X, ld, rows, cols, S, out.planes, out.rows_pad, out.ldk, out.exps)
+#define OZ_SLICE(G, NCH)                                                                                              \
+  oz_slice_kernel<T, G, NCH, WEIGH><<<blocks / (256 / G), 256, 0, s>>>(X, ld, rows, cols, S, out.planes, out.rows_pad, \
+                                                                       out.ldk, out.exps, scale, sign)
   if (out.ldk <= 256)
     OZ_SLICE(32, 1);
   else if (out.ldk <= 512)
@@ -1267,34 +1366,58 @@ kf_status oz_slice(cudaStream_t s, const void* X, int64_t ld, int f64, int64_t r
   out.rows = rows;
   out.filled = S;
   if (f64)
-    slice_rows<double>(s, static_cast<const double*>(X), ld, rows, cols, S, out);
+    slice_rows<double, false>(s, static_cast<const double*>(X), ld, rows, cols, S, out);
   else
-    slice_rows<float>(s, static_cast<const float*>(X), ld, rows, cols, S, out);
+    slice_rows<float, false>(s, static_cast<const float*>(X), ld, rows, cols, S, out);
   note_launch();
   return launch_check("oz_slice");
 }
 
-kf_status oz_slice_symmetric(cudaStream_t s, float* X, int64_t ld, int64_t n, OzSlices& out) {
-  if (n < 1 || out.S < 3 || n > out.rows_pad || n > out.ldk || ld < n || ld % 4 || (reinterpret_cast<uintptr_t>(X) & 15))
+kf_status oz_balance(cudaStream_t s, const void* P, int64_t ld, int f64, int64_t n, int64_t ldk, int* scale) {
+  if (n < 1 || ld < n || ldk < n || !P || !scale) return KF_ERR_ARG;
+  oz_balance_kernel<<<(unsigned)std::min<int64_t>(ceil_div(ldk, 64), 1024), 64, 0, s>>>(P, f64, ld, n, ldk, scale);
+  note_launch();
+  return launch_check("oz_balance");
+}
+
+kf_status oz_slice_weighed(cudaStream_t s, const void* X, int64_t ld, int f64, int64_t n, const int* scale, int sign, int S,
+                           OzSlices& out) {
+  if (n < 1 || S < 1 || S > out.S || n > out.rows_pad || n > out.ldk || ld < n || !X || !scale ||
+      (reinterpret_cast<uintptr_t>(scale) & 15))
+    return KF_ERR_ARG;
+  out.rows = n;
+  out.filled = S;
+  if (f64)
+    slice_rows<double, true>(s, static_cast<const double*>(X), ld, n, n, S, out, scale, sign);
+  else
+    slice_rows<float, true>(s, static_cast<const float*>(X), ld, n, n, S, out, scale, sign);
+  note_launch();
+  return launch_check("oz_slice_weighed");
+}
+
+kf_status oz_slice_symmetric(cudaStream_t s, float* X, int64_t ld, int64_t n, const int* scale, OzSlices& out) {
+  if (n < 1 || out.S < 3 || n > out.rows_pad || n > out.ldk || ld < n || ld % 4 || (reinterpret_cast<uintptr_t>(X) & 15) ||
+      !scale)
     return KF_ERR_ARG;
   out.rows = n;
   out.filled = 3;
-  oz_exps_kernel<<<(unsigned)out.rows_pad, 256, 0, s>>>(X, ld, n, out.exps);
+  oz_exps_kernel<<<(unsigned)out.rows_pad, 256, 0, s>>>(X, ld, n, out.ldk, scale, out.exps);
   note_launch();
   KF_TRY(launch_check("oz_exps"));
-  oz_slice_symmetric_kernel<<<(unsigned)out.rows_pad, 256, 0, s>>>(X, ld, n, out.planes, out.rows_pad, out.ldk, out.exps);
+  oz_slice_symmetric_kernel<<<(unsigned)out.rows_pad, 256, 0, s>>>(X, ld, n, scale, out.planes, out.rows_pad, out.ldk,
+                                                                   out.exps);
   note_launch();
   return launch_check("oz_slice_symmetric");
 }
 
-kf_status oz_slice_correction(cudaStream_t s, const float* C, const float* Y, int64_t ld, int64_t n, double* X,
-                              int64_t ldx, OzSlices& out) {
+kf_status oz_slice_correction(cudaStream_t s, const float* C, const float* Y, int64_t ld, int64_t n, const int* scale,
+                              double* X, int64_t ldx, OzSlices& out) {
   if (n < 1 || out.S < 2 || n > out.rows_pad || n > out.ldk || ld < n || ldx < n || ld % 4 ||
-      (reinterpret_cast<uintptr_t>(C) & 15) || (reinterpret_cast<uintptr_t>(Y) & 15))
+      (reinterpret_cast<uintptr_t>(C) & 15) || (reinterpret_cast<uintptr_t>(Y) & 15) || !scale)
     return KF_ERR_ARG;
   out.rows = n;
   out.filled = 2;
-  oz_slice_correction_kernel<<<(unsigned)out.rows_pad, 256, 0, s>>>(C, Y, ld, n, out.planes, out.rows_pad, out.ldk,
+  oz_slice_correction_kernel<<<(unsigned)out.rows_pad, 256, 0, s>>>(C, Y, ld, n, scale, out.planes, out.rows_pad, out.ldk,
                                                                     out.exps, X, ldx);
   note_launch();
   return launch_check("oz_slice_correction");

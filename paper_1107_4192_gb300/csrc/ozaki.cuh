@@ -46,15 +46,24 @@ void oz_slice_layout(OzSlices& out, void* mem, int64_t rows, int64_t cols, int S
 kf_status oz_slice(cudaStream_t s, const void* X, int64_t ld, int f64, int64_t rows, int64_t cols, int S,
                    OzSlices& out);
 
-// A symmetric n x n float32 X (16-byte aligned, ld a multiple of 4) rounded in place so that it stays
-// symmetric and three slices by rows hold it exactly (each element to 2^-24 of the larger of its two row
-// maxima), and those slices.
-kf_status oz_slice_symmetric(cudaStream_t s, float* X, int64_t ld, int64_t n, OzSlices& out);
+// The refined inverse's slices, balanced by s_i = -round(log2(P_ii) / 2) per row and column of P (scale[i], from
+// oz_balance, zero from n to the slices' ldk; 16-byte aligned; P float32 or float64).
+kf_status oz_balance(cudaStream_t s, const void* P, int64_t ld, int f64, int64_t n, int64_t ldk, int* scale);
 
-// Two slices Cs (2^-16 of the row maxima) of a float32 C, and X = Y + Cs in float64 (Y float32, both n x n with
-// leading dimension ld as above).
-kf_status oz_slice_correction(cudaStream_t s, const float* C, const float* Y, int64_t ld, int64_t n, double* X,
-                              int64_t ldx, OzSlices& out);
+// S slices of the rows of the n x n X[r][k] 2^(sign scale[k]).  Their products with slices weighed by the opposite sign
+// are X's own.
+kf_status oz_slice_weighed(cudaStream_t s, const void* X, int64_t ld, int f64, int64_t n, const int* scale, int sign, int S,
+                           OzSlices& out);
+
+// A symmetric n x n float32 X (16-byte aligned, ld a multiple of 4) rounded in place so that it stays symmetric and
+// three slices of its rows weighed by 2^(-scale[k]) hold it exactly (each element of the balanced matrix to 2^-24 of
+// the larger of its two row maxima), and those slices.
+kf_status oz_slice_symmetric(cudaStream_t s, float* X, int64_t ld, int64_t n, const int* scale, OzSlices& out);
+
+// Two slices of the rows of a float32 C weighed by 2^(-scale[k]) (2^-16 of the row maxima), and X = Y + Cs in float64
+// (Y float32, both n x n with leading dimension ld as above) for the Cs that they hold.
+kf_status oz_slice_correction(cudaStream_t s, const float* C, const float* Y, int64_t ld, int64_t n, const int* scale,
+                              double* X, int64_t ldx, OzSlices& out);
 
 // Epilogue of the exact-slice product, float64.  With acc = (A B^T)[i][j]:
 //   v = alpha acc + beta cin[i][j] + (i == j ? delta : 0) + Radd[i][j]

@@ -176,7 +176,10 @@ void refine_layout(RefineBufs& rb, void* mem, int64_t n, int64_t ld) {
   rb.X1 = reinterpret_cast<double*>(p + 2 * mat);
   rb.ld = ld;
   oz_slice_layout(rb.Ps, p + 3 * mat, n, n, 7);
-  oz_slice_layout(rb.Xs, p + 3 * mat + round_up((int64_t)oz_slice_bytes(n, n, 7), 256), n, n, 7);
+  // room for seven slices, of which three are used; the balancing exponents lie behind them
+  char* xs = p + 3 * mat + round_up((int64_t)oz_slice_bytes(n, n, 7), 256);
+  oz_slice_layout(rb.Xs, xs, n, n, 3);
+  rb.scale = reinterpret_cast<int*>(xs + round_up((int64_t)oz_slice_bytes(n, n, 3), 256));
 }
 
 kf_status refine_inverse_tc(cudaStream_t s, TcScratch& sc, int n, const void* P, int p_f64, int64_t ldp, const float* W,
@@ -197,8 +200,9 @@ kf_status refine_inverse_tc(cudaStream_t s, TcScratch& sc, int n, const void* P,
     g.status = status;
     KF_TRY(tc_gemm_ops(s, sc, TcOperand{W, ldw, 0, 1}, TcOperand{W, ldw, 0, 1}, g, 3));
   }
-  KF_TRY(oz_slice(s, P, ldp, p_f64, n, n, 7, rb.Ps));
-  KF_TRY(oz_slice_symmetric(s, Y, ld, n, rb.Xs));
+  KF_TRY(oz_balance(s, P, ldp, p_f64, n, rb.Ps.ldk, rb.scale));
+  KF_TRY(oz_slice_weighed(s, P, ldp, p_f64, n, rb.scale, 1, 7, rb.Ps));
+  KF_TRY(oz_slice_symmetric(s, Y, ld, n, rb.scale, rb.Xs));
   {
     OzEpilogue e;  // E_0 = I - Y_0 P (P symmetric: its rows are the product's columns)
     e.alpha = -1.0;
@@ -217,7 +221,7 @@ kf_status refine_inverse_tc(cudaStream_t s, TcScratch& sc, int n, const void* P,
     g.step = step;
     KF_TRY(tc_gemm_ops(s, sc, TcOperand{E, ld, 1, 0}, TcOperand{Y, ld, 0, 0}, g, 2));
   }
-  KF_TRY(oz_slice_correction(s, C, Y, ld, n, X1, ld, rb.Xs));
+  KF_TRY(oz_slice_correction(s, C, Y, ld, n, rb.scale, X1, ld, rb.Xs));
   {
     OzEpilogue e;  // E_1 = I - X_1 P = E_0 - C_s P
     e.alpha = -1.0;

@@ -24,12 +24,13 @@ kf_status gain_from_inverse_tc(cudaStream_t s, TcScratch& sc, int n, const float
 kf_status gain_identity_tc(cudaStream_t s, TcScratch& sc, int n, const float* W, int64_t ldw, int q_kind,
                            const double* q, float* J, int64_t ldj, int* status);
 
-// Buffers of refine_inverse_tc: three n x ld float64 matrices (the first holds the float32 Y_0 and C) and the
-// slices of P (7) and of the iterate (3, then 2; room for 7).
+// Buffers of refine_inverse_tc: three n x ld float64 matrices (the first holds the float32 Y_0 and C), the
+// slices of P (7) and of the iterate (3, then 2), and the balancing exponents.
 struct RefineBufs {
   double *X0 = nullptr, *R = nullptr, *X1 = nullptr;
   int64_t ld = 0;
   OzSlices Ps, Xs;
+  int* scale = nullptr;
 };
 uint64_t refine_bytes(int64_t n, int64_t ld);
 void refine_layout(RefineBufs& rb, void* mem, int64_t n, int64_t ld);
@@ -43,7 +44,10 @@ void refine_layout(RefineBufs& rb, void* mem, int64_t n, int64_t ld);
 // The iterates are rounded so that few slices hold them exactly, and the second residual updates the
 // first: 18 slice products (3 slices of Y_0 against 7 of P, levels below 7) and 9 (2 of C_s against 5,
 // levels below 5), where separate residuals of unrounded iterates took 15 + 28 (N = 8196: 19.6 + 27.9 ms;
-// now 15.8 + 9.4 ms).  The corrections are split-bf16 products (symmetric: lower triangle + mirror).
+// now 15.8 + 9.4 ms).  Row maxima are those of the balanced matrices D P D and D^{-1} X D^{-1} (D_i a power of
+// two near P_ii^(-1/2)): without that, small rows lose to the rounding of large ones (variances spread over
+// 1e6 and 1e10: errors of 2e-11 and 1e-6 relative to sqrt(X_ii X_jj), as accurate as without the spread now).
+// The corrections are split-bf16 products (symmetric: lower triangle + mirror).
 // The last correction is fused into its consumer:
 //  - gain_q != NULL (F = I, Q = q I or diagonal): J = I - Q X_2 into J64
 //    (float64) and Jf (float32), X_2 itself never stored;
