@@ -114,6 +114,14 @@ kf_status kfx_spmm_fpft(int32_t dtype, int64_t N, const int64_t* rowptr, const i
                         const double* val, const void* P, int64_t ldp, void* out, int64_t ldo,
                         int32_t q_kind, const double* Q, void* stream);
 
+/* One pass of the mesh products as the mixed path forms them for float32 matrices, from an F packed for
+ * the call: out = F P (right = 0), or out = P F^T + Q (right = 1; Q as above).  P and out N x N with leading
+ * dimensions in multiples of 4, P 16-byte aligned; nnz = rowptr[N] >= 1.  Each element is the float32
+ * rounding of its float64 sum but for ties to 2^-6 of a unit.  KF_ERR_ARG for rows of more than 55296. */
+kf_status kfx_spmm_packed(int32_t right, int64_t N, int64_t nnz, const int64_t* rowptr, const int64_t* col,
+                          const double* val, const float* P, int64_t ldp, float* out, int64_t ldo, int32_t q_kind,
+                          const double* Q, void* stream);
+
 /* Splits float32 A (rows x cols) into bf16 planes hi = bf16(A) and
  * lo = bf16(A - hi) (round to nearest), leading dimension ldh >= cols; the
  * pad columns are zeroed.  The operand form of the split-bf16 products. */

@@ -76,6 +76,7 @@ _SIGS = {
     "kfx_posv_right": (ctypes.c_int, [_I32, _I64, _P, _I64, _I64, _P, _I64, ctypes.POINTER(_I64), _P]),
     "kfx_posv_right_static": (ctypes.c_int, [_I32, _I64, _P, _I64, _I64, _P, _I64, ctypes.POINTER(_I64), _P]),
     "kfx_spmm_fpft": (ctypes.c_int, [_I32, _I64, _P, _P, _P, _P, _I64, _P, _I64, _I32, _P, _P]),
+    "kfx_spmm_packed": (ctypes.c_int, [_I32, _I64, _I64, _P, _P, _P, _P, _I64, _P, _I64, _I32, _P, _P]),
     "kfx_split_bf16": (ctypes.c_int, [_I64, _I64, _P, _I64, _P, _P, _I64, _P]),
 }
 
@@ -294,6 +295,12 @@ def kfx_posv_right_static(dtype, n, A, lda, M, B, ldb, stream=None):
 def kfx_spmm_fpft(dtype, N, rowptr, col, val, P, ldp, out, ldo, q_kind, Q, stream=None):
     _check(lib().kfx_spmm_fpft(dtype, N, _i64(rowptr), _i64(col), _f64(val), _ptr(P), ldp, _ptr(out), ldo,
                                q_kind, _f64(Q), _stream(stream)), "kfx_spmm_fpft")
+
+
+def kfx_spmm_packed(right, N, nnz, rowptr, col, val, P, ldp, out, ldo, q_kind=-1, Q=None, stream=None):
+    st = lib().kfx_spmm_packed(right, N, nnz, _i64(rowptr), _i64(col), _f64(val), _ptr(P), ldp, _ptr(out), ldo, q_kind,
+                               _f64(Q), _stream(stream))
+    _check(st, "kfx_spmm_packed")
 
 
 def kfx_split_bf16(rows, cols, A, lda, hi, lo, ldh, stream=None):

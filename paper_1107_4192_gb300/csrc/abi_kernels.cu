@@ -290,6 +290,24 @@ kf_status kfx_spmm_fpft(int32_t dtype, int64_t N, const int64_t* rowptr, const i
   return r;
 }
 
+kf_status kfx_spmm_packed(int32_t right, int64_t N, int64_t nnz, const int64_t* rowptr, const int64_t* col,
+                          const double* val, const float* P, int64_t ldp, float* out, int64_t ldo, int32_t q_kind,
+                          const double* Q, void* stream) {
+  if (N < 1 || nnz < 1 || !rowptr || !col || !val || !P || !out || ldp < N || ldo < N) return KF_ERR_ARG;
+  if (q_kind > 2 || (right && q_kind >= 0 && !Q)) return KF_ERR_ARG;
+  if (!spmm_packed_ok(N, ldp) || (reinterpret_cast<uintptr_t>(P) & 15)) return KF_ERR_ARG;
+  cudaStream_t s = (cudaStream_t)stream;
+  SpmmPacked F{rowptr, col, val, nullptr};
+  KF_CUDA_TRY(cudaMalloc((void**)&F.pack, (size_t)nnz * sizeof(float4)));
+  kf_status r = spmm_pack(s, nnz, col, val, F.pack);
+  if (r == KF_OK)
+    r = right ? spmm_wft_packed(s, N, F, P, ldp, out, ldo, q_kind, Q) : spmm_fp_packed(s, N, F, P, ldp, out, ldo);
+  cudaError_t e = cudaStreamSynchronize(s);
+  cudaFree(F.pack);
+  if (e != cudaSuccess) return KF_ERR_CUDA;
+  return r;
+}
+
 kf_status kfx_split_bf16(int64_t rows, int64_t cols, const float* A, int64_t lda, void* hi, void* lo, int64_t ldh,
                          void* stream) {
   if (rows < 0 || cols < 0 || ldh < cols || !A || !hi || !lo) return KF_ERR_ARG;

@@ -192,13 +192,20 @@ kf_status spmm_pft(cudaStream_t s, int64_t N, const int64_t* rowptr, const int64
                    const double* val, const T* P, int64_t ldp, T* out, int64_t ldo);
 
 // As spmm_fpft and spmm_pft for float32 matrices and an F packed once by spmm_pack (value, remainder and
-// column of each entry): sums in pairs of float32.  Needs spmm_packed_ok(N, ld) and 16-byte aligned rows.
+// column of each entry): sums in pairs of float32, or in float64 where a pair holds too little.  Needs
+// spmm_packed_ok(N, ld) and 16-byte aligned rows.
+struct SpmmPacked {
+  const int64_t *rowptr = nullptr, *col = nullptr;
+  const double* val = nullptr;
+  float4* pack = nullptr;
+};
 bool spmm_packed_ok(int64_t N, int64_t ld);
 kf_status spmm_pack(cudaStream_t s, int64_t nnz, const int64_t* col, const double* val, float4* out);
-kf_status spmm_fpft_packed(cudaStream_t s, int64_t N, const int64_t* rowptr, const float4* F, const float* P, int64_t ldp,
-                           float* W, int64_t ldw, float* out, int64_t ldo, int q_kind, const double* q);
-kf_status spmm_wft_packed(cudaStream_t s, int64_t N, const int64_t* rowptr, const float4* F, const float* W, int64_t ldw,
-                          float* out, int64_t ldo, int q_kind, const double* q);
+kf_status spmm_fp_packed(cudaStream_t s, int64_t N, const SpmmPacked& F, const float* P, int64_t ldp, float* W, int64_t ldw);
+kf_status spmm_wft_packed(cudaStream_t s, int64_t N, const SpmmPacked& F, const float* W, int64_t ldw, float* out,
+                          int64_t ldo, int q_kind, const double* q);
+kf_status spmm_fpft_packed(cudaStream_t s, int64_t N, const SpmmPacked& F, const float* P, int64_t ldp, float* W, int64_t ldw,
+                           float* out, int64_t ldo, int q_kind, const double* q);
 
 // Splits float A (rows x cols, lda) into `n` (2 or 3) bf16 planes:
 // plane k = bf16(A - plane 0 - .. - plane k-1) (round to nearest); columns

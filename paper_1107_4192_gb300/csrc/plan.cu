@@ -335,6 +335,8 @@ kf_status gemm_bulk<float>(kf_plan_s* p, bool transB, const GemmParams<float>& g
 
 // ------------------------------------------------------------ predict
 
+SpmmPacked packed_F(kf_plan_s* p) { return {p->Frp, p->Fcol, p->F, p->Fpack}; }
+
 template <typename B>
 kf_status predict_cov(kf_plan_s* p, const B* src, B* dst) {
   Prof pr(p, KF_KC_PREDICT);
@@ -343,8 +345,7 @@ kf_status predict_cov(kf_plan_s* p, const B* src, B* dst) {
     return add_cov<B, B>(p->s, dst, p->ldN, src, p->ldN, N, p->d.q_kind, p->Q);
   if constexpr (sizeof(B) == 4) {
     if (p->Fpack)
-      return spmm_fpft_packed(p->s, N, p->Frp, p->Fpack, src, p->ldN, (B*)p->tmpN, p->ldN, dst, p->ldN, p->d.q_kind,
-                              p->Q);
+      return spmm_fpft_packed(p->s, N, packed_F(p), src, p->ldN, (B*)p->tmpN, p->ldN, dst, p->ldN, p->d.q_kind, p->Q);
   }
   if (p->d.f_kind == KF_F_CSR)
     return spmm_fpft<B>(p->s, N, p->Frp, p->Fcol, p->F, src, p->ldN, (B*)p->tmpN, p->ldN, dst, p->ldN,
@@ -924,7 +925,7 @@ kf_status run_smoother(kf_plan_s* p, double* x_smooth, double* diagP_smooth, dou
       // J_t = P_{t|t} F^T P_{t+1|t}^{-1}
       const B* Bm = Pt;
       if (p->Fpack) {
-        KF_TRY(spmm_wft_packed(s, N, p->Frp, p->Fpack, (const float*)Pt, ldN, (float*)p->tmpN, ldN, -1, nullptr));
+        KF_TRY(spmm_wft_packed(s, N, packed_F(p), (const float*)Pt, ldN, (float*)p->tmpN, ldN, -1, nullptr));
         Bm = (const B*)p->tmpN;
       } else if (p->d.f_kind == KF_F_CSR) {
         KF_TRY(spmm_pft<B>(s, N, p->Frp, p->Fcol, p->F, Pt, ldN, (B*)p->tmpN, ldN));
