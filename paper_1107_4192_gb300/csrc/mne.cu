@@ -144,21 +144,34 @@ extern "C" kf_status mne_solve(const double* H, const double* C, int32_t c_kind,
   if (c_kind < 0 || c_kind > 2 || r_kind < 0 || r_kind > 2 || !(lambda > 0)) return KF_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
   constexpr int LV = 7;
-  const bool slices = tc_available() && N <= (1 << 20) && m <= (1 << 20) && N <= INT32_MAX - 128 && T <= INT32_MAX - 128;
+  bool slices = tc_available() && N <= (1 << 20) && m <= (1 << 20) && N <= INT32_MAX - 128 && T <= INT32_MAX - 128;
   const bool direct = m <= kInnovFactorMaxM;
   const int nb = direct ? 32 : potrf_block<double>();
   const int splits = gram_splits(m, N);
-  const bool gram_slices = slices && c_kind != KF_COV_DENSE;
-  const size_t gram = gram_slices ? 2 * oz_slice_bytes(m, N, LV) + (size_t)((splits > 1 ? splits : 0) * m + 2 * N) * m * 8 : 0;
-  const size_t outp = slices ? oz_slice_bytes(T, m, LV) + oz_slice_bytes(N, m, LV) + (size_t)(N + 1) * m * 8 : 0;
+  // G's product and X's use the same memory one after the other: about 44 bytes per element of H beside H C's 8
+  const size_t gram = c_kind == KF_COV_DENSE ? 0
+                                             : 2 * oz_slice_bytes(m, N, LV) + (size_t)((splits > 1 ? splits : 0) * m + 2 * N) * m * 8;
+  const size_t outp = oz_slice_bytes(T, m, LV) + oz_slice_bytes(N, m, LV) + (size_t)(N + 1) * m * 8;
   const size_t factor = direct ? (2 * (m + 32) * round_up(m, 32) + (T + m) * m) * 8 + innovation_factor_flags(m) * 4 : 0;
+  const size_t plain = ((size_t)m * N + m * m + round_up(m, nb) * nb + T * m) * 8 + factor + 32 * 256;
   Tmp tmp;
-  KF_TRY(tmp.reserve(((size_t)m * N + m * m + round_up(m, nb) * nb + T * m) * 8 + gram + outp + factor + 32 * 256));
+  if (slices && tmp.reserve(plain + std::max(gram, outp)) != KF_OK) slices = false;  // the float64 products need less
+  if (!slices) KF_TRY(tmp.reserve(plain));
+  const bool gram_slices = slices && c_kind != KF_COV_DENSE;
   double* HC = tmp.doubles(m * N);
   double* G = tmp.doubles(m * m);
   double* dinv = tmp.doubles(round_up(m, nb) * nb);
   double* W = tmp.doubles(T * m);
   int* st = (int*)tmp.take(ST_WORDS * sizeof(int));
+  double *Linv = nullptr, *V = nullptr, *work = nullptr;
+  int* flags = nullptr;
+  if (direct) {
+    Linv = tmp.doubles(m * m);
+    V = tmp.doubles(T * m);
+    work = tmp.doubles((m + 32) * round_up(m, 32));
+    flags = (int*)tmp.take(innovation_factor_flags(m) * sizeof(int));
+  }
+  const size_t shared = tmp.used;
   KF_CUDA_TRY(cudaMemsetAsync(st, 0, ST_WORDS * sizeof(int), s));
   // HC = H C  (m x N)
   if (c_kind == KF_COV_DENSE) {
@@ -208,10 +221,6 @@ extern "C" kf_status mne_solve(const double* H, const double* C, int32_t c_kind,
   }
   // W = Y G^{-1}
   if (direct) {
-    double* Linv = tmp.doubles(m * m);
-    double* V = tmp.doubles(T * m);
-    double* work = tmp.doubles((m + 32) * round_up(m, 32));
-    int* flags = (int*)tmp.take(innovation_factor_flags(m) * sizeof(int));
     KF_CUDA_TRY(cudaMemsetAsync(flags, 0, innovation_factor_flags(m) * sizeof(int), s));
     KF_TRY(innovation_factor(s, (int)m, G, m, dinv, Linv, nullptr, work, work + m * round_up(m, 32), flags, st, 0));
     GemmParams<double> g;  // (Y L^{-T}) L^{-1}
@@ -234,6 +243,7 @@ extern "C" kf_status mne_solve(const double* H, const double* C, int32_t c_kind,
   }
   // X = lambda W (H C)
   if (slices) {
+    tmp.used = shared;
     OzSlices a, b;
     oz_slice_layout(a, tmp.take(oz_slice_bytes(T, m, LV)), T, m, LV);
     oz_slice_layout(b, tmp.take(oz_slice_bytes(N, m, LV)), N, m, LV);
@@ -295,38 +305,57 @@ extern "C" kf_status mne_init(const double* H, const double* C, int32_t c_kind, 
                               double* x0_out, double* Q_out, void* stream) {
   if (!x0_out || !Q_out || T < 3 || N < 1 || N > INT32_MAX) return KF_ERR_ARG;
   cudaStream_t s = (cudaStream_t)stream;
-  // Q = Dt Dt^T / (T - 2) as an exact-slice product like those of mne_solve (N = 8196, T = 300: 17.8 ms on the
-  // float64 units, at their rate)
-  constexpr int LV = 7;
   const int64_t K = T - 1;
-  const bool slices = tc_available() && K <= (1 << 20) && N <= INT32_MAX - 128;
-  Tmp tmp;
-  KF_TRY(tmp.reserve((size_t)(T * N + N * K) * 8 + (slices ? oz_slice_bytes(N, K, LV) : 0) + 8 * 256));
-  double* X = X_out ? X_out : tmp.doubles(T * N);
-  double* Dt = tmp.doubles(N * K);
-  int* st = (int*)tmp.take(ST_WORDS * sizeof(int));
-  KF_TRY(mne_solve(H, C, c_kind, R, r_kind, Y, N, m, T, lambda, X, stream));
-  KF_CUDA_TRY(cudaMemcpyAsync(x0_out, X, (size_t)N * 8, cudaMemcpyDeviceToDevice, s));
-  const unsigned blocks = (unsigned)std::min<int64_t>(ceil_div(N * K, 256), 152 * 16);
-  centred_differences_kernel<<<blocks, 256, 0, s>>>(N, T, X, Dt);
-  note_launch();
-  KF_TRY(launch_check("centred_differences"));
-  if (slices) {
-    KF_CUDA_TRY(cudaMemsetAsync(st, 0, ST_WORDS * sizeof(int), s));
-    OzSlices a;
-    oz_slice_layout(a, tmp.take(oz_slice_bytes(N, K, LV)), N, K, LV);
-    KF_TRY(oz_slice(s, Dt, K, 1, N, K, LV, a));
-    OzEpilogue e;
-    e.alpha = 1.0 / (double)(T - 2);
-    e.out = Q_out; e.ldo = N;
-    e.sym = 1;
-    e.status = st;
-    KF_TRY(oz_gemm(s, a, a, (int)N, (int)N, (int)K, LV, e));
-    int h[ST_WORDS];
-    KF_CUDA_TRY(cudaMemcpyAsync(h, st, sizeof(h), cudaMemcpyDeviceToHost, s));
-    KF_CUDA_TRY(cudaStreamSynchronize(s));
-    return (kf_status)h[ST_CODE];
+  auto estimates = [&](double* X) -> kf_status {  // X and x0
+    KF_TRY(mne_solve(H, C, c_kind, R, r_kind, Y, N, m, T, lambda, X, stream));
+    KF_CUDA_TRY(cudaMemcpyAsync(x0_out, X, (size_t)N * 8, cudaMemcpyDeviceToDevice, s));
+    return KF_OK;
+  };
+  auto differences = [&](const double* X, double* Dt) -> kf_status {
+    const unsigned blocks = (unsigned)std::min<int64_t>(ceil_div(N * K, 256), 152 * 16);
+    centred_differences_kernel<<<blocks, 256, 0, s>>>(N, T, X, Dt);
+    note_launch();
+    return launch_check("centred_differences");
+  };
+  const size_t x_bytes = X_out ? 0 : (size_t)T * N * 8;
+  if (tc_available() && K <= (1 << 20) && N <= INT32_MAX - 128) {
+    // Q = Dt Dt^T / (T - 2) as an exact-slice product like those of mne_solve (N = 8196, T = 300: 17.8 ms on the
+    // float64 units, at their rate), all memory in one piece
+    constexpr int LV = 7;
+    Tmp tmp;
+    if (tmp.reserve(x_bytes + (size_t)N * K * 8 + oz_slice_bytes(N, K, LV) + 8 * 256) == KF_OK) {
+      double* X = X_out ? X_out : tmp.doubles(T * N);
+      double* Dt = tmp.doubles(N * K);
+      int* st = (int*)tmp.take(ST_WORDS * sizeof(int));
+      const kf_status r = estimates(X);
+      if (r == KF_OK) {
+        KF_TRY(differences(X, Dt));
+        KF_CUDA_TRY(cudaMemsetAsync(st, 0, ST_WORDS * sizeof(int), s));
+        OzSlices a;
+        oz_slice_layout(a, tmp.take(oz_slice_bytes(N, K, LV)), N, K, LV);
+        KF_TRY(oz_slice(s, Dt, K, 1, N, K, LV, a));
+        OzEpilogue e;
+        e.alpha = 1.0 / (double)(T - 2);
+        e.out = Q_out; e.ldo = N;
+        e.sym = 1;
+        e.status = st;
+        KF_TRY(oz_gemm(s, a, a, (int)N, (int)N, (int)K, LV, e));
+        int h[ST_WORDS];
+        KF_CUDA_TRY(cudaMemcpyAsync(h, st, sizeof(h), cudaMemcpyDeviceToHost, s));
+        KF_CUDA_TRY(cudaStreamSynchronize(s));
+        return (kf_status)h[ST_CODE];
+      }
+      if (r != KF_ERR_CUDA) return r;  // else no memory left for the estimates
+    }
   }
+  // float64 product, memory taken when it is needed
+  Tmp tx, td;
+  if (!X_out) KF_TRY(tx.reserve(x_bytes));
+  double* X = X_out ? X_out : (double*)tx.base;
+  KF_TRY(estimates(X));
+  KF_TRY(td.reserve((size_t)N * K * 8));
+  double* Dt = (double*)td.base;
+  KF_TRY(differences(X, Dt));
   GemmParams<double> g;  // lower triangle computed and mirrored
   g.M = (int)N; g.N = (int)N; g.K = (int)K;
   g.A = Dt; g.lda = K;
