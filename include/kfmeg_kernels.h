@@ -48,13 +48,14 @@ kf_status kfx_gemm_exact(int32_t levels, int64_t M, int64_t N, int64_t K, double
 /* X = A^{-1} for a symmetric positive definite float32 A (n x n, lower
  * triangle read), float64 X (n x n, full), on the tensor cores: the inverse
  * the smoother gain of eqn 11 needs (J_t = P_{t|t} F^T P_{t+1|t}^{-1}).
- *   mode 1: float32-class: recursive Cholesky A = L L^T, W = L^{-1} (split-bf16
- *           products, float32 diagonal blocks), X = W^T W;
+ *   mode 1: float32-class: Cholesky A = L L^T and W = L^{-1} (one launch up to 1536
+ *           rows, on halves with split-bf16 products above), X = W^T W;
  *   mode 2: float64-accurate: mode 1's X refined by two Newton steps
  *           X <- X + X (I - A X) whose residuals I - A X are exact-slice
- *           products (kfx_gemm_exact with 5, then 7 levels): the result
- *           agrees with a float64 inversion to float64 rounding times the
- *           condition number.
+ *           products of iterates rounded to few slices (3 x 7, then 2 x 5), A and X
+ *           balanced by powers of two: element (i, j) agrees with a float64
+ *           inversion to float64 rounding times the condition number of the
+ *           balanced A, relative to sqrt(X_ii X_jj).
  * A non-positive pivot returns KF_ERR_NOT_PD with *fail_index (else -1).
  * Allocates its work buffers for the call. */
 kf_status kfx_spd_inverse(int32_t mode, int64_t n, const float* A, int64_t lda, double* X, int64_t ldx,

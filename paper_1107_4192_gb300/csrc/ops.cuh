@@ -44,10 +44,10 @@ struct GemmParams {
   int check_diag = 0;
   int step = 0;
   int sym = 0;
-  // Tensor-core path only: transA = 1 means A is stored K x M (row-major) and
-  // is used transposed.  tri_a / tri_b: +1 when row r of the operand as used
-  // (A: M x K, op(B): N x K) is zero for k > r, -1 when zero for k < r, so
-  // k-tiles outside the band are skipped; 0 = dense (every kernel).
+  // transA = 1 (tensor-core path only): A is stored K x M (row-major) and is
+  // used transposed.  tri_a / tri_b (every kernel): +1 when row r of the
+  // operand as used (A: M x K, op(B): N x K) is zero for k > r, -1 when zero
+  // for k < r, so k-tiles outside the band are skipped; 0 = dense.
   int transA = 0;
   int tri_a = 0, tri_b = 0;
   // Smoother gain from an inverse (J = I - Q P^{-1}, F = I): when gain_q is

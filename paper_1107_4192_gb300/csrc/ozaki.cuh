@@ -42,7 +42,8 @@ void oz_slice_layout(OzSlices& out, void* mem, int64_t rows, int64_t cols, int S
 
 // Fills `out` (laid out by oz_slice_layout for at least these rows, cols and
 // S slices) from X (float64 when f64, else float32; rows x cols, leading
-// dimension ld, row-major).  A non-finite row gives NaN slices.
+// dimension ld, row-major).  A row that holds an infinity or NaN gets zero slices and a
+// marked exponent, from which the product's row or column becomes NaN.
 kf_status oz_slice(cudaStream_t s, const void* X, int64_t ld, int f64, int64_t rows, int64_t cols, int S,
                    OzSlices& out);
 
@@ -105,8 +106,8 @@ struct OzEpilogue {
 extern thread_local TcLaunchTimer* g_oz_timer;
 
 // C = A B^T for A (M x K) and B (N x K) given by their slices, keeping the
-// slice levels l < levels (4 to 7; both operands need at least `levels`
-// slices).  K <= 2^20.  splits > 1 divides K among that many CTAs per output
+// slice levels l < levels (4 to 7; B needs at least `levels` slices, A as
+// many or a_slices).  K <= 2^20.  splits > 1 divides K among that many CTAs per output
 // tile, whose float64 partial sums (splits x M x N doubles at `partials`) are
 // added in a fixed order by a second kernel that applies the epilogue.
 //
