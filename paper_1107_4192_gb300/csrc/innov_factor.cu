@@ -6,9 +6,9 @@
 // the number of active lanes (measured; 19 cycles per instruction and SM when all four are busy), so
 // the factorisation is a chain of m pivots (square root, reciprocal, scaled column: about 900 cycles
 // each alone, 1300 beside the tile's updates and inverse) and every product has to be spread over many
-// SMs.  Measured: m = 306 0.33 ms, m = 128 0.127 ms, m = 64 0.065 ms; as a sequence of launches of
-// block kernels (32-wide leaves of one warp, 64 x 64 product tiles on one SM each) 1.87 ms and
-// 0.32 ms at m = 306 and 64.
+// SMs.  Measured: m = 384 0.36 ms, m = 306 0.30 ms, m = 128 0.117 ms, m = 64 0.058 ms (0.9 us per
+// pivot; 900 cycles are 0.43 us); as a sequence of launches of block kernels (32-wide leaves of one
+// warp, 64 x 64 product tiles on one SM each) 1.87 ms and 0.32 ms at m = 306 and 64.
 //
 // Layout: 32-wide tiles, T = ceil(m / 32).  One warp per row of S (lane = column of the tile) does the
 // row's panel products and updates in global dataflow order, one CTA per diagonal tile factors and
@@ -97,7 +97,7 @@ __device__ __forceinline__ double half_of(double x) {  // x / 2 for a normal x, 
 // estimate of 1 / sqrt(d), one Newton step for it and for sqrt(d) (the same instruction on even and
 // odd lanes), then one correction each from an exact residual (fused multiply-add), which leaves an
 // error of about 2^-94 before the last rounding (Markstein's scheme; checked bit for bit against
-// sqrt and division by the tests).  Seven dependent float64 instructions instead of about fifteen.
+// correctly rounded square roots and reciprocals through kfx_innovation_factor).  Seven dependent float64 instructions instead of about fifteen.
 // Pivots outside 2^+-100 (or not positive) take the library functions.
 __device__ __forceinline__ void pivot_warp(double d, int lane, double& q, double& l) {
   const int ex = (__double2hiint(d) >> 20) & 0xfff;  // sign and exponent

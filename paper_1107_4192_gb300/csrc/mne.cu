@@ -76,7 +76,7 @@ __global__ void transpose_balanced_kernel(int64_t m, int64_t N, const double* sr
 // of the two row maxima (2^exw[t] and 2^exh[j]); an element far below that product (a source that only weakly
 // weighted sensors see, a sample that is large in other sensors) would lose its digits.  Elements below 2^-6 of it are
 // summed again from the same operands, so each is good to 2^-46 or float64's own rounding.  With Gaussian data these are
-// one in a hundred (N = 5124, m = 306, T = 200: 24 us, of which the reading of X about 8).
+// one in a hundred (N = 5124, m = 306, T = 200: 24 us; eight loads ahead of the sum's chain changed nothing).
 __global__ void __launch_bounds__(256) small_elements_kernel(int64_t T, int64_t N, int64_t m, const double* W,
                                                              const double* HCt, const int* exw, const int* exh, double lambda,
                                                              double* X, const int* status) {
@@ -137,7 +137,7 @@ int gram_splits(int64_t m, int64_t K) {
 // per term) on the tensor cores, G's with rows weighted so that their maxima are bounded by its diagonal, as the factor's
 // own rounding errors are, X's with its small elements summed again in float64: at N = 5124,
 // m = 306, T = 200 the m x m one took 0.74 ms and the T x N one 1.0 ms on the float64 units; 0.06 ms each now.
-// G's factor and inverse come from the one-launch factorisation (block kernels 1.3 ms, now 0.33 ms).
+// G's factor and inverse come from the one-launch factorisation (block kernels 1.3 ms, now 0.30 ms).
 extern "C" kf_status mne_solve(const double* H, const double* C, int32_t c_kind, const double* R, int32_t r_kind,
                                const double* Y, int64_t N, int64_t m, int64_t T, double lambda, double* X_out,
                                void* stream) {
